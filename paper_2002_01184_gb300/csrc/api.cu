@@ -58,6 +58,7 @@ struct hmc_ctx {
   bool use_lrgemm = false;      // tensor-core logistic regression, one-CTA tile products (dim > 128)
   hmc::LogregGemm lrg;
   int* lr_err = nullptr;
+  hmc::ChainSync chain_sync;       // multi-transition launches (elementwise targets)
   // replica exchange (Section 2.2): K replicas per chain, rows c*K + k
   int K = 1;
   int64_t outer_chains = 0;
@@ -310,6 +311,7 @@ CreatePlan plan_create(const hmc_target& t, int64_t num_chains, const hmc_config
   q.fused_logreg = fused && !q.use_lrtc && !q.use_lrgemm && hmc::logreg_fused_supported(t);
   q.fused_elementwise = fused && (t.id == HMC_T_STD_NORMAL || t.id == HMC_T_FUNNEL) &&
                         t.dim <= hmc::kFusedElementwiseMaxDim;
+  if (q.fused_elementwise) add(hmc::chain_sync_bytes(num_chains));
   q.plain_buffers = !q.fused_elementwise && !q.use_tc;
   if (q.plain_buffers) {
     add(4 * C * D);
@@ -399,22 +401,29 @@ cudaError_t enqueue_transition(hmc_ctx* ctx, const StepArgs& a) {
   if (uses_fused_logreg(ctx))
     return hmc::launch_logreg_fused_transition(ctx->target, a, ctx->stream, &ctx->timer);
   if (uses_fused_elementwise(ctx))
-    return hmc::launch_fused_elementwise(ctx->target.id, a, ctx->stream, &ctx->timer);
+    return hmc::launch_elementwise_chain(ctx->target.id, a, false, 1, a.t_full, a.sample_out, a.trace_eps,
+                                         a.trace_acc, ctx->chain_sync, ctx->stream, &ctx->timer);
   return hmc::launch_plain_transition(ctx->target, a, ctx->plain, ctx->grad_ws, ctx->stream,
                                       &ctx->timer);
 }
 
 // After a stream synchronisation: report a bounded device wait that gave up.
 hmc_status check_device_flag(hmc_ctx* ctx) {
-  if (!ctx->use_tc && !ctx->use_lrtc && !ctx->use_lrgemm) return HMC_OK;
+  // (of the chain launches only the adapting ones wait)
+  const bool chain_waits = ctx->chain_sync.err && ctx->cfg.adapt;
+  if (!ctx->use_tc && !ctx->use_lrtc && !ctx->use_lrgemm && !chain_waits) return HMC_OK;
   int flag = 0;
-  cudaError_t e = cudaMemcpyAsync(&flag, ctx->use_tc ? ctx->tc.err : ctx->use_lrtc ? ctx->lr_err : ctx->lrg.err,
+  cudaError_t e = cudaMemcpyAsync(&flag,
+                                  ctx->use_tc ? ctx->tc.err : ctx->use_lrtc ? ctx->lr_err
+                                  : ctx->use_lrgemm ? ctx->lrg.err : ctx->chain_sync.err,
                                   sizeof(int),
                                   cudaMemcpyDeviceToHost, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "read device error flag");
   if (flag == 2 && ctx->nuts_dense)
     return fail(ctx, HMC_E_TIMEOUT, "the NUTS leaf loop ran past 2^max_depth iterations and was stopped");
+  if (flag && chain_waits)
+    return fail(ctx, HMC_E_TIMEOUT, "the grid barrier of a multi-transition launch gave up");
   if (flag)
     return fail(ctx, HMC_E_TIMEOUT,
                 "a tensor-core kernel's bounded wait gave up (site " + std::to_string(flag) + ")");
@@ -511,6 +520,27 @@ hmc_status enqueue_range(hmc_ctx* ctx, float* x, int64_t B, int64_t t_begin, int
       if (e != cudaSuccess) return cuda_fail(ctx, e, "pair transition launch");
     }
     ctx->dom_transitions = chunk;
+    return HMC_OK;
+  }
+  // elementwise targets: the transitions that adapt the step size in one
+  // cooperative launch, the others in one ordinary launch
+  // (moments of transitions that still adapt: one launch per transition, below)
+  const int64_t t_fixed = ctx->cfg.adapt ? std::min(t_end, std::max(t_begin, ctx->cfg.num_adapt_steps)) : t_begin;
+  if (uses_fused_elementwise(ctx) && ctx->K == 1 && T > 0 && !(ctx->s_mean && t_fixed > B)) {
+    for (int64_t t0 = t_begin; t0 < t_end;) {
+      const int64_t stop = t0 < t_fixed ? t_fixed : t_end;
+      const int n = static_cast<int>(std::min(chunk, stop - t0));
+      StepArgs a = make_args(ctx, x, static_cast<uint64_t>(t0));
+      if (ctx->s_mean && t0 >= t_fixed)
+        a.w = hmc::WelfordOut{ctx->s_mean, ctx->s_m2, ctx->s_bsize, ctx->bm_sum, ctx->bm_mean, ctx->bm_m2};
+      cudaError_t e = hmc::launch_elementwise_chain(ctx->target.id, a, t0 < t_fixed, n, B + out0, samples, trace_eps,
+                                                    trace_acc, ctx->chain_sync, ctx->stream,
+                                                    &ctx->timer);
+      if (e != cudaSuccess) return cuda_fail(ctx, e, "chain launch");
+      t0 += n;
+    }
+    // (the last launch's)
+    ctx->dom_transitions = std::min(chunk, t_end - (t_fixed < t_end ? t_fixed : t_begin));
     return HMC_OK;
   }
   // NUTS: the transitions that do not adapt the step size run in as few
@@ -727,6 +757,16 @@ hmc_status hmc_create(const hmc_target* target, int64_t num_chains, const hmc_co
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&nd.side, cudaStreamNonBlocking);
   }
   if (e == cudaSuccess && plan.fused_logreg) e = hmc::logreg_fused_setup(*target);
+  if (e == cudaSuccess && plan.fused_elementwise) {
+    char* w = nullptr;
+    const size_t bytes = hmc::chain_sync_bytes(num_chains);
+    e = ctx_alloc(ctx, &w, bytes);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w, 0, 16, ctx->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w + 16, 0xFF, bytes - 16, ctx->stream);
+    ctx->chain_sync.left = reinterpret_cast<unsigned*>(w);
+    ctx->chain_sync.err = reinterpret_cast<int*>(w + 4);
+    ctx->chain_sync.slots = reinterpret_cast<unsigned long long*>(w + 16);
+  }
   if (e == cudaSuccess && plan.plain_buffers) {
     e = ctx_alloc(ctx, &ctx->plain.xp, C * D);
     if (e == cudaSuccess) e = ctx_alloc(ctx, &ctx->plain.gp, C * D);
@@ -1284,8 +1324,8 @@ hmc_status hmc_dominant_kernel_info(const hmc_ctx* ctx, char* name, int32_t name
     n = "k_logreg_fused";
     per = ctx->C * ctx->cfg.num_leapfrog;
   } else if (uses_fused_elementwise(ctx)) {
-    n = "k_fused_elementwise";
-    per = ctx->C * ctx->cfg.num_leapfrog;
+    n = "k_elementwise_chain";
+    per = ctx->C * ctx->cfg.num_leapfrog * ctx->dom_transitions;
   } else if (ctx->target.id == HMC_T_CORR_GAUSS) {
     n = "k_corr_gauss_grad";
   } else if (ctx->target.id == HMC_T_LOGREG) {

@@ -154,10 +154,11 @@ struct DACoef {
 };
 static_assert(kDAKappa == 0.75, "eta below is m^-3/4");
 
-__device__ __forceinline__ DACoef da_prepare(const DAState* s, long long t) {
+// (`ahead`: of the step that many adapting transitions after the next one)
+__device__ __forceinline__ DACoef da_prepare(const DAState* s, long long t, int ahead = 0) {
   DACoef c{0.0, 0.0, 0.0, 0};
   if (!s->adapt || t >= s->num_adapt) return c;
-  const double m = static_cast<double>(s->m + 1);
+  const double m = static_cast<double>(s->m + 1 + ahead);
   const double r = sqrt(m);
   c.w = 1.0 / (m + kDAT0);
   c.sq = r / kDAGamma;

@@ -154,8 +154,24 @@ constexpr int kFusedElementwiseMaxDim = 1024;
 // Blocks the accept / fused kernels launch for C chains (one warp per chain).
 unsigned accept_blocks(int C);
 
-cudaError_t launch_fused_elementwise(int target_id, const StepArgs& a, cudaStream_t s,
-                                     KernelTimer* timer = nullptr);
+// Device words through which the CTAs of an adapting multi-transition launch
+// meet: CTAs that left (0 between launches), a flag that a wait gave up, and
+// two statistics per 8-chain tile (all bits set between launches).
+struct ChainSync {
+  unsigned* left = nullptr;
+  int* err = nullptr;
+  unsigned long long* slots = nullptr;
+};
+inline size_t chain_sync_bytes(int64_t C) { return 16 + 16 * static_cast<size_t>((C + 7) / 8); }
+
+// Transitions a.t_full .. a.t_full + T - 1 of the standard normal or the
+// funnel in one launch; transition keep_from + k writes output k (samples
+// [k][C x D], trace_eps [k], trace_acc [k][C]; each may be null).  adapting:
+// every transition of the range adapts the step size (a cooperative launch);
+// otherwise none but, with T = 1, the one does.
+cudaError_t launch_elementwise_chain(int target_id, const StepArgs& a, bool adapting, int T, long long keep_from,
+                                     float* samples, float* trace_eps, uint8_t* trace_acc, const ChainSync& sync,
+                                     cudaStream_t s, KernelTimer* timer);
 cudaError_t launch_plain_transition(const hmc_target& t, const StepArgs& a, const PlainBuffers& b,
                                     void* grad_ws, cudaStream_t s, KernelTimer* timer = nullptr);
 // The plain transition in two halves: the proposal with its log alpha into

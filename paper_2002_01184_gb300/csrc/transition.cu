@@ -1,17 +1,11 @@
 // HMC transition kernels (Section 2.1): momentum draw, leapfrog, energy,
 // Metropolis-Hastings select and the dual-averaging update.
 //
-// Fused path for targets whose gradient is elementwise plus row reductions
-// (standard normal, funnel): one warp per chain keeps x, p and g of its chain
-// in registers for all L leapfrog steps and the accept test, so one
-// transition is one launch that reads x, g once and writes them once.
-//
 // Plain path (any target): one launch per operation per leapfrog step --
 // begin (momentum + H_0), kick-drift, gradient, kick, ..., accept -- the
 // shape a framework that evaluates a batched target op by op produces.
 #include <cmath>
 
-#include "elementwise_tile.cuh"
 #include "hmc_device.cuh"
 #include "hmc_internal.h"
 
@@ -25,12 +19,6 @@ constexpr int kWarpsPerBlock = 8;
 
 __device__ __forceinline__ void finish_block(const StepArgs& a, float prob, bool has_chain) {
   accept_block_finish<kWarpsPerBlock>(a.da, a.partials, prob, has_chain, a.C, a.t_full);
-}
-
-// ------------------------------------------------------ fused elementwise --
-template <int TARGET, int NB>
-__global__ void __launch_bounds__(256) k_fused_elementwise(StepArgs a) {
-  elementwise_tile<TARGET, NB>(a, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x));
 }
 
 // ------------------------------------------------------------ plain path --
@@ -214,38 +202,12 @@ __global__ void k_momentum(uint64_t seed, uint32_t t, int C, int D, uint32_t cha
 }
 
 
-template <int TARGET, int NB>
-void launch_fe(const StepArgs& a, cudaStream_t s) {
-  k_fused_elementwise<TARGET, NB><<<accept_blocks(a.C), 256, 0, s>>>(a);
-}
-
-template <int TARGET>
-void launch_fe_dim(const StepArgs& a, cudaStream_t s) {
-  const int nblk = (a.D + 3) / 4;           // Philox blocks per chain
-  if (nblk <= 32) launch_fe<TARGET, 1>(a, s);
-  else if (nblk <= 64) launch_fe<TARGET, 2>(a, s);
-  else if (nblk <= 128) launch_fe<TARGET, 4>(a, s);
-  else launch_fe<TARGET, 8>(a, s);
-}
-
 inline unsigned elementwise_blocks(int64_t n) {
   const int64_t b = (n + 255) / 256;
   return static_cast<unsigned>(std::min<int64_t>(b, 152 * 16));
 }
 
 }  // namespace
-
-cudaError_t launch_fused_elementwise(int target_id, const StepArgs& a, cudaStream_t s,
-                                     KernelTimer* timer) {
-  if (a.D > kFusedElementwiseMaxDim) return cudaErrorInvalidValue;
-  if (target_id != HMC_T_STD_NORMAL && target_id != HMC_T_FUNNEL) return cudaErrorInvalidValue;
-  if (timer) timer->begin(s);
-  if (target_id == HMC_T_STD_NORMAL) launch_fe_dim<HMC_T_STD_NORMAL>(a, s);
-  else launch_fe_dim<HMC_T_FUNNEL>(a, s);
-  if (timer) timer->end(s);
-  count_launch();
-  return cudaGetLastError();
-}
 
 // the proposal: leapfrog trajectory (HMC; MALA at L = 1) or random walk
 static cudaError_t plain_proposal(const hmc_target& t, const StepArgs& a, const PlainBuffers& b,
