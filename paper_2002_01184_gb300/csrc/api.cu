@@ -58,7 +58,7 @@ struct hmc_ctx {
   bool use_lrgemm = false;      // tensor-core logistic regression, one-CTA tile products (dim > 128)
   hmc::LogregGemm lrg;
   int* lr_err = nullptr;
-  hmc::ChainSync chain_sync;       // multi-transition launches (elementwise targets)
+  hmc::ChainSync chain_sync;       // multi-transition launches (elementwise targets, small logistic regressions)
   // replica exchange (Section 2.2): K replicas per chain, rows c*K + k
   int K = 1;
   int64_t outer_chains = 0;
@@ -231,6 +231,7 @@ struct CreatePlan {
   bool use_lrtc = false, use_lrgemm = false;
   bool fused_logreg = false, fused_elementwise = false, plain_buffers = false;
   bool nuts_dense = false;
+  size_t chain_sync = 0;   // multi-transition launches: the words their CTAs meet through
   size_t grad_ws = 0;
   uint64_t bytes = 0;      // sum of the allocation requests, each at least 16 bytes
 };
@@ -311,7 +312,10 @@ CreatePlan plan_create(const hmc_target& t, int64_t num_chains, const hmc_config
   q.fused_logreg = fused && !q.use_lrtc && !q.use_lrgemm && hmc::logreg_fused_supported(t);
   q.fused_elementwise = fused && (t.id == HMC_T_STD_NORMAL || t.id == HMC_T_FUNNEL) &&
                         t.dim <= hmc::kFusedElementwiseMaxDim;
-  if (q.fused_elementwise) add(hmc::chain_sync_bytes(num_chains));
+  q.chain_sync = q.fused_elementwise ? hmc::chain_sync_bytes(num_chains)
+                 : q.fused_logreg && hmc::logreg_chain_supported(t) ? hmc::logreg_chain_sync_bytes(num_chains)
+                                                                    : 0;
+  if (q.chain_sync) add(q.chain_sync);
   q.plain_buffers = !q.fused_elementwise && !q.use_tc;
   if (q.plain_buffers) {
     add(4 * C * D);
@@ -366,6 +370,21 @@ bool uses_fused_elementwise(const hmc_ctx* ctx) {
          ctx->target.dim <= hmc::kFusedElementwiseMaxDim;
 }
 
+// small logistic regressions whose data fits shared memory
+bool uses_logreg_chain(const hmc_ctx* ctx) {
+  return uses_fused_logreg(ctx) && hmc::logreg_chain_supported(ctx->target);
+}
+
+// T transitions in one launch, either kind
+cudaError_t launch_chain(hmc_ctx* ctx, const StepArgs& a, bool adapting, int T, long long keep_from, float* samples,
+                         float* trace_eps, uint8_t* trace_acc) {
+  return uses_fused_elementwise(ctx)
+             ? hmc::launch_elementwise_chain(ctx->target.id, a, adapting, T, keep_from, samples, trace_eps, trace_acc,
+                                             ctx->chain_sync, ctx->stream, &ctx->timer)
+             : hmc::launch_logreg_chain(ctx->target, a, adapting, T, keep_from, samples, trace_eps, trace_acc,
+                                        ctx->chain_sync, ctx->stream, &ctx->timer);
+}
+
 StepArgs make_args(hmc_ctx* ctx, float* x, uint64_t t) {
   StepArgs a{};
   a.C = static_cast<int>(ctx->C);
@@ -398,11 +417,10 @@ cudaError_t enqueue_transition(hmc_ctx* ctx, const StepArgs& a) {
   if (ctx->use_lrtc)
     return hmc::launch_logreg_tc_transition(a, ctx->lrtc, ctx->lr_err, ctx->stream, &ctx->timer);
   if (ctx->use_lrgemm) return hmc::launch_logreg_gemm_transition(a, ctx->lrg, ctx->stream, &ctx->timer);
+  if (uses_fused_elementwise(ctx) || uses_logreg_chain(ctx))
+    return launch_chain(ctx, a, false, 1, a.t_full, a.sample_out, a.trace_eps, a.trace_acc);
   if (uses_fused_logreg(ctx))
     return hmc::launch_logreg_fused_transition(ctx->target, a, ctx->stream, &ctx->timer);
-  if (uses_fused_elementwise(ctx))
-    return hmc::launch_elementwise_chain(ctx->target.id, a, false, 1, a.t_full, a.sample_out, a.trace_eps,
-                                         a.trace_acc, ctx->chain_sync, ctx->stream, &ctx->timer);
   return hmc::launch_plain_transition(ctx->target, a, ctx->plain, ctx->grad_ws, ctx->stream,
                                       &ctx->timer);
 }
@@ -522,20 +540,20 @@ hmc_status enqueue_range(hmc_ctx* ctx, float* x, int64_t B, int64_t t_begin, int
     ctx->dom_transitions = chunk;
     return HMC_OK;
   }
-  // elementwise targets: the transitions that adapt the step size in one
-  // cooperative launch, the others in one ordinary launch
-  // (moments of transitions that still adapt: one launch per transition, below)
+  // elementwise targets and small logistic regressions: the transitions that
+  // adapt the step size in one cooperative launch, the others in one ordinary
+  // launch (elementwise moments of transitions that still adapt: one launch
+  // per transition, below)
   const int64_t t_fixed = ctx->cfg.adapt ? std::min(t_end, std::max(t_begin, ctx->cfg.num_adapt_steps)) : t_begin;
-  if (uses_fused_elementwise(ctx) && ctx->K == 1 && T > 0 && !(ctx->s_mean && t_fixed > B)) {
+  if (ctx->K == 1 && T > 0 &&
+      (uses_logreg_chain(ctx) || (uses_fused_elementwise(ctx) && !(ctx->s_mean && t_fixed > B)))) {
     for (int64_t t0 = t_begin; t0 < t_end;) {
       const int64_t stop = t0 < t_fixed ? t_fixed : t_end;
       const int n = static_cast<int>(std::min(chunk, stop - t0));
       StepArgs a = make_args(ctx, x, static_cast<uint64_t>(t0));
-      if (ctx->s_mean && t0 >= t_fixed)
+      if (ctx->s_mean && t0 + n > B)
         a.w = hmc::WelfordOut{ctx->s_mean, ctx->s_m2, ctx->s_bsize, ctx->bm_sum, ctx->bm_mean, ctx->bm_m2};
-      cudaError_t e = hmc::launch_elementwise_chain(ctx->target.id, a, t0 < t_fixed, n, B + out0, samples, trace_eps,
-                                                    trace_acc, ctx->chain_sync, ctx->stream,
-                                                    &ctx->timer);
+      cudaError_t e = launch_chain(ctx, a, t0 < t_fixed, n, B + out0, samples, trace_eps, trace_acc);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "chain launch");
       t0 += n;
     }
@@ -757,9 +775,10 @@ hmc_status hmc_create(const hmc_target* target, int64_t num_chains, const hmc_co
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&nd.side, cudaStreamNonBlocking);
   }
   if (e == cudaSuccess && plan.fused_logreg) e = hmc::logreg_fused_setup(*target);
-  if (e == cudaSuccess && plan.fused_elementwise) {
+  if (e == cudaSuccess && plan.fused_logreg && plan.chain_sync) e = hmc::logreg_chain_setup();
+  if (e == cudaSuccess && plan.chain_sync) {
     char* w = nullptr;
-    const size_t bytes = hmc::chain_sync_bytes(num_chains);
+    const size_t bytes = plan.chain_sync;
     e = ctx_alloc(ctx, &w, bytes);
     if (e == cudaSuccess) e = cudaMemsetAsync(w, 0, 16, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(w + 16, 0xFF, bytes - 16, ctx->stream);
@@ -1320,6 +1339,9 @@ hmc_status hmc_dominant_kernel_info(const hmc_ctx* ctx, char* name, int32_t name
     n = "k_lr_grad";
   } else if (ctx->use_lrgemm) {
     n = "k_gauss_tc_step<logreg>";   // both products of one gradient
+  } else if (uses_logreg_chain(ctx)) {
+    n = "k_logreg_chain";
+    per = ctx->C * ctx->cfg.num_leapfrog * ctx->dom_transitions;
   } else if (uses_fused_logreg(ctx)) {
     n = "k_logreg_fused";
     per = ctx->C * ctx->cfg.num_leapfrog;

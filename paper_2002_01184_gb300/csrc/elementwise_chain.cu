@@ -33,9 +33,7 @@
 #include <algorithm>
 #include <cmath>
 
-#include "hmc_device.cuh"
-#include "hmc_internal.h"
-#include "sm100_ptx.cuh"
+#include "chain_sync.cuh"
 
 namespace hmc {
 
@@ -55,7 +53,7 @@ struct EwArgs {
   uint8_t* trace_acc;
   unsigned* ctr;         // adapting launches: CTAs that left (0 between launches)
   int* err;
-  unsigned long long* slots;   // adapting launches: [2][tiles] statistics (kEmptySlot between launches)
+  unsigned long long* slots;   // adapting launches: [2][tiles] statistics (chain_sync.cuh)
 };
 
 template <int G>
@@ -63,28 +61,6 @@ __device__ __forceinline__ float group_sum(float v) {
 #pragma unroll
   for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// A tile's statistic -- the sum of its eight acceptance probabilities, never
-// negative -- meets the other CTAs in one 64-bit word whose sign bit says
-// whether it has been written: a transition uses one of two slots, and each
-// use of a slot flips the sign that means "written".  The word that announces
-// the value is the value, so no fence, arrival counter or second read lies
-// between the last CTA's store and everyone's sum (which took 3.3 us of every
-// adapting transition).  A slot is reused two transitions later: a CTA that
-// writes it has seen every CTA's next statistic, so all have read it.
-constexpr unsigned long long kEmptySlot = ~0ull;
-constexpr unsigned long long kSlotSign = 1ull << 63;
-
-__device__ __forceinline__ void put_slot(unsigned long long* p, double v, bool negative) {
-  const unsigned long long w = static_cast<unsigned long long>(__double_as_longlong(v)) | (negative ? kSlotSign : 0ull);
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
-}
-
-__device__ __forceinline__ unsigned long long read_slot(const unsigned long long* p) {
-  unsigned long long w;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
-  return w;
 }
 
 // Sum of all tiles' slots once written, in the order of tile_partial_then_da
@@ -116,7 +92,7 @@ __device__ __forceinline__ bool slots_sum(const unsigned long long* slots, int n
       }
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) acc += __longlong_as_double(static_cast<long long>(w[i] & ~kSlotSign));
+    for (int i = 0; i < 8; ++i) acc += slot_value(w[i]);
   }
   *sum = warp_sum_d(acc);
   return ok;
@@ -449,10 +425,7 @@ __global__ void __launch_bounds__(32 * W, W == 32 ? 1 : W == 16 ? 2 : NB == 1 ? 
         const bool ok = slots_sum(e.slots + (i & 1 ? ntiles : 0), ntiles, (i & 2) != 0, &sum);
         if (lane == 0) {
           if (ok) {
-            // sum / C, correctly rounded (Markstein 1990: the rounded
-            // reciprocal's quotient, corrected by its exact remainder)
-            const double q0 = sum * inv_c;
-            da_apply(&da_s, coef_s[i & 31], fma(fma(-q0, n_c, sum), inv_c, q0), a.t_full + i);
+            da_apply_sum(&da_s, coef_s[i & 31], sum, n_c, inv_c, a.t_full + i);
           } else {
             atomicExch(e.err, 4);
             flag_s = 1;
@@ -465,21 +438,7 @@ __global__ void __launch_bounds__(32 * W, W == 32 ? 1 : W == 16 ? 2 : NB == 1 ? 
     }
   }
   if (COOP) {
-    // CTA 0 writes the adaptation state (every CTA has read it: all have
-    // passed a meeting); the last CTA out empties the slots for the next launch
-    if (threadIdx.x == 0) {
-      if (blockIdx.x == 0) {
-        da_s.arrive = 0u;
-        *a.da = da_s;
-      }
-      __threadfence();
-      flag_s = atomicAdd(e.ctr, 1u) == gridDim.x - 1u ? 1 : 0;
-    }
-    __syncthreads();
-    if (flag_s) {
-      for (int b = threadIdx.x; b < 2 * ntiles; b += 32 * W) e.slots[b] = kEmptySlot;
-      if (threadIdx.x == 0) *e.ctr = 0u;
-    }
+    leave_adapting(a.da, &da_s, e.ctr, e.slots, 2 * ntiles);
   } else if (warp == 0) {
     // the last CTA to finish applies the last transition's statistic
     __syncwarp();

@@ -188,6 +188,14 @@ cudaError_t logreg_fused_setup(const hmc_target& t);
 unsigned logreg_fused_grid(int64_t C);
 cudaError_t launch_logreg_fused_transition(const hmc_target& t, const StepArgs& a, cudaStream_t s,
                                            KernelTimer* timer);
+// The same for a small logistic regression whose data fits an SM's shared
+// memory (one slot per chain; moments of adapting transitions too).
+bool logreg_chain_supported(const hmc_target& t);
+cudaError_t logreg_chain_setup();
+size_t logreg_chain_sync_bytes(int64_t C);
+cudaError_t launch_logreg_chain(const hmc_target& t, const StepArgs& a, bool adapting, int T, long long keep_from,
+                                float* samples, float* trace_eps, uint8_t* trace_acc, const ChainSync& sync,
+                                cudaStream_t s, KernelTimer* timer);
 // lp[r] *= beta, g[r, :] *= beta with beta = betas[r % K]
 cudaError_t launch_temper(int64_t rows, int D, float* lp, float* g, const float* betas, int K,
                           cudaStream_t s);

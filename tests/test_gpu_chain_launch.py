@@ -1,6 +1,7 @@
-"""Multi-transition launches of the elementwise targets: bit-identical to the
-batch's grouped launch (one warp per chain, one tile function per transition)
-at the edges of the lane groups, the chains packed into a warp and the CTAs."""
+"""Multi-transition launches of the elementwise targets and of small logistic
+regressions: bit-identical to the batch's grouped launch (one tile function per
+transition) at the edges of the lane groups, the chains packed into a warp, the
+row blocks and the CTAs."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -48,7 +49,30 @@ def test_chain_launch_equals_grouped_launch(kind, dim, chains, adapt, B, K):
     x0 = torch.randn(chains, dim, device="cuda", generator=g)
     cfg = H.make_config(4, 0.4 / dim ** 0.25, seed=7, adapt=adapt, target_accept=0.8, num_adapt_steps=B,
                         chain_offset=3)
-    target = H.make_target(kind, dim)
+    check_equal(H.make_target(kind, dim), cfg, x0, B, K)
+
+
+# (rows, dim, chains): rows around 16-row blocks and 256-row passes, dims around
+# the row strides, chains around the groups per CTA; the last does not fit
+# shared memory and takes one launch per transition
+LOGREG = [(1, 1, 1), (16, 2, 9), (17, 3, 153), (255, 7, 152), (257, 10, 305), (513, 11, 64), (769, 14, 300),
+          (800, 11, 70), (1025, 19, 20), (500, 20, 33), (500, 8, 1048), (30, 23, 700), (19, 512, 10), (40, 129, 90),
+          (2048, 64, 8)]
+
+
+@pytest.mark.parametrize("rows,dim,chains", LOGREG)
+@pytest.mark.parametrize("adapt,B,K", [(False, 2, 7), (True, 34, 3)])
+def test_logreg_chain_launch_equals_grouped_launch(rows, dim, chains, adapt, B, K):
+    g = torch.Generator(device="cuda").manual_seed(rows * 10007 + chains)
+    X = torch.randn(rows, dim, device="cuda", generator=g)
+    y = (torch.rand(rows, device="cuda", generator=g) < 0.5).float()
+    x0 = torch.randn(chains, dim, device="cuda", generator=g) / dim ** 0.5
+    cfg = H.make_config(3, 0.5 / (rows * dim) ** 0.5, seed=11, adapt=adapt, target_accept=0.8, num_adapt_steps=B,
+                        impl=H.HMC_IMPL_FUSED_SIMT)
+    check_equal(H.make_target("logreg", dim, X=X, y=y), cfg, x0, B, K)
+
+
+def check_equal(target, cfg, x0, B, K):
     one, ref = chain(target, cfg, x0, B, K, False), chain(target, cfg, x0, B, K, True)
     for u, v in zip(one[:4], ref[:4]):
         assert torch.equal(u, v)
