@@ -535,6 +535,13 @@ hmc_status hmc_target_vjp(const hmc_target* target, int64_t num_chains, const fl
                           const float* w, float* dx, void* workspace, uint64_t workspace_bytes,
                           void* cuda_stream);
 
+/* The same product from a gradient that hmc_target_log_prob_and_grad has
+ * already returned: dx[c, :] = w[c] * grad[c, :] (all device, caller-owned; dx
+ * may be grad).  The autograd binding keeps the forward pass's gradient and
+ * calls this in its backward pass.  HMC_E_INVALID on bad sizes or pointers. */
+hmc_status hmc_target_vjp_from_grad(int64_t num_chains, int32_t dim, const float* w, const float* grad,
+                                    float* dx, void* cuda_stream);
+
 /* Same as hmc_target_log_prob_and_grad, for callers that cannot allocate
  * device memory at all (no counterpart in the paper).  Some callers must not
  * call cudaMalloc when they evaluate a gradient: a host process that owns the

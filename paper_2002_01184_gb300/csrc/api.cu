@@ -404,6 +404,7 @@ StepArgs make_args(hmc_ctx* ctx, float* x, uint64_t t) {
   a.betas = ctx->betas;
   a.K = ctx->K;
   a.proposal = ctx->cfg.proposal;
+  a.merged = ctx->cfg.impl != HMC_IMPL_PLAIN;
   return a;
 }
 
@@ -1412,6 +1413,16 @@ hmc_status hmc_target_vjp(const hmc_target* target, int64_t num_chains, const fl
   float* lp_tmp = reinterpret_cast<float*>(base + ((gbytes + 255) & ~static_cast<size_t>(255)));
   cudaError_t e = hmc::launch_vjp(*target, num_chains, x, w, dx, lp_tmp, base,
                                   static_cast<cudaStream_t>(cuda_stream));
+  if (e != cudaSuccess) return cuda_fail(nullptr, e, "vjp launch");
+  return HMC_OK;
+}
+
+hmc_status hmc_target_vjp_from_grad(int64_t num_chains, int32_t dim, const float* w, const float* grad,
+                                    float* dx, void* cuda_stream) {
+  if (num_chains < 1 || num_chains > (1ll << 30) || dim < 1 || num_chains * static_cast<int64_t>(dim) > (1ll << 40))
+    return fail(nullptr, HMC_E_INVALID, "bad num_chains or dim");
+  if (!w || !grad || !dx) return fail(nullptr, HMC_E_INVALID, "w, grad and dx must be non-NULL");
+  cudaError_t e = hmc::launch_scale_rows(num_chains, dim, w, grad, dx, static_cast<cudaStream_t>(cuda_stream));
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "vjp launch");
   return HMC_OK;
 }

@@ -60,6 +60,9 @@ struct KernelTimer {
 cudaError_t launch_vjp(const hmc_target& t, int64_t C, const float* x, const float* w, float* dx,
                        float* lp_tmp, void* ws, cudaStream_t s);
 
+// dx[c, :] = w[c] g[c, :]
+cudaError_t launch_scale_rows(int64_t C, int D, const float* w, const float* g, float* dx, cudaStream_t s);
+
 // Set the error text that hmc_last_error(NULL) returns on this thread.
 void set_global_error(const std::string& msg);
 
@@ -69,8 +72,8 @@ int current_sm_count();
 // Bytes of scratch the batched gradient of `t` needs for C chains.
 size_t grad_workspace_bytes(const hmc_target& t, int64_t C);
 
-// log p and gradient of x [C x D] into lp [C], g [C x D] with the plain
-// (one GEMM per product) kernels; `ws` holds grad_workspace_bytes bytes.
+// log p (dense targets: or null, none) and gradient of x [C x D] into lp [C],
+// g [C x D] with the plain (one GEMM per product) kernels; `ws` holds grad_workspace_bytes bytes.
 cudaError_t launch_grad(const hmc_target& t, int64_t C, const float* x, float* lp, float* g,
                         void* ws, cudaStream_t s, KernelTimer* timer = nullptr);
 
@@ -113,6 +116,7 @@ struct StepArgs {
   const float* betas;     // replica exchange: row r targets p^betas[r % K]; null = 1
   int K;                  // replicas per chain (1: no tempering)
   int proposal;           // hmc_proposal_kind
+  int merged;             // general path: the elementwise steps between two gradients in one launch
   WelfordOut w;           // the pair kernel updates these at kept transitions (streaming)
 };
 
@@ -124,6 +128,7 @@ struct PlainBuffers {
   float* lpp;  // log-prob at the proposal [C]
   float* h0;   // initial Hamiltonian [C]
   float* la;   // log alpha [C] (the propose / select split)
+  bool half_dot;   // the accept kernel forms log p = <xp, gp> / 2 (dense Gaussian)
 };
 
 // NUTS (elementwise targets): per-chain scratch slots, the largest dim, and

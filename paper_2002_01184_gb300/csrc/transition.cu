@@ -67,10 +67,64 @@ __global__ void k_plain_kick(int64_t n, float* __restrict__ p, const float* __re
     p[i] = fmaf(0.5f * eps, gp[i], p[i]);
 }
 
+// The fused implementations' form of the same steps (dense Gaussians whose rows
+// the tensor maps cannot take): the elementwise steps between two gradients in
+// one launch, each operation rounded as in the launches above.
+// p ~ N(0, I), h0, then the first half kick (with the cached gradient) and drift
+__global__ void k_merged_begin(StepArgs a, PlainBuffers b) {
+  const int c = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (c >= a.C) return;
+  const int D = a.D;
+  const int64_t row = static_cast<int64_t>(c) * D;
+  const uint32_t chain = static_cast<uint32_t>(c) + a.chain_offset;
+  const float eps = a.da->eps;
+  float kin = 0.f;
+  for (int j = lane; 4 * j < D; j += 32) {
+    const float4 z = momentum4(a.seed, static_cast<uint32_t>(j), chain, a.t);
+    const float zz[4] = {z.x, z.y, z.z, z.w};
+    for (int i = 0; i < 4 && 4 * j + i < D; ++i) {
+      const int64_t e = row + 4 * j + i;
+      kin = fmaf(zz[i], zz[i], kin);
+      const float p = fmaf(0.5f * eps, a.g[e], zz[i]);
+      b.p[e] = p;
+      b.xp[e] = fmaf(eps, p, a.x[e]);
+    }
+  }
+  kin = warp_sum(kin);
+  if (lane == 0) b.h0[c] = -a.lp[c] + 0.5f * kin;
+}
+
+// two half kicks with the same gradient, then a drift
+__global__ void k_merged_step(int64_t n, float* __restrict__ p, const float* __restrict__ gp,
+                              float* __restrict__ xp, const DAState* __restrict__ da) {
+  const float eps = da->eps, h = 0.5f * eps;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  auto step = [&](float g, float& pi, float& xi) {
+    pi = fmaf(h, g, fmaf(h, g, pi));
+    xi = fmaf(eps, pi, xi);
+  };
+  // (the buffers are the context's own: aligned)
+  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; 4 * i < n; i += stride) {
+    if (4 * i + 4 <= n) {
+      const float4 g = reinterpret_cast<const float4*>(gp)[i];
+      float4 q = reinterpret_cast<float4*>(p)[i], x = reinterpret_cast<float4*>(xp)[i];
+      step(g.x, q.x, x.x);
+      step(g.y, q.y, x.y);
+      step(g.z, q.z, x.z);
+      step(g.w, q.w, x.w);
+      reinterpret_cast<float4*>(p)[i] = q;
+      reinterpret_cast<float4*>(xp)[i] = x;
+    } else {
+      for (int64_t k = 4 * i; k < n; ++k) step(gp[k], p[k], xp[k]);
+    }
+  }
+}
+
 // Random-walk proposal (Section 4.1's composition with a symmetric inner
-// kernel): xp = x + eps z with z the transition's momentum draws; p = 0, so
-// the energies below reduce to log alpha = log p(xp) - log p(x).
-__global__ void k_rw_begin(StepArgs a, PlainBuffers b) {
+// kernel): xp = x + eps z with z the transition's momentum draws; without a
+// momentum the energies below reduce to log alpha = log p(xp) - log p(x).
+__global__ void k_rw_begin(StepArgs a, PlainBuffers b, bool vec) {
   const int c = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (c >= a.C) return;
@@ -79,26 +133,50 @@ __global__ void k_rw_begin(StepArgs a, PlainBuffers b) {
   const uint32_t chain = static_cast<uint32_t>(c) + a.chain_offset;
   const float eps = a.da->eps;
   for (int j = lane; 4 * j < D; j += 32) {
-    const float4 z = momentum4(a.seed, static_cast<uint32_t>(j), chain, a.t);
-    const float zz[4] = {z.x, z.y, z.z, z.w};
-    for (int i = 0; i < 4 && 4 * j + i < D; ++i) {
-      const int64_t e = row + 4 * j + i;
-      b.p[e] = 0.f;
-      b.xp[e] = fmaf(eps, zz[i], a.x[e]);
+    const int64_t e = row + 4 * j;
+    if (vec) {
+      const float4 x = *reinterpret_cast<const float4*>(a.x + e);
+      const float4 z = momentum4(a.seed, static_cast<uint32_t>(j), chain, a.t);
+      *reinterpret_cast<float4*>(b.xp + e) =
+          make_float4(fmaf(eps, z.x, x.x), fmaf(eps, z.y, x.y), fmaf(eps, z.z, x.z), fmaf(eps, z.w, x.w));
+    } else {
+      const float4 z = momentum4(a.seed, static_cast<uint32_t>(j), chain, a.t);
+      const float zz[4] = {z.x, z.y, z.z, z.w};
+      for (int i = 0; i < 4 && 4 * j + i < D; ++i) b.xp[e + i] = fmaf(eps, zz[i], a.x[e + i]);
     }
   }
   if (lane == 0) b.h0[c] = -a.lp[c];
 }
 
-// log alpha = H_0 - H_L of chain c (warp per chain; every lane gets it)
+// log alpha = H_0 - H_L of chain c (warp per chain; every lane gets it).  The
+// dense Gaussian's log p = <xp, gp> / 2 is formed here (a launch of its own
+// would read both rows once more).
 __device__ __forceinline__ float plain_log_alpha(const StepArgs& a, const PlainBuffers& b, int c,
                                                  int lane) {
   const int D = a.D;
   const int64_t row = static_cast<int64_t>(c) * D;
+  float lpp;
+  if (b.half_dot) {
+    float s = 0.f;
+#pragma unroll 4
+    for (int d = lane; d < D; d += 32) s = fmaf(b.xp[row + d], b.gp[row + d], s);
+    lpp = 0.5f * warp_sum(s);
+    if (lane == 0) b.lpp[c] = lpp;
+  } else {
+    lpp = b.lpp[c];
+  }
   float kin = 0.f;
-  for (int d = lane; d < D; d += 32) kin = fmaf(b.p[row + d], b.p[row + d], kin);
-  kin = 0.5f * warp_sum(kin);
-  const float h1 = -b.lpp[c] + kin;
+  if (a.proposal != HMC_PROPOSAL_RANDOM_WALK) {
+    const float h = 0.5f * a.da->eps;
+#pragma unroll 4
+    for (int d = lane; d < D; d += 32) {
+      float p = b.p[row + d];
+      if (a.merged) p = fmaf(h, b.gp[row + d], p);      // the trajectory's last half kick
+      kin = fmaf(p, p, kin);
+    }
+    kin = 0.5f * warp_sum(kin);
+  }
+  const float h1 = -lpp + kin;
   float la = b.h0[c] - h1;
   if (!isfinite(la)) la = -INFINITY;
   return la;
@@ -113,12 +191,17 @@ __device__ __forceinline__ float plain_select(const StepArgs& a, const PlainBuff
   int acc = 0;
   if (lane == 0) acc = accept_log_uniform(a.seed, chain, a.t) < la;
   acc = __shfl_sync(0xffffffffu, acc, 0);
+#pragma unroll 4
   for (int d = lane; d < D; d += 32) {
+    float x;
     if (acc) {
-      a.x[row + d] = b.xp[row + d];
+      x = b.xp[row + d];
+      a.x[row + d] = x;
       a.g[row + d] = b.gp[row + d];
+    } else if (a.sample_out) {
+      x = a.x[row + d];
     }
-    if (a.sample_out) a.sample_out[row + d] = a.x[row + d];
+    if (a.sample_out) a.sample_out[row + d] = x;
   }
   if (lane == 0) {
     if (acc) a.lp[c] = b.lpp[c];
@@ -209,24 +292,47 @@ inline unsigned elementwise_blocks(int64_t n) {
 
 }  // namespace
 
+// whether log p of the proposal is left to plain_log_alpha
+static bool plain_half_dot(const hmc_target& t, const StepArgs& a) {
+  return t.id == HMC_T_CORR_GAUSS && a.K == 1;
+}
+
 // the proposal: leapfrog trajectory (HMC; MALA at L = 1) or random walk
 static cudaError_t plain_proposal(const hmc_target& t, const StepArgs& a, const PlainBuffers& b,
                                   void* grad_ws, cudaStream_t s, KernelTimer* timer) {
   const int64_t n = static_cast<int64_t>(a.C) * a.D;
-  if (a.proposal == HMC_PROPOSAL_RANDOM_WALK) {
-    k_rw_begin<<<accept_blocks(a.C), 256, 0, s>>>(a, b);
-    count_launch();
-    cudaError_t e = launch_grad(t, a.C, b.xp, b.lpp, b.gp, grad_ws, s, timer);
+  auto gradient = [&](bool end) {
+    // (a trajectory's middle needs no log p)
+    const bool lp = end ? !plain_half_dot(t, a) : a.K > 1 || (t.id != HMC_T_CORR_GAUSS && t.id != HMC_T_LOGREG);
+    cudaError_t e = launch_grad(t, a.C, b.xp, lp ? b.lpp : nullptr, b.gp, grad_ws, s, timer);
     if (e == cudaSuccess && a.K > 1) e = launch_temper(a.C, a.D, b.lpp, b.gp, a.betas, a.K, s);
     return e;
+  };
+  if (a.proposal == HMC_PROPOSAL_RANDOM_WALK) {
+    const bool vec = a.D % 4 == 0 && (reinterpret_cast<uintptr_t>(a.x) & 15u) == 0;
+    k_rw_begin<<<accept_blocks(a.C), 256, 0, s>>>(a, b, vec);
+    count_launch();
+    return gradient(true);
+  }
+  if (a.merged) {
+    k_merged_begin<<<accept_blocks(a.C), 256, 0, s>>>(a, b);
+    count_launch();
+    for (int l = 0; l < a.L; ++l) {
+      if (l > 0) {
+        k_merged_step<<<elementwise_blocks((n + 3) / 4), 256, 0, s>>>(n, b.p, b.gp, b.xp, a.da);
+        count_launch();
+      }
+      const cudaError_t e = gradient(l == a.L - 1);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaGetLastError();
   }
   k_plain_begin<<<accept_blocks(a.C), 256, 0, s>>>(a, b);
   count_launch();
   for (int l = 0; l < a.L; ++l) {
     k_plain_kick_drift<<<elementwise_blocks(n), 256, 0, s>>>(n, b.p, b.gp, b.xp, a.da);
     count_launch();
-    cudaError_t e = launch_grad(t, a.C, b.xp, b.lpp, b.gp, grad_ws, s, timer);
-    if (e == cudaSuccess && a.K > 1) e = launch_temper(a.C, a.D, b.lpp, b.gp, a.betas, a.K, s);
+    const cudaError_t e = gradient(l == a.L - 1);
     if (e != cudaSuccess) return e;
     k_plain_kick<<<elementwise_blocks(n), 256, 0, s>>>(n, b.p, b.gp, a.da);
     count_launch();
@@ -234,8 +340,10 @@ static cudaError_t plain_proposal(const hmc_target& t, const StepArgs& a, const 
   return cudaGetLastError();
 }
 
-cudaError_t launch_plain_transition(const hmc_target& t, const StepArgs& a, const PlainBuffers& b,
+cudaError_t launch_plain_transition(const hmc_target& t, const StepArgs& a, const PlainBuffers& bufs,
                                     void* grad_ws, cudaStream_t s, KernelTimer* timer) {
+  PlainBuffers b = bufs;
+  b.half_dot = plain_half_dot(t, a);
   cudaError_t e = plain_proposal(t, a, b, grad_ws, s, timer);
   if (e != cudaSuccess) return e;
   k_plain_accept<<<accept_blocks(a.C), 256, 0, s>>>(a, b);
@@ -243,8 +351,10 @@ cudaError_t launch_plain_transition(const hmc_target& t, const StepArgs& a, cons
   return cudaGetLastError();
 }
 
-cudaError_t launch_plain_propose(const hmc_target& t, const StepArgs& a, const PlainBuffers& b,
+cudaError_t launch_plain_propose(const hmc_target& t, const StepArgs& a, const PlainBuffers& bufs,
                                  void* grad_ws, cudaStream_t s) {
+  PlainBuffers b = bufs;
+  b.half_dot = plain_half_dot(t, a);
   cudaError_t e = plain_proposal(t, a, b, grad_ws, s, nullptr);
   if (e != cudaSuccess) return e;
   k_plain_ratio<<<accept_blocks(a.C), 256, 0, s>>>(a, b);

@@ -108,6 +108,7 @@ def _load():
                                            ctypes.POINTER(ctypes.c_uint64)],
         "hmc_target_vjp": [ctypes.POINTER(hmc_target), ctypes.c_int64, P, P, P, P, ctypes.c_uint64,
                            P],
+        "hmc_target_vjp_from_grad": [ctypes.c_int64, ctypes.c_int32, P, P, P, P],
         "hmc_target_log_prob_and_grad_noalloc": [ctypes.POINTER(hmc_target), ctypes.c_int64, P, P,
                                                  P, P],
         "hmc_profile_dominant_kernel": [P, ctypes.c_int32],
@@ -359,6 +360,11 @@ def hmc_target_vjp_workspace_bytes(target, num_chains):
 def hmc_target_vjp(target, num_chains, x, w, dx, workspace, workspace_bytes, stream=None):
     _check(lib.hmc_target_vjp(ctypes.byref(target), int(num_chains), _ptr(x), _ptr(w), _ptr(dx),
                               _ptr(workspace), int(workspace_bytes), _stream(stream)))
+
+
+def hmc_target_vjp_from_grad(num_chains, dim, w, grad, dx, stream=None):
+    _check(lib.hmc_target_vjp_from_grad(int(num_chains), int(dim), _ptr(w), _ptr(grad), _ptr(dx),
+                                        _stream(stream)))
 
 
 def hmc_dominant_kernel_info(ctx):
