@@ -1,9 +1,11 @@
 """torch.autograd binding of the batched target log-density.
 
 ``TargetLogProb.apply(x, target)`` returns log p(x_c) for every chain row of
-x [C, D]; its backward calls the library's hand-written adjoint
-(``hmc_target_vjp``), which recomputes the forward pass instead of storing
-anything from it.  Both directions run in libhmc's kernels.
+x [C, D].  The forward call returns the gradient with it, so the gradient
+([C, D] floats) is what autograd keeps and the backward call only weights its
+rows (``hmc_target_vjp_from_grad``): evaluating the target a second time, as
+``hmc_target_vjp`` does, took as long as the forward pass.  Both directions run
+in libhmc's kernels.
 """
 import torch
 
@@ -33,20 +35,17 @@ class TargetLogProb(torch.autograd.Function):
         lp = torch.empty(C, dtype=torch.float32, device=x.device)
         g = torch.empty_like(x)
         hmc.hmc_target_log_prob_and_grad(target.c, C, x, lp, g, ws, nbytes)
-        ctx.save_for_backward(x)
-        ctx.target = target
+        # (x too: a backward pass after x was changed in place stays an error)
+        ctx.save_for_backward(x, g)
         return lp
 
     @staticmethod
     def backward(ctx, grad_lp):
-        (x,) = ctx.saved_tensors
-        target = ctx.target
-        C = x.shape[0]
-        nbytes = hmc.hmc_target_vjp_workspace_bytes(target.c, C)
-        ws = target.workspace(nbytes)
-        dx = torch.empty_like(x)
+        _, g = ctx.saved_tensors
+        C, D = g.shape
+        dx = torch.empty_like(g)
         w = grad_lp.to(torch.float32).contiguous()
-        hmc.hmc_target_vjp(target.c, C, x, w, dx, ws, nbytes)
+        hmc.hmc_target_vjp_from_grad(C, D, w, g, dx)
         return dx, None
 
 
