@@ -46,11 +46,11 @@ constexpr int kEpiWarps = 16;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr uint32_t kABytes = kBM * kBK * 4;                  // 16 KB
 
-// A tile of BN output columns (MMA N = 64, 128 or 256): the stage ring fills
-// the same 192 KB of shared memory with 4, 3 or 2 stages; the accumulator
-// takes BN tensor-memory columns.  Wider tiles re-read their A operand (the
+// A tile of BN output columns (MMA N): the stage ring fills about 192 KB of
+// shared memory with 4, 3 or 2 stages; the accumulator takes BN tensor-memory
+// columns.  Wider tiles re-read their A operand (the
 // chains' rows) fewer times: the logistic regression's products use them.
-template <int BN, int ST = (BN == 64 ? 4 : BN == 128 ? 3 : 2)>
+template <int BN, int ST = (BN <= 64 ? 4 : BN <= 160 ? 3 : 2)>
 struct Tile {
   static constexpr int kStages = ST;
   // two CTAs per SM when the ring is small enough (so that one's epilogue
@@ -59,12 +59,19 @@ struct Tile {
   static constexpr uint32_t kBBytes = BN * kBK * 4;
   static constexpr uint32_t kStageBytes = 2 * kABytes + 2 * kBBytes;
   static constexpr size_t kSmem = kStages * kStageBytes + 1024 + 256;
-  static constexpr uint32_t kTmemCols = BN;
-  static_assert(BN == 64 || BN == 128 || BN == 256, "tile width");
+  static constexpr uint32_t kTmemCols = BN <= 64 ? 64 : BN <= 128 ? 128 : 256;   // a power of 2
+  static_assert(BN % 32 == 0 && BN >= 64 && BN <= 256, "tile width");
   static_assert(kBM * (BN + 1) * 4 <= kStages * kStageBytes, "epilogue staging must fit the ring");
   static_assert(kSmem <= 227 * 1024, "shared memory");
 };
 constexpr size_t kSmemBytes = Tile<kBN>::kSmem;
+
+// k_gauss_tc_traj: a ring of 3 stages (144 KB) and a staging tile of its own
+// (the next step's loads are on their way while it is read)
+constexpr int kTrajBN = 64, kTrajStages = 3;
+constexpr uint32_t kTrajStgBytes = kBM * (kTrajBN + 1) * 4;
+constexpr size_t kTrajSmem = kTrajStages * Tile<kTrajBN, kTrajStages>::kStageBytes + kTrajStgBytes + 1024 + 256;
+static_assert(kTrajSmem <= 227 * 1024, "shared memory");
 
 // Epilogues of the tile product (the pipeline is the same for all three):
 //   kEpiGauss   G = -X P: the dense Gaussian's leapfrog update
@@ -103,7 +110,13 @@ struct TcStepArgs {
   const uint8_t* active;    // null, or per-chain flags: a tile with none set is skipped
 };
 
-template <int EPI, int BN = kBN, int ST = Tile<BN>::kStages>
+// Clusters of CM x CN tiles (CM chain blocks, CN column blocks): tiles of one
+// chain block read the same A, tiles of one column block the same B, so each CTA
+// loads its share of the rows of both and multicasts it to the others.  What
+// bounds these products without it is L2: a 128 x 64 tile takes 48 KB per 12
+// MMAs (0.28 us).  A stage is refilled once every CTA that gets this one's rows has
+// consumed it: the MMA issuer's commit arrives at all senders' barriers.
+template <int EPI, int BN = kBN, int ST = Tile<BN>::kStages, int CM = 1, int CN = 1>
 __global__ void __launch_bounds__(kThreads, Tile<BN, ST>::kCtasPerSm)
 k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant__ CUtensorMap mAlo,
                 const __grid_constant__ CUtensorMap mBhi, const __grid_constant__ CUtensorMap mBlo,
@@ -123,7 +136,15 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
-  if (a.active) {
+  constexpr bool kCluster = CM * CN > 1;
+  // place in the cluster (grid x: chain blocks, y: column blocks)
+  const int cm = CM > 1 ? static_cast<int>(blockIdx.x) % CM : 0, cn = CN > 1 ? static_cast<int>(blockIdx.y) % CN : 0;
+  uint16_t row_mask = 0, col_mask = 0;      // the tiles that share this one's A, B
+  if (kCluster) {
+    for (int j = 0; j < CN; ++j) row_mask |= static_cast<uint16_t>(1u << (cm + CM * j));
+    for (int i = 0; i < CM; ++i) col_mask |= static_cast<uint16_t>(1u << (i + CM * cn));
+  }
+  if (!kCluster && a.active) {
     // NUTS: a tile whose chains have all finished their trees has no work
     const int r = threadIdx.x;
     const bool mine = r < kBM && m0 + r < a.C && a.active[m0 + r] != 0;
@@ -136,7 +157,7 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       ptx::mbar_init(&full[s], 1);
-      ptx::mbar_init(&empty[s], 1);
+      ptx::mbar_init(&empty[s], CM + CN - 1);
     }
     ptx::mbar_init(acc_full, 1);
     ptx::fence_mbar_init();
@@ -150,7 +171,9 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
-  __syncthreads();
+  __syncwarp();
+  if (kCluster) ptx::cluster_sync();      // the peers' barriers exist before anything is sent
+  else __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
@@ -158,13 +181,26 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
     // ---- TMA producer
     for (int kc = 0; kc < nk; ++kc) {
       const int s = kc % kStages, round = kc / kStages;
-      if (kc >= kStages && !ptx::mbar_wait(&empty[s], (round - 1) & 1)) {
+      if (kc >= kStages &&
+          !(kCluster ? ptx::mbar_wait_cluster(&empty[s], (round - 1) & 1) : ptx::mbar_wait(&empty[s], (round - 1) & 1))) {
         atomicExch(a.err, 1);
         break;
       }
       uint8_t* st = smem + s * kStageBytes;
       ptx::mbar_arrive_expect_tx(&full[s], kStageBytes);
       const int kx = (kc0 + kc) * kBK;
+      if (kCluster) {
+        // this CTA's share: 128 / CN rows of A, BN / CM rows of B
+        constexpr int kRowsA = kBM / CN, kRowsB = BN / CM;
+        static_assert(kRowsA % 8 == 0 && kRowsB % 8 == 0, "whole swizzle atoms");
+        uint8_t* sa = st + cn * kRowsA * 128;
+        uint8_t* sb = st + 2 * kABytes + cm * kRowsB * 128;
+        ptx::tma_load_2d_multicast(sa, &mAhi, &full[s], kx, m0 + cn * kRowsA, row_mask);
+        ptx::tma_load_2d_multicast(sa + kABytes, &mAlo, &full[s], kx, m0 + cn * kRowsA, row_mask);
+        ptx::tma_load_2d_multicast(sb, &mBhi, &full[s], kx, n0 + cm * kRowsB, col_mask);
+        ptx::tma_load_2d_multicast(sb + kBBytes, &mBlo, &full[s], kx, n0 + cm * kRowsB, col_mask);
+        continue;
+      }
       ptx::tma_load_2d(st, &mAhi, &full[s], kx, m0);
       ptx::tma_load_2d(st + kABytes, &mAlo, &full[s], kx, m0);
       ptx::tma_load_2d(st + 2 * kABytes, &mBhi, &full[s], kx, n0);
@@ -191,7 +227,10 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
         ptx::mma_tf32(tmem, a_hi, b_lo, idesc, 1u);
         ptx::mma_tf32(tmem, a_hi, b_hi, idesc, 1u);
       }
-      ptx::mma_commit(&empty[s]);
+      // (the last stages are not refilled: no arrival may be on its way to a
+      // peer that has left)
+      if (!kCluster) ptx::mma_commit(&empty[s]);
+      else if (kc + kStages < nk) ptx::mma_commit_multicast(&empty[s], row_mask | col_mask);
     }
     ptx::mma_commit(acc_full);
   } else if (warp >= 2) {
@@ -200,6 +239,24 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
     // the last MMA has completed; (2) the four warps walk the tile row by row
     // with lanes along the columns, so every global access is a coalesced
     // 128-byte row segment.
+    const int ew = warp - 2;
+    constexpr int kRows = kBM / kEpiWarps;            // rows per warp
+    // (Gaussian) this warp's positions and momenta, on their way during the MMAs
+    constexpr int kPre = EPI == kEpiGauss ? kRows : 1;
+    constexpr int kPreH = EPI == kEpiGauss ? BN / 32 : 1;
+    float pre_x[kPre][kPreH], pre_p[kPre][kPreH];
+    if (EPI == kEpiGauss) {
+#pragma unroll
+      for (int rr = 0; rr < kPre; ++rr)
+#pragma unroll
+        for (int h = 0; h < kPreH; ++h) {
+          const int m = m0 + ew + kEpiWarps * rr, n = n0 + lane + 32 * h;
+          const bool in = m < a.C && n < a.D;
+          const int64_t e = static_cast<int64_t>(m) * a.ld + n;
+          pre_x[rr][h] = in ? a.xhi_in[e] + a.xlo_in[e] : 0.f;
+          pre_p[rr][h] = in ? a.p[e] : 0.f;
+        }
+    }
     const bool ok = ptx::mbar_wait(acc_full, 0);
     if (!ok) atomicExch(a.err, 1);
     ptx::tc_fence_after();
@@ -207,9 +264,8 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
     const int cgroup = (warp - 2) >> 2;               // which quarter of the columns
     float* stg = reinterpret_cast<float*>(smem);
     constexpr int kLd = BN + 1;
-    constexpr int kCols = BN / 4;                     // 16, 32 or 64 per warp
 #pragma unroll
-    for (int c0 = cgroup * kCols; c0 < (cgroup + 1) * kCols; c0 += 16) {
+    for (int c0 = 16 * cgroup; c0 < BN; c0 += 64) {
       float acc[16];
       ptx::tmem_ld16(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + c0, acc);
 #pragma unroll
@@ -217,15 +273,12 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
     }
     asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
     const float eps = a.da->eps;
-    const float* __restrict__ xhi_in = a.xhi_in;
-    const float* __restrict__ xlo_in = a.xlo_in;
     float* __restrict__ xhi_out = a.xhi_out;
     float* __restrict__ xlo_out = a.xlo_out;
     float* __restrict__ pm = a.p;
     float* __restrict__ g_out = a.g_out;
-    const int ew = warp - 2;
-#pragma unroll 2
-    for (int rr = 0; rr < kBM / kEpiWarps; ++rr) {
+#pragma unroll(EPI == kEpiGauss ? kRows : 2)
+    for (int rr = 0; rr < kRows; ++rr) {
       const int r = ew + kEpiWarps * rr;
       const int m = m0 + r;
       if (!ok || m >= a.C) continue;                  // warp-uniform
@@ -267,17 +320,17 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
           const int n = n0 + cl;
           if (n < a.D) {
             const int64_t e = rowoff + n;
-            const float x = xhi_in[e] + xlo_in[e];
+            const float x = pre_x[rr][h];
             const float g = -stg[r * kLd + cl];
             if (!a.last) {
-              const float p = fmaf(eps, g, pm[e]);
+              const float p = fmaf(eps, g, pre_p[rr][h]);
               pm[e] = p;
               float hi, lo;
               split_tf32(fmaf(eps, p, x), hi, lo);
               xhi_out[e] = hi;
               xlo_out[e] = lo;
             } else {
-              pm[e] = fmaf(0.5f * eps, g, pm[e]);
+              pm[e] = fmaf(0.5f * eps, g, pre_p[rr][h]);
               g_out[e] = g;
               part = fmaf(x, g, part);
             }
@@ -289,15 +342,265 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
         // Gaussian: log p = <x, g> / 2; logistic regression: the rows'
         // log-likelihood terms, or the prior's -|theta|^2 / 2
         const float v = EPI == kEpiLrResid ? part : 0.5f * part;
-        if (lane == 0) a.lp_part[static_cast<int64_t>(m) * a.ntn + a.lp_col0 + blockIdx.y] = v;
+        // (a cluster's last column blocks may lie past the columns)
+        if (lane == 0 && n0 < a.ncols) a.lp_part[static_cast<int64_t>(m) * a.ntn + a.lp_col0 + blockIdx.y] = v;
       }
     }
   }
   ptx::tc_fence_before();
-  __syncthreads();
+  __syncwarp();
+  if (kCluster) ptx::cluster_sync();      // no CTA leaves while a peer's loads or arrivals may still reach it
+  else __syncthreads();
   if (warp == 0) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, kTmemCols);
+  }
+}
+
+// All leapfrog steps of a transition in one cooperative launch, one tile per
+// CTA, for trajectories whose tiles are all resident at once.  A launch per step
+// paid about 8 us besides its products (launch, tensor-memory and barrier
+// set-up, the first loads, the drain); here a step ends with a meeting of the
+// CTAs that share its chains (one counter per 128-chain block): the epilogue
+// keeps positions and momenta in registers, writes the next positions for the
+// others' loads, and the producer waits for all column blocks before it loads
+// them -- the next stages' rows of P, which never change, are on their way by
+// then.  Arithmetic, and the order of every sum, are k_gauss_tc_step's.
+// Measured, per step of 16 with begin and accept: 2048 chains x 512 dims 17.7 ->
+// 13.7 us, 2048 x 300 16.5 -> 10.6 us, 64 x 512 14.7 -> 13.0 us.  What bounds it
+// now is shared memory: 32 dims of a 128 x 64 tile bring 48 KB and their 12 MMAs
+// read 72 KB, 0.46 us at 128 bytes a cycle, 7.4 us for 512 dims.
+struct TcTrajArgs {
+  int C, D, L, ntn;
+  float* xhi[2];            // x_l at [(l - 1) & 1], row length D
+  float* xlo[2];
+  float* p;                 // momentum: read at the start, written after the last step
+  float* g_out;
+  float* lp_part;           // [C x ntn]
+  unsigned* met;            // [chain blocks] column blocks that have written their positions (zeroed before)
+  const DAState* da;
+  int* err;
+};
+
+template <int CM, int CN>
+__global__ void __launch_bounds__(kThreads, 1)
+k_gauss_tc_traj(const __grid_constant__ CUtensorMap mAhi0, const __grid_constant__ CUtensorMap mAlo0,
+                const __grid_constant__ CUtensorMap mAhi1, const __grid_constant__ CUtensorMap mAlo1,
+                const __grid_constant__ CUtensorMap mBhi, const __grid_constant__ CUtensorMap mBlo, TcTrajArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  using T = Tile<kTrajBN, kTrajStages>;
+  constexpr int BN = kTrajBN, kStages = kTrajStages;
+  constexpr bool kCluster = CM * CN > 1;
+  float* stg = reinterpret_cast<float*>(smem + kStages * T::kStageBytes);     // [kBM][BN + 1]
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * T::kStageBytes + kTrajStgBytes);
+  uint64_t* empty = full + kStages;
+  uint64_t* acc_full = empty + kStages;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
+  const int cm = CM > 1 ? static_cast<int>(blockIdx.x) % CM : 0, cn = CN > 1 ? static_cast<int>(blockIdx.y) % CN : 0;
+  uint16_t row_mask = 0, col_mask = 0;
+  for (int j = 0; j < CN; ++j) row_mask |= static_cast<uint16_t>(1u << (cm + CM * j));
+  for (int i = 0; i < CM; ++i) col_mask |= static_cast<uint16_t>(1u << (i + CM * cn));
+  const int nk = (a.D + kBK - 1) / kBK;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      ptx::mbar_init(&full[s], 1);
+      ptx::mbar_init(&empty[s], CM + CN - 1);
+    }
+    ptx::mbar_init(acc_full, 1);
+    ptx::fence_mbar_init();
+    ptx::prefetch_tensormap(&mAhi0);
+    ptx::prefetch_tensormap(&mAlo0);
+    ptx::prefetch_tensormap(&mAhi1);
+    ptx::prefetch_tensormap(&mAlo1);
+    ptx::prefetch_tensormap(&mBhi);
+    ptx::prefetch_tensormap(&mBlo);
+  }
+  if (warp == 0) {
+    ptx::tmem_alloc(tmem_slot, T::kTmemCols);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncwarp();
+  if (kCluster) ptx::cluster_sync();
+  else __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0 && lane == 0) {
+    // ---- TMA producer
+    constexpr int kRowsA = kBM / CN, kRowsB = BN / CM;
+    static_assert(kRowsA % 8 == 0 && kRowsB % 8 == 0, "whole swizzle atoms");
+    bool ok = true;
+    auto load = [&](const CUtensorMap* map, uint8_t* dst, int s, int k, int r, uint16_t mask) {
+      if (kCluster) ptx::tma_load_2d_multicast(dst, map, &full[s], k, r, mask);
+      else ptx::tma_load_2d(dst, map, &full[s], k, r);
+    };
+    auto arm_and_load_b = [&](int it, int kc) {
+      const int s = it % kStages, round = it / kStages;
+      if (it >= kStages && !(kCluster ? ptx::mbar_wait_cluster(&empty[s], (round - 1) & 1)
+                                      : ptx::mbar_wait(&empty[s], (round - 1) & 1))) {
+        ok = false;
+        return;
+      }
+      uint8_t* sb = smem + s * T::kStageBytes + 2 * kABytes + cm * kRowsB * 128;
+      ptx::mbar_arrive_expect_tx(&full[s], T::kStageBytes);
+      load(&mBhi, sb, s, kc * kBK, n0 + cm * kRowsB, col_mask);
+      load(&mBlo, sb + T::kBBytes, s, kc * kBK, n0 + cm * kRowsB, col_mask);
+    };
+    for (int l = 1; l <= a.L && ok; ++l) {
+      const CUtensorMap* hi = l & 1 ? &mAhi0 : &mAhi1;
+      const CUtensorMap* lo = l & 1 ? &mAlo0 : &mAlo1;
+      auto load_a = [&](int it, int kc) {
+        const int s = it % kStages;
+        uint8_t* sa = smem + s * T::kStageBytes + cn * kRowsA * 128;
+        load(hi, sa, s, kc * kBK, m0 + cn * kRowsA, row_mask);
+        load(lo, sa + kABytes, s, kc * kBK, m0 + cn * kRowsA, row_mask);
+      };
+      const int it0 = (l - 1) * nk, ahead = min(kStages, nk);
+      for (int kc = 0; kc < ahead && ok; ++kc) arm_and_load_b(it0 + kc, kc);
+      if (l > 1 && ok) {
+        // every column block of these chains has written x_l
+        const unsigned target = static_cast<unsigned>(l - 1) * gridDim.y;
+        const unsigned long long t0 = ptx::global_timer_ns();
+        unsigned seen = 0;
+        while (true) {
+          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.met + blockIdx.x) : "memory");
+          if (seen >= target) break;
+          if (ptx::global_timer_ns() - t0 > ptx::kWaitLimitNs) {
+            ok = false;
+            break;
+          }
+        }
+        // (written with generic stores, read by the async proxy)
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+      }
+      for (int kc = 0; kc < ahead && ok; ++kc) load_a(it0 + kc, kc);
+      for (int kc = ahead; kc < nk && ok; ++kc) {
+        arm_and_load_b(it0 + kc, kc);
+        if (ok) load_a(it0 + kc, kc);
+      }
+    }
+    if (!ok) atomicExch(a.err, 1);
+  } else if (warp == 1 && lane == 0) {
+    // ---- MMA issuer
+    constexpr uint32_t idesc = ptx::idesc_tf32(kBM, BN);
+    bool ok = true;
+    for (int l = 1; l <= a.L && ok; ++l) {
+      for (int kc = 0; kc < nk; ++kc) {
+        const int it = (l - 1) * nk + kc, s = it % kStages, round = it / kStages;
+        // (x_l is loaded once the epilogues of step l - 1, which read the
+        // accumulator, have all written it: the accumulator is free)
+        if (!ptx::mbar_wait(&full[s], round & 1)) {
+          atomicExch(a.err, 1);
+          ok = false;
+          break;
+        }
+        ptx::tc_fence_after();
+        const uint32_t st = ptx::smem_u32(smem + s * T::kStageBytes);
+#pragma unroll
+        for (int j = 0; j < kBK / 8; ++j) {
+          const uint64_t a_hi = ptx::sw128_kmajor_desc(st + 32 * j);
+          const uint64_t a_lo = ptx::sw128_kmajor_desc(st + kABytes + 32 * j);
+          const uint64_t b_hi = ptx::sw128_kmajor_desc(st + 2 * kABytes + 32 * j);
+          const uint64_t b_lo = ptx::sw128_kmajor_desc(st + 2 * kABytes + T::kBBytes + 32 * j);
+          ptx::mma_tf32(tmem, a_lo, b_hi, idesc, (kc | j) != 0 ? 1u : 0u);
+          ptx::mma_tf32(tmem, a_hi, b_lo, idesc, 1u);
+          ptx::mma_tf32(tmem, a_hi, b_hi, idesc, 1u);
+        }
+        // (no arrival for a stage that is not refilled: it may find its CTA gone)
+        if (it + kStages < a.L * nk) {
+          if (kCluster) ptx::mma_commit_multicast(&empty[s], row_mask | col_mask);
+          else ptx::mma_commit(&empty[s]);
+        }
+      }
+      if (ok) ptx::mma_commit(acc_full);
+    }
+  } else if (warp >= 2) {
+    // ---- epilogue: warp ew owns rows ew + 16 rr, lane columns lane + 32 h
+    const int ew = warp - 2, quarter = warp & 3, cgroup = ew >> 2;
+    constexpr int kRows = kBM / kEpiWarps, kH = BN / 32, kLd = BN + 1;
+    const float eps = a.da->eps;
+    float x[kRows][kH], p[kRows][kH];
+#pragma unroll
+    for (int rr = 0; rr < kRows; ++rr)
+#pragma unroll
+      for (int h = 0; h < kH; ++h) {
+        const int m = m0 + ew + kEpiWarps * rr, n = n0 + lane + 32 * h;
+        const bool in = m < a.C && n < a.D;
+        const int64_t e = static_cast<int64_t>(m) * a.D + n;
+        x[rr][h] = in ? a.xhi[0][e] + a.xlo[0][e] : 0.f;
+        p[rr][h] = in ? a.p[e] : 0.f;
+      }
+    bool ok = true;
+    for (int l = 1; l <= a.L && ok; ++l) {
+      ok = ptx::mbar_wait(acc_full, (l - 1) & 1);
+      if (!ok) atomicExch(a.err, 1);
+      ptx::tc_fence_after();
+      {
+        float acc[16];
+        const int c0 = 16 * cgroup;
+        ptx::tmem_ld16(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + c0, acc);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) stg[(quarter * 32 + lane) * kLd + c0 + j] = acc[j];
+      }
+      ptx::tc_fence_before();
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+      const bool last = l == a.L;
+      float* xhi = l & 1 ? a.xhi[1] : a.xhi[0];
+      float* xlo = l & 1 ? a.xlo[1] : a.xlo[0];
+#pragma unroll
+      for (int rr = 0; rr < kRows; ++rr) {
+        const int r = ew + kEpiWarps * rr, m = m0 + r;
+        float part = 0.f;
+#pragma unroll
+        for (int h = 0; h < kH; ++h) {
+          const int n = n0 + lane + 32 * h;
+          const int64_t e = static_cast<int64_t>(m) * a.D + n;
+          const bool in = ok && m < a.C && n < a.D;
+          const float g = -stg[r * kLd + lane + 32 * h];
+          if (!last) {
+            p[rr][h] = fmaf(eps, g, p[rr][h]);
+            x[rr][h] = fmaf(eps, p[rr][h], x[rr][h]);
+            if (in) {
+              float hi, lo;
+              split_tf32(x[rr][h], hi, lo);
+              xhi[e] = hi;
+              xlo[e] = lo;
+            }
+          } else if (in) {
+            a.p[e] = fmaf(0.5f * eps, g, p[rr][h]);
+            a.g_out[e] = g;
+            part = fmaf(x[rr][h], g, part);
+          }
+        }
+        if (last && ok && m < a.C) {
+          part = warp_sum(part);
+          if (lane == 0 && n0 < a.D) a.lp_part[static_cast<int64_t>(m) * a.ntn + blockIdx.y] = 0.5f * part;
+        }
+      }
+      if (!last) {
+        // positions for the other CTAs' loads (another proxy), then this
+        // CTA's arrival
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+        if (threadIdx.x == 64 && ok) {
+          __threadfence();
+          atomicAdd(a.met + blockIdx.x, 1u);
+        }
+      }
+    }
+  }
+  ptx::tc_fence_before();
+  __syncwarp();
+  if (kCluster) ptx::cluster_sync();
+  else __syncthreads();
+  if (warp == 0) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, T::kTmemCols);
   }
 }
 
@@ -519,11 +822,15 @@ struct TcBeginAccept {
   float* lp_part;
   float* h0;
   int ntn;
+  unsigned* met;     // begin: the trajectory launch's counters, zeroed (null: none)
+  int nmet;
 };
 
 // p0 ~ N(0, I); H0; half kick with the cached gradient; first drift (warp per chain)
 __global__ void k_gauss_tc_begin(TcBeginAccept b) {
   const StepArgs& a = b.s;
+  if (b.met && blockIdx.x == 0)
+    for (int i = threadIdx.x; i < b.nmet; i += blockDim.x) b.met[i] = 0u;
   const int c = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (c >= a.C) return;
@@ -531,20 +838,41 @@ __global__ void k_gauss_tc_begin(TcBeginAccept b) {
   const int64_t row = static_cast<int64_t>(c) * D, rowi = static_cast<int64_t>(c) * b.ld;
   const uint32_t chain = static_cast<uint32_t>(c) + a.chain_offset;
   const float eps = a.da->eps;
+  // (the workspace's rows are a multiple of 4 floats; the state's as D has it)
+  const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(a.x) & 15u) == 0;
   float kin = 0.f;
   for (int j = lane; 4 * j < D; j += 32) {
+    float xx[4] = {0.f, 0.f, 0.f, 0.f}, gg[4] = {0.f, 0.f, 0.f, 0.f};
+    if (vec) {
+      const float4 xv = *reinterpret_cast<const float4*>(a.x + row + 4 * j);
+      const float4 gv = *reinterpret_cast<const float4*>(a.g + row + 4 * j);
+      xx[0] = xv.x; xx[1] = xv.y; xx[2] = xv.z; xx[3] = xv.w;
+      gg[0] = gv.x; gg[1] = gv.y; gg[2] = gv.z; gg[3] = gv.w;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (4 * j + i < D) {
+          xx[i] = a.x[row + 4 * j + i];
+          gg[i] = a.g[row + 4 * j + i];
+        }
+    }
     const float4 z = momentum4(a.seed, static_cast<uint32_t>(j), chain, a.t);
     const float zz[4] = {z.x, z.y, z.z, z.w};
-    for (int i = 0; i < 4 && 4 * j + i < D; ++i) {
-      const int64_t e = row + 4 * j + i, ei = rowi + 4 * j + i;
-      kin = fmaf(zz[i], zz[i], kin);
-      const float p = fmaf(0.5f * eps, a.g[e], zz[i]);
-      b.p[ei] = p;
-      float hi, lo;
-      split_tf32(fmaf(eps, p, a.x[e]), hi, lo);
-      b.xhi[ei] = hi;
-      b.xlo[ei] = lo;
+    float p[4], hi[4], lo[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      // (a ragged row's last padding columns stay zero)
+      const bool in = 4 * j + i < D;
+      p[i] = hi[i] = lo[i] = 0.f;
+      if (in) {
+        kin = fmaf(zz[i], zz[i], kin);
+        p[i] = fmaf(0.5f * eps, gg[i], zz[i]);
+        split_tf32(fmaf(eps, p[i], xx[i]), hi[i], lo[i]);
+      }
     }
+    *reinterpret_cast<float4*>(b.p + rowi + 4 * j) = make_float4(p[0], p[1], p[2], p[3]);
+    *reinterpret_cast<float4*>(b.xhi + rowi + 4 * j) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<float4*>(b.xlo + rowi + 4 * j) = make_float4(lo[0], lo[1], lo[2], lo[3]);
   }
   kin = warp_sum(kin);
   if (lane == 0) b.h0[c] = -a.lp[c] + 0.5f * kin;
@@ -563,24 +891,34 @@ __global__ void k_gauss_tc_accept(TcBeginAccept b) {
     const int64_t row = static_cast<int64_t>(c) * D, rowi = static_cast<int64_t>(c) * b.ld;
     const uint32_t chain = static_cast<uint32_t>(c) + a.chain_offset;
     float kin = 0.f;
+#pragma unroll 8
     for (int d = lane; d < D; d += 32) kin = fmaf(b.p[rowi + d], b.p[rowi + d], kin);
     kin = 0.5f * warp_sum(kin);
+    // the tiles' terms in order (a logistic regression has one per 64 rows):
+    // the lanes load 32 at a time, every lane adds them up
     float lp1 = 0.f;
-    if (lane == 0)
-      for (int k = 0; k < b.ntn; ++k) lp1 += b.lp_part[static_cast<int64_t>(c) * b.ntn + k];
-    lp1 = __shfl_sync(0xffffffffu, lp1, 0);
+    for (int k0 = 0; k0 < b.ntn; k0 += 32) {
+      const float v = k0 + lane < b.ntn ? b.lp_part[static_cast<int64_t>(c) * b.ntn + k0 + lane] : 0.f;
+      const int nv = min(32, b.ntn - k0);
+      for (int k = 0; k < nv; ++k) lp1 += __shfl_sync(0xffffffffu, v, k);
+    }
     float la = b.h0[c] - (-lp1 + kin);
     if (!isfinite(la)) la = -INFINITY;
     int acc = 0;
     if (lane == 0) acc = accept_log_uniform(a.seed, chain, a.t) < la;
     acc = __shfl_sync(0xffffffffu, acc, 0);
+#pragma unroll 8
     for (int d = lane; d < D; d += 32) {
       const int64_t e = row + d, ei = rowi + d;
+      float x = 0.f;
       if (acc) {
-        a.x[e] = b.xhi[ei] + b.xlo[ei];
+        x = b.xhi[ei] + b.xlo[ei];
+        a.x[e] = x;
         a.g[e] = b.gL[ei];
+      } else if (a.sample_out) {
+        x = a.x[e];
       }
-      if (a.sample_out) a.sample_out[e] = a.x[e];
+      if (a.sample_out) a.sample_out[e] = x;
     }
     if (lane == 0) {
       if (acc) a.lp[c] = lp1;
@@ -610,6 +948,48 @@ struct LrSumArgs {
   const DAState* da;
 };
 
+// The middle steps need no sum over the dims: a thread per four dims, so that
+// the chip's loads are in flight together (a warp per chain left 700 chains of
+// 301 dims on 88 CTAs with 16 dependent rounds: 20.8 us, now 7.0 us).
+constexpr int kMaxSplit = 16;      // the most K-splits of the gradient product G = R X
+
+__global__ void __launch_bounds__(256) k_lr_gemm_update_middle(LrSumArgs b) {
+  const int ld4 = b.ld >> 2;
+  const int64_t n4 = static_cast<int64_t>(b.C) * ld4;
+  const int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (e >= n4) return;
+  const int j = static_cast<int>(e % ld4);
+  const float eps = b.da->eps;
+  const float4* part = reinterpret_cast<const float4*>(b.part);
+  float4 v[kMaxSplit];
+#pragma unroll
+  for (int sp = 0; sp < kMaxSplit; ++sp)
+    if (sp < b.S) v[sp] = part[sp * n4 + e];
+  const float4 h = reinterpret_cast<const float4*>(b.xhi_in)[e];
+  const float4 l = reinterpret_cast<const float4*>(b.xlo_in)[e];
+  const float4 pv = reinterpret_cast<float4*>(b.p)[e];
+  float g[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int sp = 0; sp < kMaxSplit; ++sp)
+    if (sp < b.S) {
+      g[0] += v[sp].x; g[1] += v[sp].y; g[2] += v[sp].z; g[3] += v[sp].w;
+    }
+  const float th[4] = {h.x + l.x, h.y + l.y, h.z + l.z, h.w + l.w};
+  const float pin[4] = {pv.x, pv.y, pv.z, pv.w};
+  float pout[4], hi[4], lo[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    // padding dims (>= D) hold zeros everywhere and stay zero
+    const float gk = 4 * j + k < b.D ? g[k] - th[k] : 0.f;
+    pout[k] = fmaf(eps, gk, pin[k]);
+    split_tf32(fmaf(eps, pout[k], th[k]), hi[k], lo[k]);
+  }
+  reinterpret_cast<float4*>(b.p)[e] = make_float4(pout[0], pout[1], pout[2], pout[3]);
+  reinterpret_cast<float4*>(b.xhi_out)[e] = make_float4(hi[0], hi[1], hi[2], hi[3]);
+  reinterpret_cast<float4*>(b.xlo_out)[e] = make_float4(lo[0], lo[1], lo[2], lo[3]);
+}
+
+// the last step (and its |theta|^2)
 __global__ void k_lr_gemm_update(LrSumArgs b) {
   const int c = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -727,6 +1107,68 @@ inline unsigned blocks_for(int64_t n) {
 
 }  // namespace
 
+namespace {
+using StepKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, TcStepArgs);
+using TrajKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, TcTrajArgs);
+StepKernel gauss_step_kernel(int c) {
+  return c == 1 ? k_gauss_tc_step<kEpiGauss> : k_gauss_tc_step<kEpiGauss, kBN, Tile<kBN>::kStages, 2, 2>;
+}
+TrajKernel gauss_traj_kernel(int c) { return c == 1 ? k_gauss_tc_traj<1, 1> : k_gauss_tc_traj<2, 2>; }
+
+// grid, block and attributes of a trajectory launch
+struct TrajLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  TrajLaunch(const GaussTc& tc, int64_t mt, cudaStream_t s) {
+    const unsigned cm = static_cast<unsigned>(tc.cm), cn = static_cast<unsigned>(tc.cn);
+    cfg.gridDim = dim3((static_cast<unsigned>(mt) + cm - 1) / cm * cm, (tc.ntn + cn - 1) / cn * cn);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kTrajSmem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cm;
+    attr[0].val.clusterDim.y = cn;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeCooperative;
+    attr[1].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+  }
+};
+
+// whether all tiles of the trajectory launch are resident at once
+cudaError_t gauss_traj_fits(const GaussTc& tc, int64_t mt, bool* fits) {
+  *fits = false;
+  if (mt * tc.ntn > 4096) return cudaSuccess;
+  TrajLaunch t(tc, mt, nullptr);
+  t.cfg.numAttrs = 1;
+  int clusters = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&clusters, gauss_traj_kernel(tc.cm), &t.cfg);
+  if (e != cudaSuccess) return e;
+  *fits = clusters * tc.cm * tc.cn >= static_cast<int>(t.cfg.gridDim.x * t.cfg.gridDim.y);
+  return cudaSuccess;
+}
+
+// one launch of a tile kernel whose clusters are cm x cn tiles
+cudaError_t launch_clusters(StepKernel k, dim3 grid, int cm, int cn, size_t smem, cudaStream_t s,
+                            const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const CUtensorMap& md,
+                            const TcStepArgs& st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((grid.x + cm - 1) / cm * cm, (grid.y + cn - 1) / cn * cn, grid.z);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(cm);
+  attr[0].val.clusterDim.y = static_cast<unsigned>(cn);
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cm * cn > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, ma, mb, mc, md, st);
+}
+}  // namespace
+
 bool gauss_tc_supported(const hmc_target& t) {
   return t.id == HMC_T_CORR_GAUSS && t.dim % 4 == 0 && encode_fn() != nullptr;
 }
@@ -737,7 +1179,8 @@ size_t gauss_tc_workspace_bytes(const hmc_target& t, int64_t C) {
   auto a = [](size_t b) { return (b + 1023) & ~static_cast<size_t>(1023); };
   const size_t image = t.dim <= 256 ? a(kGaussPairImageFloats * 4) : 0;
   const size_t blocks = t.dim <= 256 ? 6 * a(static_cast<size_t>(gauss_pair_padded_chains(C)) * t.dim * 4) + a(24) : 0;
-  return 2 * a(DD * 4) + 6 * a(CD * 4) + a(C * ntn * 4) + a(C * 4) + a(sizeof(int)) + image + blocks;
+  const size_t met = t.dim > 256 ? a(((static_cast<size_t>(C) + kBM - 1) / kBM + 1) * 4) : 0;
+  return 2 * a(DD * 4) + 6 * a(CD * 4) + a(C * ntn * 4) + a(C * 4) + a(sizeof(int)) + image + blocks + met;
 }
 
 cudaError_t gauss_tc_setup(GaussTc* tc, const hmc_target& t, int64_t C, void* ws, cudaStream_t s) {
@@ -765,6 +1208,7 @@ cudaError_t gauss_tc_setup(GaussTc* tc, const hmc_target& t, int64_t C, void* ws
     tc->pair_w = take(3 * blk);
     tc->pair_stat = reinterpret_cast<unsigned long long*>(take(3 * sizeof(unsigned long long)));
   }
+  tc->met = t.dim > 256 ? reinterpret_cast<unsigned*>(take(((static_cast<size_t>(C) + kBM - 1) / kBM + 1) * 4)) : nullptr;
   bool ok = make_map(&tc->mBhi, tc->Phi, t.dim, t.dim, kBN) &&
             make_map(&tc->mBlo, tc->Plo, t.dim, t.dim, kBN) &&
             make_map(&tc->mPhi128, tc->Phi, t.dim, t.dim, 128) &&
@@ -772,9 +1216,25 @@ cudaError_t gauss_tc_setup(GaussTc* tc, const hmc_target& t, int64_t C, void* ws
   for (int i = 0; i < 2 && ok; ++i)
     ok = make_map(&tc->mAhi[i], tc->xhi[i], C, t.dim, kBM) &&
          make_map(&tc->mAlo[i], tc->xlo[i], C, t.dim, kBM);
+  // the per-step kernel's clusters (dim > 256)
+  const int64_t mt = (C + kBM - 1) / kBM;
+  tc->cm = tc->cn = mt > 1 ? 2 : 1;
+  for (int i = 0; i < 2 && ok; ++i)
+    ok = make_map(&tc->mAhi_share[i], tc->xhi[i], C, t.dim, kBM / tc->cn) &&
+         make_map(&tc->mAlo_share[i], tc->xlo[i], C, t.dim, kBM / tc->cn);
+  ok = ok && make_map(&tc->mBhi_share, tc->Phi, t.dim, t.dim, kBN / tc->cm) &&
+       make_map(&tc->mBlo_share, tc->Plo, t.dim, t.dim, kBN / tc->cm);
   if (!ok) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k_gauss_tc_step<kEpiGauss>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(kSmemBytes));
+  cudaError_t e = cudaSuccess;
+  for (int c : {1, 2}) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(gauss_step_kernel(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               static_cast<int>(kSmemBytes));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(gauss_traj_kernel(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               static_cast<int>(kTrajSmem));
+  }
+  if (e == cudaSuccess && t.dim > 256) e = gauss_traj_fits(*tc, mt, &tc->traj);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_gauss_tc_step<kEpiStore>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kSmemBytes));
@@ -810,10 +1270,25 @@ cudaError_t launch_gauss_tc_transition(const StepArgs& a, GaussTc& tc, cudaStrea
   b.xhi = tc.xhi[0];
   b.xlo = tc.xlo[0];
   const unsigned nb = static_cast<unsigned>((a.C + kWarpsPerBlock - 1) / kWarpsPerBlock);
+  const int mt = (a.C + kBM - 1) / kBM;
+  b.met = tc.traj ? tc.met : nullptr;
+  b.nmet = (mt + tc.cm - 1) / tc.cm * tc.cm;
   k_gauss_tc_begin<<<nb, 32 * kWarpsPerBlock, 0, s>>>(b);
   count_launch();
-  const dim3 grid((a.C + kBM - 1) / kBM, tc.ntn);
-  for (int l = 1; l <= a.L; ++l) {
+  if (tc.traj) {
+    TcTrajArgs st{a.C, a.D, a.L, tc.ntn, {tc.xhi[0], tc.xhi[1]}, {tc.xlo[0], tc.xlo[1]}, tc.p, tc.gL, tc.lp_part,
+                  tc.met, a.da, tc.err};
+    TrajLaunch t(tc, mt, s);
+    if (timer) timer->begin(s);
+    const cudaError_t e =
+        cudaLaunchKernelEx(&t.cfg, gauss_traj_kernel(tc.cm), tc.mAhi_share[0], tc.mAlo_share[0], tc.mAhi_share[1],
+                           tc.mAlo_share[1], tc.mBhi_share, tc.mBlo_share, st);
+    if (e != cudaSuccess) return e;
+    if (timer) timer->end(s);
+    count_launch();
+  }
+  const dim3 grid(mt, tc.ntn);
+  for (int l = 1; l <= a.L && !tc.traj; ++l) {
     TcStepArgs st{};
     st.C = a.C;
     st.D = a.D;
@@ -834,8 +1309,9 @@ cudaError_t launch_gauss_tc_transition(const StepArgs& a, GaussTc& tc, cudaStrea
     st.da = a.da;
     st.err = tc.err;
     if (timer) timer->begin(s);
-    k_gauss_tc_step<kEpiGauss><<<grid, kThreads, kSmemBytes, s>>>(tc.mAhi[in], tc.mAlo[in], tc.mBhi, tc.mBlo,
-                                                                   st);
+    const cudaError_t e = launch_clusters(gauss_step_kernel(tc.cm), grid, tc.cm, tc.cn, kSmemBytes, s,
+                                          tc.mAhi_share[in], tc.mAlo_share[in], tc.mBhi_share, tc.mBlo_share, st);
+    if (e != cudaSuccess) return e;
     if (timer) timer->end(s);
     count_launch();
   }
@@ -875,8 +1351,6 @@ namespace {
 // data rows padded to whole 64-row tiles (the residual product's columns,
 // the gradient product's K)
 int64_t lr_npad(int64_t n) { return (n + kBN - 1) / kBN * kBN; }
-// the most K-splits of the gradient product G = R X
-constexpr int kMaxSplit = 16;
 size_t a1k(size_t b) { return (b + 1023) & ~static_cast<size_t>(1023); }
 
 // Tile widths: Z = Theta X^T in 64-row tiles of the data with a 2-stage ring
@@ -888,13 +1362,22 @@ size_t a1k(size_t b) { return (b + 1023) & ~static_cast<size_t>(1023); }
 struct LrTiles {
   int bnz, bng, nrt, ndt;
 };
+// R X's tile: split-K products, bn columns (a multiple of 32)
 template <int EPI>
 void launch_tile(int bn, dim3 grid, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc,
                  const CUtensorMap& md, const TcStepArgs& st, cudaStream_t s) {
   if (bn == 64)
     k_gauss_tc_step<EPI, 64><<<grid, kThreads, Tile<64>::kSmem, s>>>(ma, mb, mc, md, st);
+  else if (bn == 96)
+    k_gauss_tc_step<EPI, 96><<<grid, kThreads, Tile<96>::kSmem, s>>>(ma, mb, mc, md, st);
   else if (bn == 128)
     k_gauss_tc_step<EPI, 128><<<grid, kThreads, Tile<128>::kSmem, s>>>(ma, mb, mc, md, st);
+  else if (bn == 160)
+    k_gauss_tc_step<EPI, 160><<<grid, kThreads, Tile<160>::kSmem, s>>>(ma, mb, mc, md, st);
+  else if (bn == 192)
+    k_gauss_tc_step<EPI, 192><<<grid, kThreads, Tile<192>::kSmem, s>>>(ma, mb, mc, md, st);
+  else if (bn == 224)
+    k_gauss_tc_step<EPI, 224><<<grid, kThreads, Tile<224>::kSmem, s>>>(ma, mb, mc, md, st);
   else
     k_gauss_tc_step<EPI, 256><<<grid, kThreads, Tile<256>::kSmem, s>>>(ma, mb, mc, md, st);
 }
@@ -902,9 +1385,12 @@ void launch_tile(int bn, dim3 grid, const CUtensorMap& ma, const CUtensorMap& mb
 LrTiles lr_tiles(int64_t npad, int ld) {
   LrTiles q{};
   q.bnz = 64;
-  q.bng = ld <= 64 ? 64 : ld <= 128 ? 128 : 256;
   q.nrt = static_cast<int>((npad + q.bnz - 1) / q.bnz);
-  q.ndt = (ld + q.bng - 1) / q.bng;
+  // the dims in tiles of up to 256, as even as multiples of 32 allow: 301 dims
+  // take two tiles of 160, not 256 + 48 (each tile's width costs its loads of X
+  // and its MMAs; 47.7 us -> 32.5 us at 8000 rows, 700 chains)
+  q.ndt = (ld + 255) / 256;
+  q.bng = std::max(64, ((ld + q.ndt - 1) / q.ndt + 31) / 32 * 32);
   return q;
 }
 
@@ -990,15 +1476,17 @@ cudaError_t logreg_gemm_setup(LogregGemm* g, const hmc_target& t, int64_t C, voi
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_lr_z_persist, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kZpSmem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gauss_tc_step<kEpiStore, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(Tile<64>::kSmem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gauss_tc_step<kEpiStore, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(Tile<128>::kSmem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gauss_tc_step<kEpiStore, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(Tile<256>::kSmem));
+  auto tile_attr = [&](StepKernel k, size_t smem) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  };
+  tile_attr(k_gauss_tc_step<kEpiStore, 64>, Tile<64>::kSmem);
+  tile_attr(k_gauss_tc_step<kEpiStore, 96>, Tile<96>::kSmem);
+  tile_attr(k_gauss_tc_step<kEpiStore, 128>, Tile<128>::kSmem);
+  tile_attr(k_gauss_tc_step<kEpiStore, 160>, Tile<160>::kSmem);
+  tile_attr(k_gauss_tc_step<kEpiStore, 192>, Tile<192>::kSmem);
+  tile_attr(k_gauss_tc_step<kEpiStore, 224>, Tile<224>::kSmem);
+  tile_attr(k_gauss_tc_step<kEpiStore, 256>, Tile<256>::kSmem);
   if (e == cudaSuccess)
     e = launch_lr_prepare(static_cast<int>(t.n_data), static_cast<int>(npad), t.dim, ld, t.X, t.y, g->Xhi,
                           g->Xlo, g->XThi, g->XTlo, g->ypad, s);
@@ -1085,7 +1573,9 @@ cudaError_t launch_logreg_gemm_transition(const StepArgs& a, LogregGemm& g, cuda
       launch_tile<kEpiStore>(g.bng, dim3(mt, g.ndt, S), g.mRhi, g.mRlo, g.mXThi, g.mXTlo, st, s);
       LrSumArgs u{a.C, a.D, g.ld, S, last ? 1 : 0, g.nrt, g.ntot, g.part, g.xhi[in], g.xlo[in],
                   g.xhi[out], g.xlo[out], g.p, g.gL, g.lp_part, a.da};
-      k_lr_gemm_update<<<nb, 32 * kWarpsPerBlock, 0, s>>>(u);
+      const int64_t n4 = static_cast<int64_t>(a.C) * (g.ld / 4);
+      if (last) k_lr_gemm_update<<<nb, 32 * kWarpsPerBlock, 0, s>>>(u);
+      else k_lr_gemm_update_middle<<<static_cast<unsigned>((n4 + 255) / 256), 256, 0, s>>>(u);
       count_launch();
     }
     if (timer) timer->end(s);

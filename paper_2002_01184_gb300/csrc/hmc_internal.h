@@ -224,6 +224,11 @@ namespace hmc {
 // Device buffers and TMA descriptors of the tensor-core Gaussian path.
 struct GaussTc {
   CUtensorMap mAhi[2], mAlo[2], mBhi, mBlo;
+  // the per-step kernel's clusters of cm x cn tiles: a CTA's share of the rows
+  CUtensorMap mAhi_share[2], mAlo_share[2], mBhi_share, mBlo_share;
+  int cm = 1, cn = 1;
+  bool traj = false;         // all steps of a trajectory in one launch (every tile resident)
+  unsigned* met = nullptr;   // ... and its counters, one per 128 chains
   CUtensorMap mPhi128, mPlo128;  // P head / remainder, 32 x 128 boxes
   float* Phi = nullptr;      // tf32 head / remainder of P
   float* Plo = nullptr;

@@ -99,3 +99,28 @@ def test_merged_steps_equal_one_launch_per_operation(C, D, L):
         out.append((x, s, e, a))
     for u, v in zip(*out):
         assert torch.equal(u, v)
+
+
+# one launch per trajectory (clusters of 2 x 2 tiles, a lone chain block, a
+# chain or column block past the edge) against one launch per step, which the
+# 4300 chains' tiles need: a chain's result does not depend on the others
+@pytest.mark.parametrize("D,L", [(260, 1), (260, 5), (320, 4), (512, 3)])
+def test_trajectory_launch_equals_step_launches(D, L):
+    gen = torch.Generator(device="cuda").manual_seed(D)
+    A = torch.randn(D, D, device="cuda", generator=gen, dtype=torch.float64)
+    P = (A @ A.T / D + 0.1 * torch.eye(D, device="cuda", dtype=torch.float64)).float().contiguous()
+    x0 = torch.randn(4300, D, device="cuda", generator=gen)
+    out = []
+    for C in (4300, 100, 300, 513):
+        cfg = H.make_config(L, 0.05, seed=9)
+        ctx = H.hmc_create(H.make_target("corr_gauss", D, P=P), C, cfg)
+        x, s = x0[:C].clone(), torch.empty(3, C, D, device="cuda")
+        e, a = torch.empty(3, device="cuda"), torch.empty(3, C, dtype=torch.uint8, device="cuda")
+        H.hmc_sample_chain(ctx, x, 1, 3, s, e, a)
+        H.hmc_synchronize(ctx)
+        H.hmc_destroy(ctx)
+        out.append((x, s, a))
+    assert 0 < out[0][2].float().mean().item()
+    for x, s, a in out[1:]:
+        C = x.shape[0]
+        assert torch.equal(x, out[0][0][:C]) and torch.equal(s, out[0][1][:, :C]) and torch.equal(a, out[0][2][:, :C])
