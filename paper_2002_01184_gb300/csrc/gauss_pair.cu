@@ -1214,6 +1214,398 @@ k_gauss_pair(const __grid_constant__ CUtensorMap mPhi, const __grid_constant__ C
   }
 }
 
+// The same chains for dim <= 128, one CTA each 32 chains (half a pair), without
+// a peer: a pair's second CTA would own dims past 128 alone, yet every step
+// crossed the pair and back.  P's 128 rows (head and remainder of at most four
+// K-chunks) stay in tensor memory, and since a thread owns one dim of 16 chains
+// (not of 32), their current positions, cached gradients and next momenta all
+// stay in registers; the streaming driver's running moments in shared memory.  A step is
+// N = 64 and N = 32 products of M = 128, an accumulator read, 16 elements'
+// updates and one barrier each way.  Products, order of every sum and decisions
+// are the pair's: rows 0-31 of a pair add P_lo x_hi to their P_hi x_lo column,
+// rows 32-63 to their P_hi x_hi column, so odd CTAs do the latter.
+// Measured, 16 steps, per transition: 1000 chains x 100 dims 42.5 -> 26.1 us, 4096
+// x 128 42.8 -> 26.1, 4096 x 64 35.9 -> 19.9, 64 x 32 30.2 -> 16.7.  What bounds it:
+// a step's dependent chain (0.6-1.0 us of MMAs at their issue rate, the commit,
+// the accumulator read, the tile's stores and their proxy fence).
+constexpr int kOneAccCols = 64;                    // head columns 0-31, remainder columns 32-63
+constexpr int kOneColP = kOneAccCols;              // P head chunk c at kOneColP + 32 c, remainder 128 further
+constexpr uint32_t kOneSmemUsed = 4 * kBChunk + 3 * 16 * 256 * 4 + 1024;
+constexpr size_t kOneSmem = 120 * 1024;            // one CTA per SM: it allocates all of tensor memory
+static_assert(kOneSmemUsed <= kOneSmem, "shared memory");
+static_assert(kOneColP + 2 * 128 <= static_cast<int>(kTmemCols), "tensor-memory columns");
+
+template <bool MOMENTS>
+__global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
+  const StepArgs& a = fa.s;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* Bt = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  __shared__ uint64_t acc_full[1], own_full[1];
+  __shared__ uint32_t tmem_slot[4];
+  __shared__ float red[2][4][kHalf], kin_s[2][4][kHalf], lu_s[2][kHalf];
+  __shared__ DAState da_s;
+  __shared__ DACoef coef_s;
+  __shared__ unsigned long long psum_s;
+  __shared__ int abort_s;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int C = a.C, D = a.D, L = a.L, T = fa.T;
+  const int nk = (D + 31) >> 5;
+  const int c0 = static_cast<int>(blockIdx.x) * kHalf;
+  const bool persistent = T > 1;
+  if (threadIdx.x == 0) {
+    ptx::mbar_init(acc_full, 1);
+    ptx::mbar_init(own_full, 256);
+    ptx::fence_mbar_init();
+    if (persistent) da_s = *a.da;
+    abort_s = 0;
+  }
+  if (warp == 0) {
+    ptx::tmem_alloc(tmem_slot, kTmemCols);
+    ptx::tmem_relinquish();
+  }
+  // dims >= D and chains >= C of the tile are never written
+  for (uint32_t i = threadIdx.x; i < 4 * kBChunk / 16; i += kThreads)
+    reinterpret_cast<uint4*>(Bt)[i] = make_uint4(0u, 0u, 0u, 0u);
+  proxy_fence_cta();
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 1) {
+    if (lane == 0) {
+      // ---- MMA issuer
+      constexpr uint32_t idesc_wide = ptx::idesc_tf32(128, 2 * kHalf);   // head + remainder rows
+      constexpr uint32_t idesc_head = ptx::idesc_tf32(128, kHalf);       // head rows only
+      const uint32_t lo_product = tmem + (blockIdx.x & 1u ? 0u : static_cast<uint32_t>(kHalf));
+      for (int s = 0; s < T * L; ++s) {
+        if (!ptx::mbar_wait(own_full, s & 1)) {
+          atomicCAS(fa.err, 0, 2);
+          break;
+        }
+        ptx::tc_fence_after();
+        for (int kc = 0; kc < nk; ++kc) {
+          const uint32_t b = ptx::smem_u32(Bt + kc * kBChunk);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint64_t db = ptx::sw128_kmajor_desc(b + 32 * j);
+            const uint32_t ahi = tmem + kOneColP + 32 * kc + 8 * j;
+            ptx::mma_tf32_tmem_a(tmem, ahi, db, idesc_wide, (kc | j) != 0 ? 1u : 0u);
+            ptx::mma_tf32_tmem_a(lo_product, ahi + 128, db, idesc_head, 1u);
+          }
+        }
+        ptx::mma_commit(acc_full);
+      }
+    }
+  } else if (warp >= 2) {
+    // ---- epilogue: thread (quarter, lane) of dim d, chains c0 + 16 sub + i
+    const int ew = warp - 2, sub = ew >> 2, quarter = warp & 3;
+    const int d = quarter * 32 + lane;
+    const int nv = d < D ? max(0, min(16, C - (c0 + 16 * sub))) : 0;
+    auto elem = [&](int i) { return static_cast<int64_t>(c0 + 16 * sub + i) * D + d; };
+    const uint32_t hi0 = ptx::smem_u32(Bt) + static_cast<uint32_t>((d >> 5) * kBChunk + (d & 3) * 4);
+    uint32_t sw[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) sw[r] = r * kRowBytes + ((((lane >> 2) ^ r) & 7) << 4);
+    auto store_x = [&](int i, float xi) {
+      if (i < nv) {
+        float hi, lo;
+        split_tf32(xi, hi, lo);
+        const uint32_t a0 = hi0 + (2 * sub + (i >> 3)) * 1024 + sw[i & 7];
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(a0), "f"(hi) : "memory");
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(a0 + kLoOff), "f"(lo) : "memory");
+      }
+    };
+    auto publish = [&]() {
+      proxy_fence_cta();          // generic stores -> async proxy (MMA)
+      ptx::tc_fence_before();     // this thread's accumulator reads precede the next MMA
+      ptx::mbar_arrive_local(own_full);
+    };
+    const uint32_t acc_col = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(16 * sub);
+    auto load_acc = [&](float (&acc)[16]) {
+      ptx::tmem_ld8x2_sum(acc_col, acc_col + 32, acc);
+      ptx::tmem_ld8x2_sum(acc_col + 8, acc_col + 40, acc + 8);
+    };
+    bool ok = true;
+    auto wait_acc = [&](int s) {
+      if (!ptx::mbar_wait(acc_full, s & 1)) {
+        atomicCAS(fa.err, 0, 4);
+        ok = false;
+      }
+      ptx::tc_fence_after();
+    };
+    // |p0|^2 of the warp's 16 chains over its 32 dims, in the pair's order:
+    // the butterfly's first step in full, then halving
+    auto kinetic = [&](const float (&z)[16], uint32_t tn) {
+      float v[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] = z[i] * z[i];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], 16);
+#pragma unroll
+      for (int w = 8; w >= 1; w >>= 1) {
+        const bool upper = (lane & w) != 0;
+#pragma unroll
+        for (int k = 0; k < w; ++k) {
+          const float send = upper ? v[k] : v[k + w];
+          const float keep = upper ? v[k + w] : v[k];
+          v[k] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+        }
+      }
+      if (lane < 16) kin_s[tn & 1u][quarter][16 * sub + lane] = v[0];
+    };
+    // momenta of slots 4 g .. 4 g + 3 at transition tn
+    auto draw = [&](float (&z)[16], int g0, int g1, uint32_t tn) {
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+        if (g >= g0 && g < g1) {
+          float v[4] = {0.f, 0.f, 0.f, 0.f};
+          draw_quad(a.seed, d, lane, static_cast<uint32_t>(c0 + 16 * sub) + a.chain_offset, 0u, nv, 0, g, tn, v);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) z[4 * g + e] = v[e];
+        }
+    };
+    const int per_wait = (4 + L - 1) / L;
+
+    // P into tensor memory from the pair kernel's image (its first CTA's rows):
+    // the two warps of a quarter take the head and the remainder
+    for (int kc = 0; kc < nk; ++kc) {
+#pragma unroll
+      for (int q16 = 0; q16 < 2; ++q16) {
+        float v[16];
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4) {
+          const float4 u = *reinterpret_cast<const float4*>(
+              fa.Ptm + image_index(0, sub == 0 ? kc : kChunks + kc, q16, quarter, q4, lane));
+          v[4 * q4] = u.x; v[4 * q4 + 1] = u.y; v[4 * q4 + 2] = u.z; v[4 * q4 + 3] = u.w;
+        }
+        ptx::tmem_st16(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + kOneColP + 128 * sub + 32 * kc + 16 * q16,
+                       v);
+      }
+    }
+    ptx::tmem_wait_st();
+
+    float xc[16], gc[16], z[16], zn[16];
+    // running mean, m2 and batch sum of element i (in registers they spilled)
+    float* mom = reinterpret_cast<float*>(Bt + 4 * kBChunk) + ew * 32 + lane;
+    auto moment = [&](int k, int i) -> float& { return mom[(16 * k + i) * 256]; };
+    const bool batches = MOMENTS && a.w.bsize > 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      xc[i] = i < nv ? a.x[elem(i)] : 0.f;
+      gc[i] = i < nv ? a.g[elem(i)] : 0.f;
+      zn[i] = 0.f;
+      if (MOMENTS) {
+        moment(0, i) = i < nv ? a.w.mean[elem(i)] : 0.f;
+        moment(1, i) = i < nv ? a.w.m2[elem(i)] : 0.f;
+        moment(2, i) = batches && i < nv ? a.w.bsum[elem(i)] : 0.f;
+      }
+    }
+    draw(z, 0, 4, a.t);
+    kinetic(z, a.t);
+    // lane c of every warp decides chain c0 + c (the same inputs, the same answer)
+    const int chain = c0 + lane;
+    float lpc = chain < C ? a.lp[chain] : 0.f;
+
+    int nbar = 0;
+    for (int j = 0; j < T; ++j) {
+      const uint32_t t = a.t + static_cast<uint32_t>(j);
+      const bool more = j + 1 < T;
+      const float eps = persistent ? da_s.eps : a.da->eps;
+      float p[16], x[16], acc[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        p[i] = fmaf(0.5f * eps, gc[i], z[i]);
+        x[i] = fmaf(eps, p[i], xc[i]);
+        store_x(i, x[i]);
+      }
+      publish();
+      // the accept test's log u, off the critical path
+      if (warp == 2 && chain < C)
+        lu_s[j & 1][lane] = accept_log_uniform(a.seed, static_cast<uint32_t>(chain) + a.chain_offset, t);
+      const int s0 = j * L;
+      for (int l = 1; l < L; ++l) {
+        if (more) draw(zn, (l - 1) * per_wait, l * per_wait, t + 1);
+        wait_acc(s0 + l - 1);
+        load_acc(acc);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          p[i] = fmaf(-eps, acc[i], p[i]);
+          x[i] = fmaf(eps, p[i], x[i]);
+          store_x(i, x[i]);
+        }
+        publish();
+      }
+      if (more) {
+        draw(zn, (L - 1) * per_wait, 4, t + 1);
+        kinetic(zn, t + 1);
+      }
+      wait_acc(s0 + L - 1);
+      load_acc(acc);
+      {
+        // <x, g> and |p|^2 partials: lanes 0-15 end with the former of the
+        // warp's 16 chains, lanes 16-31 with the latter
+        float v[32];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          p[i] = fmaf(-0.5f * eps, acc[i], p[i]);
+          v[i] = i < nv ? -x[i] * acc[i] : 0.f;
+          v[16 + i] = i < nv ? p[i] * p[i] : 0.f;
+        }
+        red[lane >> 4][quarter][16 * sub + (lane & 15)] = transpose_reduce32(v, lane);
+      }
+      if (!ok) abort_s = 1;
+      epi_barrier();
+      const bool stop = *reinterpret_cast<volatile int*>(&abort_s) != 0;
+      const long long t_full = a.t_full + j;
+      const long long k_out = t_full - fa.keep_from;
+      int take = 0;
+      float prob = 0.f, la = 0.f;
+      if (chain < C) {
+        float xg = 0.f, pp = 0.f, k0 = 0.f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          xg += red[0][q][lane];
+          pp += red[1][q][lane];
+          k0 += kin_s[t & 1u][q][lane];
+        }
+        const float kin0 = 0.5f * k0, lp1 = 0.5f * xg;
+        la = (-lpc + kin0) - (-lp1 + 0.5f * pp);
+        if (!isfinite(la)) la = -INFINITY;
+        take = lu_s[j & 1][lane] < la;
+        prob = accept_prob(la);
+        if (take) lpc = lp1;
+      }
+      const uint32_t accw = __ballot_sync(0xffffffffu, take != 0) >> (16 * sub);
+      if (stop) break;
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if ((accw >> i) & 1u) {
+          xc[i] = x[i];
+          gc[i] = -acc[i];
+        }
+      if (k_out >= 0 && fa.samples) {
+        float* samp = fa.samples + k_out * static_cast<int64_t>(C) * D;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          if (i < nv) samp[elem(i)] = xc[i];
+      }
+      if (warp == 2 && chain < C) {
+        if (!more) {
+          a.lp[chain] = lpc;
+          a.is_accepted[chain] = static_cast<uint8_t>(take);
+          a.log_accept[chain] = la;
+        }
+        if (k_out >= 0 && fa.trace_acc) fa.trace_acc[k_out * C + chain] = static_cast<uint8_t>(take);
+        if (chain == 0 && k_out >= 0 && fa.trace_eps) fa.trace_eps[k_out] = eps;
+      }
+      if (MOMENTS && k_out >= 0) {
+        const WelfordCoef wq = welford_coef(k_out, a.w.bsize);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float xv = xc[i];
+          float m1 = xv, s1 = 0.f;
+          if (k_out > 0) {
+            const float m0 = moment(0, i);
+            const float delta = xv - m0;
+            m1 = fmaf(delta, wq.inv, m0);
+            s1 = fmaf(delta, xv - m1, moment(1, i));
+          }
+          moment(0, i) = m1;
+          moment(1, i) = s1;
+          if (batches) moment(2, i) = wq.pos == 0 ? xv : moment(2, i) + xv;
+        }
+        if (batches && wq.closes) {
+          // eight elements' loads before their stores (which may alias, as far
+          // as the compiler knows)
+#pragma unroll
+          for (int h = 0; h < 16; h += 8) {
+            float b0[8], q0[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const bool have = wq.batch > 0 && h + i < nv;
+              b0[i] = have ? a.w.bmean[elem(h + i)] : 0.f;
+              q0[i] = have ? a.w.bm2[elem(h + i)] : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if (h + i < nv) {
+                const float bm = __fmul_rn(moment(2, h + i), wq.inv_b);   // (not contracted into the differences)
+                float bn = bm, qn = 0.f;
+                if (wq.batch > 0) {
+                  const float delta = bm - b0[i];
+                  bn = fmaf(delta, wq.inv_j, b0[i]);
+                  qn = fmaf(delta, bm - bn, q0[i]);
+                }
+                a.w.bmean[elem(h + i)] = bn;
+                a.w.bm2[elem(h + i)] = qn;
+              }
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 16; ++i) z[i] = zn[i];
+      // dual averaging, as in the pair launch (whose comments explain it)
+      if (persistent) {
+        const bool adapts = da_s.adapt && t_full < da_s.num_adapt;
+        if (adapts || !more) {
+          ++nbar;
+          if (warp == 2) {
+            const unsigned long long v = warp_sum_u64(prob_fixed(prob, fa.stat_hi_scale));
+            if (lane == 0) {
+              unsigned long long total = 0ull;
+              if (!grid_barrier_sum(fa.stat, static_cast<unsigned>(nbar), v, fa.grid_wait_ns, fa.unreachable_gen,
+                                    &total)) {
+                atomicCAS(fa.err, 0, 7);
+                abort_s = 1;
+              } else {
+                psum_s = total;
+              }
+            }
+          } else if (warp == 3 && lane == 0) {
+            coef_s = da_prepare(&da_s, t_full);
+          }
+          epi_barrier();
+          if (warp == 2 && lane == 0 && *reinterpret_cast<volatile int*>(&abort_s) == 0)
+            da_apply(&da_s, coef_s, stat_mean(psum_s, fa.stat_scale), t_full);
+          epi_barrier();
+          if (*reinterpret_cast<volatile int*>(&abort_s)) break;
+        }
+      } else if (warp == 2) {
+        const unsigned long long v = warp_sum_u64(prob_fixed(prob, fa.stat_hi_scale));
+        if (lane == 0) psum_s = v;
+      }
+    }
+    const bool fine = *reinterpret_cast<volatile int*>(&abort_s) == 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (fine && i < nv) {
+        a.x[elem(i)] = xc[i];
+        a.g[elem(i)] = gc[i];
+        if (MOMENTS) {
+          a.w.mean[elem(i)] = moment(0, i);
+          a.w.m2[elem(i)] = moment(1, i);
+          if (batches) a.w.bsum[elem(i)] = moment(2, i);
+        }
+      }
+    if (persistent && blockIdx.x == 0 && threadIdx.x == 64 && fine) *a.da = da_s;
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, kTmemCols);
+  }
+  if (!persistent && threadIdx.x == 64) {
+    // one transition: the CTA that arrives last applies the update
+    atomicAdd(fa.stat, psum_s);
+    if (atom_add_acq_rel(fa.stat + 1, 1ull) + 1ull == gridDim.x)
+      da_update(a.da, stat_mean(ld_acquire_u64(fa.stat), fa.stat_scale), a.t_full);
+  }
+}
+
 }  // namespace
 
 // Test support: the grid barrier's wait limit and an unreachable generation
@@ -1241,6 +1633,12 @@ cudaError_t launch_gauss_pair_image(const float* Phi, const float* Plo, int D, f
 cudaError_t gauss_pair_setup() {
   cudaError_t e = cudaFuncSetAttribute(k_gauss_pair<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(kSmem));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_gauss_one<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kOneSmem));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_gauss_one<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kOneSmem));
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_gauss_pair<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(kSmem));
@@ -1294,6 +1692,25 @@ cudaError_t launch_gauss_pair_transitions(const StepArgs& a, GaussTc& tc, int T,
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg = {};
+  if (a.D <= 128 && !a.betas) {
+    // half a pair per CTA (C <= 64 x the pairs that run at once is C <= 32 x the
+    // SMs, so T > 1 finds its CTAs resident here too)
+    cfg.gridDim = dim3(static_cast<unsigned>((a.C + kHalf - 1) / kHalf));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kOneSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute coop[1];
+    coop[0].id = cudaLaunchAttributeCooperative;
+    coop[0].val.cooperative = 1;
+    cfg.attrs = coop;
+    cfg.numAttrs = T > 1 ? 1 : 0;
+    if (timer) timer->begin(s);
+    const cudaError_t e = a.w.mean && nkeep > 0 ? cudaLaunchKernelEx(&cfg, k_gauss_one<true>, fa)
+                                                : cudaLaunchKernelEx(&cfg, k_gauss_one<false>, fa);
+    if (timer) timer->end(s);
+    count_launch();
+    return e;
+  }
   cfg.gridDim = dim3(gauss_pair_grid(a.C));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = kSmem;
