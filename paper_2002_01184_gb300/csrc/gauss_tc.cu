@@ -1211,6 +1211,8 @@ cudaError_t gauss_tc_setup(GaussTc* tc, const hmc_target& t, int64_t C, void* ws
   tc->met = t.dim > 256 ? reinterpret_cast<unsigned*>(take(((static_cast<size_t>(C) + kBM - 1) / kBM + 1) * 4)) : nullptr;
   bool ok = make_map(&tc->mBhi, tc->Phi, t.dim, t.dim, kBN) &&
             make_map(&tc->mBlo, tc->Plo, t.dim, t.dim, kBN) &&
+            make_map(&tc->mAhi_blk, tc->xhi[0], C, t.dim, nuts_cluster_chains(t.dim)) &&
+            make_map(&tc->mAlo_blk, tc->xlo[0], C, t.dim, nuts_cluster_chains(t.dim)) &&
             make_map(&tc->mPhi128, tc->Phi, t.dim, t.dim, 128) &&
             make_map(&tc->mPlo128, tc->Plo, t.dim, t.dim, 128);
   for (int i = 0; i < 2 && ok; ++i)

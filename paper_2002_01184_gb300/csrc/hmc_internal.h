@@ -229,6 +229,7 @@ struct GaussTc {
   int cm = 1, cn = 1;
   bool traj = false;         // all steps of a trajectory in one launch (every tile resident)
   unsigned* met = nullptr;   // ... and its counters, one per 128 chains
+  CUtensorMap mAhi_blk, mAlo_blk;   // positions xhi[0], xlo[0] in boxes of a NUTS cluster's chains
   CUtensorMap mPhi128, mPlo128;  // P head / remainder, 32 x 128 boxes
   float* Phi = nullptr;      // tf32 head / remainder of P
   float* Plo = nullptr;
@@ -300,6 +301,8 @@ cudaError_t launch_logreg_gemm_products(LogregGemm& g, int C, int D, const DASta
                                         const uint8_t* active, int* splits, cudaStream_t s);
 
 bool gauss_tc_supported(const hmc_target& t);
+// Chains of a cluster of the NUTS loop (dim <= 256): 32 per 64 output dims
+inline int nuts_cluster_chains(int D) { return 32 * ((D + 63) / 64 < 4 ? (D + 63) / 64 : 4); }
 // Tensor map of [K x C x D] float32 samples, box 128 dims x 64 chains x 1
 // (false: no encoder, D % 4 != 0 or a base without 16-byte alignment).
 bool make_sample_map(CUtensorMap* map, const float* base, int D, int64_t C, int64_t K);
@@ -396,7 +399,8 @@ struct NutsDense {
   void* chains = nullptr;         // per-chain tree state [C]
   uint8_t* active = nullptr;      // [C] chains still building their trees
   unsigned* ctr = nullptr;        // [8] leaf-loop counters: [0-2] the graph loop's, [3] the
-                                  // persistent loop's grid barrier, [4-5] its chains left
+                                  // persistent loop's grid barrier, [4-5] its chains left,
+                                  // [6] the cluster launch's longest loop
   int* err = nullptr;             // the products' flag; 2: the leaf loop ran past its bound
   float* scratch = nullptr;       // [C][kNutsSlots][ld]
   unsigned long long* leaves = nullptr;   // leapfrog steps of the chains (useful gradients)

@@ -74,7 +74,8 @@ struct NdArgs {
   float* scratch;         // [C][kNutsSlots][ld]
   NdChain* st;
   uint8_t* active;
-  unsigned* ctr;          // [0] chains left, [1] blocks arrived, [2] iterations of this transition
+  unsigned* ctr;          // [0] chains left, [1] blocks arrived, [2] iterations of this transition,
+                          // [6] the cluster launch's longest loop
   int* err;
   unsigned long long* leaves;
   unsigned long long* iters;
@@ -429,6 +430,10 @@ __global__ void __launch_bounds__(32 * kNdWarps) k_nuts_dense_finish(NdArgs na) 
   const int c = blockIdx.x * kNdWarps + (threadIdx.x >> 5);
   const bool has = c < a.C;
   const float eps = a.da->eps;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && na.ctr[6]) {
+    *na.iters += na.ctr[6];        // the cluster launch's longest loop
+    na.ctr[6] = 0u;
+  }
   float prob = 0.f;
   unsigned n_a = 0u;
   if (has) {
@@ -498,7 +503,6 @@ __device__ __forceinline__ bool pl_grid_barrier(unsigned* counter, unsigned gen)
   return true;
 }
 
-template <int NB>
 __global__ void __launch_bounds__(kPlThreads, 1)
 k_nuts_gauss_loop(const __grid_constant__ CUtensorMap mAhi, const __grid_constant__ CUtensorMap mAlo,
                   const __grid_constant__ CUtensorMap mBhi, const __grid_constant__ CUtensorMap mBlo,
@@ -656,7 +660,7 @@ k_nuts_gauss_loop(const __grid_constant__ CUtensorMap mAhi, const __grid_constan
     // ---- one leaf of every active chain
     int mine = 0;
     for (int c = gw; c < C; c += gwarps)
-      if (na.st[c].active && nuts_leaf<kModeGauss, NB>(na, c, lane)) ++mine;
+      if (na.st[c].active && nuts_leaf<kModeGauss, 4>(na, c, lane)) ++mine;
     // positions written for the next products' TMA loads (another proxy)
     asm volatile("fence.proxy.async.global;" ::: "memory");
     if (lane == 0 && mine) atomicAdd(&left[it & 1], static_cast<unsigned>(mine));
@@ -687,6 +691,189 @@ k_nuts_gauss_loop(const __grid_constant__ CUtensorMap mAhi, const __grid_constan
   }
 }
 
+// ---- the same loop per chain block (dim <= 256)
+//
+// A chain's next products need its own row of positions and nothing of the
+// other chains, so the loop needs no meeting of the whole grid: a cluster of
+// ceil(D / 64) CTAs, one per 64 output dims, owns 32 chains per CTA and builds
+// their trees to the end, with hardware cluster barriers where the grid loop
+// has barriers through memory, and stops when its own chains are done.  Each
+// CTA keeps its 64 rows of P (tf32 head and remainder) in shared memory for
+// the launch and loads the block's positions by TMA (each its own: sharing the
+// loads by multicast put a trip between CTAs into every refill of the ring,
+// and gained nothing: 16.0 us an iteration).  Every warp has one chain.  Clusters are
+// independent, so the launch need not be resident as a whole.
+//
+// Measured, per leaf iteration: 4096 chains x 256 dims 18.7 -> 15.6 us, 4096 x 64
+// 10.9 -> 5.9, 1000 x 100 11.5 -> 8.9, 64 x 256 14.1 -> 12.1.  What bounds it now, of
+// 27000 cycles at 4096 x 256: the products (9600; a 128 x 64 x 256 tile moves 0.8 MB
+// through shared memory, 6700 at least), the accumulator's way to the leaves (4300),
+// the leaf's dependent loads (7300; 4300 with the chip to itself), the proxy fence
+// that waits for its stores (3000) and the cluster barrier (1600).
+constexpr int kClWarps = 32;                          // 0 TMA, 1 MMA, 2-17 epilogue; all: a chain's leaf each
+constexpr int kClThreads = 32 * kClWarps;
+constexpr int kClStages = 3;
+constexpr uint32_t kClA = 128 * kPlBK * 4;            // 128 rows x 32 dims (head or remainder)
+constexpr uint32_t kClB = kPlBN * kPlBK * 4;          // 64 rows of P x 32 dims
+constexpr int kClMaxChunks = 256 / kPlBK;
+constexpr size_t kClSmem = kClMaxChunks * 2 * kClB + kClStages * 2 * kClA + 1024 + 256;
+static_assert(kClSmem <= 227 * 1024, "shared memory");
+
+template <int NB>
+__global__ void __launch_bounds__(kClThreads, 1)
+k_nuts_gauss_cluster(const __grid_constant__ CUtensorMap mAhi, const __grid_constant__ CUtensorMap mAlo,
+                     const __grid_constant__ CUtensorMap mBhi, const __grid_constant__ CUtensorMap mBlo, NdArgs na,
+                     int ctas) {
+  const StepArgs& a = na.s;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint8_t* ring = smem + kClMaxChunks * 2 * kClB;
+  uint64_t* full = reinterpret_cast<uint64_t*>(ring + kClStages * 2 * kClA);
+  uint64_t* empty = full + kClStages;
+  uint64_t* acc_full = empty + kClStages;
+  uint64_t* p_full = acc_full + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(p_full + 1);
+  __shared__ int left_s[2][8];      // chains left per CTA of the cluster, by iteration parity
+  __shared__ int bad_s;             // a bounded wait gave up
+  constexpr int kBad = 1 << 20;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = static_cast<int>(ptx::cluster_rank());
+  const int slices = min(ctas, 4);                 // 32-chain shares of the cluster's chain block
+  const int C = a.C, D = a.D, rows = 32 * slices;
+  const int m0 = static_cast<int>(blockIdx.x) / ctas * rows, n0 = rank * kPlBN;
+  const int nk = (D + kPlBK - 1) / kPlBK;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kClStages; ++i) {
+      ptx::mbar_init(&full[i], 1);
+      ptx::mbar_init(&empty[i], 1);
+    }
+    ptx::mbar_init(acc_full, 1);
+    ptx::mbar_init(p_full, 1);
+    ptx::fence_mbar_init();
+    bad_s = 0;
+  }
+  if (warp == 0) {
+    ptx::tmem_alloc(tmem_slot, kPlBN);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncwarp();
+  ptx::cluster_sync();
+  ptx::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  if (threadIdx.x == 0) {
+    // this CTA's rows of P, once
+    ptx::mbar_arrive_expect_tx(p_full, static_cast<uint32_t>(nk) * 2 * kClB);
+    for (int kc = 0; kc < nk; ++kc) {
+      ptx::tma_load_2d(smem + kc * 2 * kClB, &mBhi, p_full, kc * kPlBK, n0);
+      ptx::tma_load_2d(smem + kc * 2 * kClB + kClB, &mBlo, p_full, kc * kPlBK, n0);
+    }
+  }
+  // pipeline positions, kept by the thread of each role across iterations
+  int pit = 0, mit = 0, it = 0;
+  for (;; ++it) {
+    if (warp == 0 && lane == 0) {
+      // ---- TMA producer: the block's positions
+      for (int kc = 0; kc < nk; ++kc, ++pit) {
+        const int st = pit % kClStages, round = pit / kClStages;
+        if (pit >= kClStages && !ptx::mbar_wait(&empty[st], (round - 1) & 1)) {
+          atomicExch(na.err, 1);
+          bad_s = 1;
+          break;
+        }
+        uint8_t* sp = ring + st * 2 * kClA;
+        ptx::mbar_arrive_expect_tx(&full[st], static_cast<uint32_t>(rows) * 128 * 2);
+        ptx::tma_load_2d(sp, &mAhi, &full[st], kc * kPlBK, m0);
+        ptx::tma_load_2d(sp + kClA, &mAlo, &full[st], kc * kPlBK, m0);
+      }
+    } else if (warp == 1 && lane == 0) {
+      // ---- MMA issuer: 3xTF32, A_lo B_hi + A_hi B_lo + A_hi B_hi (rows past
+      // the block's chains hold whatever was there: their products are unused)
+      constexpr uint32_t idesc = ptx::idesc_tf32(128, kPlBN);
+      bool ok = it > 0 || ptx::mbar_wait(p_full, 0);
+      for (int kc = 0; kc < nk && ok; ++kc, ++mit) {
+        const int st = mit % kClStages, round = mit / kClStages;
+        if (!ptx::mbar_wait(&full[st], round & 1)) {
+          ok = false;
+          break;
+        }
+        ptx::tc_fence_after();
+        const uint32_t sa = ptx::smem_u32(ring + st * 2 * kClA), sb = ptx::smem_u32(smem + kc * 2 * kClB);
+#pragma unroll
+        for (int j = 0; j < kPlBK / 8; ++j) {
+          const uint64_t a_hi = ptx::sw128_kmajor_desc(sa + 32 * j);
+          const uint64_t a_lo = ptx::sw128_kmajor_desc(sa + kClA + 32 * j);
+          const uint64_t b_hi = ptx::sw128_kmajor_desc(sb + 32 * j);
+          const uint64_t b_lo = ptx::sw128_kmajor_desc(sb + kClB + 32 * j);
+          ptx::mma_tf32(tmem, a_lo, b_hi, idesc, (kc | j) != 0 ? 1u : 0u);
+          ptx::mma_tf32(tmem, a_hi, b_lo, idesc, 1u);
+          ptx::mma_tf32(tmem, a_hi, b_hi, idesc, 1u);
+        }
+        ptx::mma_commit(&empty[st]);
+      }
+      if (ok) {
+        ptx::mma_commit(acc_full);
+      } else {
+        atomicExch(na.err, 1);
+        bad_s = 1;
+      }
+    } else if (warp >= 2 && warp < 18) {
+      // ---- epilogue: warp (quarter q, column group g) stores X P for rows
+      // 32 q .. 32 q + 31 of the block, columns 16 g .. 16 g + 15, a row per lane
+      const int quarter = warp & 3, cg = (warp - 2) >> 2;
+      if (!ptx::mbar_wait(acc_full, it & 1)) {
+        atomicExch(na.err, 1);
+        bad_s = 1;
+      }
+      ptx::tc_fence_after();
+      float v[16];
+      ptx::tmem_ld16(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + 16 * cg, v);
+      ptx::tc_fence_before();
+      const int m = m0 + quarter * 32 + lane, n = n0 + 16 * cg;
+      if (quarter < slices && m < C) {
+        // D % 4 == 0 on this path: a float4 lies wholly inside or past the row
+        float4* out = reinterpret_cast<float4*>(const_cast<float*>(na.part) + static_cast<int64_t>(m) * D + n);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (n + 4 * q < D) out[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      }
+    }
+    __syncwarp();
+    ptx::cluster_sync();          // every CTA's columns are in
+    // ---- one leaf of every chain still building (chains dealt over the cluster's warps)
+    bool still = false;
+    {
+      const int r = warp * ctas + rank;      // (more warps than chains past 4 CTAs)
+      const int c = m0 + r;
+      if (r < rows && c < C && na.st[c].active) still = nuts_leaf<kModeGauss, NB>(na, c, lane);
+    }
+    // positions written for the next products' TMA loads (another proxy)
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    const int mine = __syncthreads_count(lane == 0 && still) + (bad_s ? kBad : 0);
+    if (threadIdx.x < ctas)
+      ptx::st_cluster_s32(ptx::mapa(ptx::smem_u32(&left_s[it & 1][rank]), threadIdx.x), mine);
+    __syncwarp();
+    ptx::cluster_sync();          // every CTA's positions and counts are in
+    int total = 0;
+    for (int i = 0; i < ctas; ++i) total += left_s[it & 1][i];
+    if (total == 0 || total >= kBad) break;
+    if (it + 1 >= (1 << na.max_depth)) {
+      if (threadIdx.x == 0) atomicExch(na.err, 2);
+      break;
+    }
+  }
+  if (threadIdx.x == 0 && rank == 0) atomicMax(&na.ctr[6], static_cast<unsigned>(it + 1));
+  ptx::tc_fence_before();
+  __syncwarp();
+  ptx::cluster_sync();
+  if (warp == 0) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, kPlBN);
+  }
+}
+
 template <int NB>
 cudaError_t set_leaf_attrs() {
   cudaError_t e = cudaFuncSetAttribute(k_nuts_dense_leaf<kModeGauss, NB>,
@@ -711,10 +898,7 @@ int gauss_loop_grid(int C, int D, int* sms_out = nullptr) {
   }
   if (occ < 0) {
     int o = 0;
-    const int nb = (D + 3) / 4 * 4 <= 128 ? 1 : (D + 3) / 4 * 4 <= 256 ? 2 : 4;
-    cudaError_t e = nb == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_nuts_gauss_loop<1>, kPlThreads, kPlSmem)
-                  : nb == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_nuts_gauss_loop<2>, kPlThreads, kPlSmem)
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_nuts_gauss_loop<4>, kPlThreads, kPlSmem);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_nuts_gauss_loop, kPlThreads, kPlSmem);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return 0;
@@ -741,6 +925,30 @@ cudaError_t enqueue_nb(const hmc_target& t, const NdArgs& base_args, NutsDense& 
   count_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  if (nd.mode == kModeGauss && a.D <= kClMaxChunks * kPlBK) {
+    GaussTc& tc = *nd.tc;
+    const int ctas = (a.D + kPlBN - 1) / kPlBN, rows = nuts_cluster_chains(a.D);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>((a.C + rows - 1) / rows * ctas));
+    cfg.blockDim = dim3(kClThreads);
+    cfg.dynamicSmemBytes = kClSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(ctas);
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    // (dim <= 256: at most two blocks of 128 dims per lane)
+    e = cudaLaunchKernelEx(&cfg, k_nuts_gauss_cluster<(NB < 4 ? NB : 2)>, tc.mAhi_blk, tc.mAlo_blk, tc.mBhi, tc.mBlo, na,
+                           ctas);
+    count_launch();
+    if (e != cudaSuccess) return e;
+    k_nuts_dense_finish<<<nb, 32 * kNdWarps, 0, s>>>(na);
+    count_launch();
+    if (timer) timer->end(s);
+    return cudaGetLastError();
+  }
   const int pgrid = nd.mode == kModeGauss ? gauss_loop_grid(a.C, a.D) : 0;
   if (pgrid > 0) {
     // the whole leaf loop in one cooperative launch (grid barrier and the
@@ -758,7 +966,7 @@ cudaError_t enqueue_nb(const hmc_target& t, const NdArgs& base_args, NutsDense& 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     GaussTc& tc = *nd.tc;
-    e = cudaLaunchKernelEx(&cfg, k_nuts_gauss_loop<NB>, tc.mAhi[0], tc.mAlo[0], tc.mBhi, tc.mBlo, na);
+    e = cudaLaunchKernelEx(&cfg, k_nuts_gauss_loop, tc.mAhi[0], tc.mAlo[0], tc.mBhi, tc.mBlo, na);
     count_launch();
     if (e != cudaSuccess) return e;
     k_nuts_dense_finish<<<nb, 32 * kNdWarps, 0, s>>>(na);
@@ -835,13 +1043,13 @@ cudaError_t nuts_dense_prepare() {
   if (e == cudaSuccess) e = set_leaf_attrs<2>();
   if (e == cudaSuccess) e = set_leaf_attrs<4>();
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_nuts_gauss_loop<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kPlSmem));
+    e = cudaFuncSetAttribute(k_nuts_gauss_cluster<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kClSmem));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_nuts_gauss_loop<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kPlSmem));
+    e = cudaFuncSetAttribute(k_nuts_gauss_cluster<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kClSmem));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_nuts_gauss_loop<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(k_nuts_gauss_loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kPlSmem));
   return e;
 }
