@@ -343,8 +343,9 @@ k_lr_grad(const __grid_constant__ CUtensorMap mThi, const __grid_constant__ CUte
       }
       if (ok && chain < a.C)
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-          if (d0 + k < a.ld) gout[d0 + k] = gv[k];    // (zero past D: X's padding)
+        for (int k = 0; k < 16; k += 4)
+          if (d0 + k < a.ld)                          // (zero past D: X's padding)
+            *reinterpret_cast<float4*>(gout + d0 + k) = make_float4(gv[k], gv[k + 1], gv[k + 2], gv[k + 3]);
     }
     lpred[group * 128 + r] = lp_acc;
   }
@@ -381,7 +382,7 @@ struct LrStepArgs {
   const float* Gpart;
   const float* lp_part;
   int nsplit;
-  int last;         // update kernel: final leapfrog step
+  int last;         // final leapfrog step
 };
 
 // p0 ~ N(0, I); H0; half kick with the cached gradient; first drift
@@ -409,68 +410,93 @@ __global__ void k_lr_begin(LrStepArgs b) {
   if (lane == 0) b.h0[c] = -a.lp[c] + 0.5f * kin;
 }
 
-// gradient and log p from the range partials (fixed order) and the prior;
-// leapfrog update (merged kicks + drift), or the final half kick.  One warp
-// per chain, four dims per lane (float4: every buffer here is the library's
-// own, 16-byte aligned, with rows of ld = D rounded up to 4), so that a
-// lane's loads of all range partials are in flight together.
+// v = sum over s < n of src[s * stride], in order, 16 loads in flight
+__device__ __forceinline__ void sum_ranges(const float4* src, int64_t stride, int n, float (&g)[4]) {
+  g[0] = g[1] = g[2] = g[3] = 0.f;
+  for (int s0 = 0; s0 < n; s0 += 16) {
+    float4 v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      if (s0 + k < n) v[k] = src[(s0 + k) * stride];
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      if (s0 + k < n) {
+        g[0] += v[k].x; g[1] += v[k].y; g[2] += v[k].z; g[3] += v[k].w;
+      }
+  }
+}
+
+// The middle steps' update -- gradient from the range partials (fixed order)
+// and the prior, merged kicks, drift -- needs no sum over the dims: a thread per
+// four dims (every buffer here is the library's own, 16-byte aligned, with rows
+// of ld = D rounded up to 4), in small blocks over all SMs.  (A warp per chain
+// with four loads in flight: %LRU%)
+__global__ void __launch_bounds__(128) k_lr_update_middle(LrStepArgs b) {
+  const int D4 = b.ld >> 2;           // (the padding stays zero: X's padding columns are zero)
+  const int64_t n4 = static_cast<int64_t>(b.s.C) * D4;
+  const int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (e >= n4) return;
+  const float eps = b.s.da->eps;
+  const float4 h = reinterpret_cast<const float4*>(b.thi)[e], l = reinterpret_cast<const float4*>(b.tlo)[e];
+  const float4 pv = reinterpret_cast<const float4*>(b.p)[e];
+  float g[4];
+  sum_ranges(reinterpret_cast<const float4*>(b.Gpart) + e, n4, b.nsplit, g);
+  const float th[4] = {h.x + l.x, h.y + l.y, h.z + l.z, h.w + l.w};
+  const float pin[4] = {pv.x, pv.y, pv.z, pv.w};
+  float pout[4], hi[4], lo[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    g[k] -= th[k];
+    pout[k] = fmaf(eps, g[k], pin[k]);
+    split_tf32(fmaf(eps, pout[k], th[k]), hi[k], lo[k]);
+  }
+  reinterpret_cast<float4*>(b.p)[e] = make_float4(pout[0], pout[1], pout[2], pout[3]);
+  reinterpret_cast<float4*>(b.thi)[e] = make_float4(hi[0], hi[1], hi[2], hi[3]);
+  reinterpret_cast<float4*>(b.tlo)[e] = make_float4(lo[0], lo[1], lo[2], lo[3]);
+}
+
+// The last step: gradient, log p and the final half kick.  One warp per
+// chain, four dims per lane.
 __global__ void k_lr_update(LrStepArgs b) {
   const StepArgs& a = b.s;
   const int c = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (c >= a.C) return;
-  const int D4 = b.ld >> 2;           // (the padding stays zero: X's padding columns are zero)
+  const int D4 = b.ld >> 2;
   const int64_t row4 = static_cast<int64_t>(c) * D4;
   const int64_t split4 = static_cast<int64_t>(a.C) * D4;
   const float eps = a.da->eps;
-  const float4* thi = reinterpret_cast<const float4*>(b.thi);
-  const float4* tlo = reinterpret_cast<const float4*>(b.tlo);
-  const float4* Gp = reinterpret_cast<const float4*>(b.Gpart);
-  float4* p4 = reinterpret_cast<float4*>(b.p);
   float sq = 0.f;
-  for (int j = lane; j < D4; j += 32) {
+  for (int j = lane; j < D4; j += 32) {      // (dim <= 128: once)
     const int64_t e = row4 + j;
-    const float4 h = thi[e], l = tlo[e];
+    const float4 h = reinterpret_cast<const float4*>(b.thi)[e], l = reinterpret_cast<const float4*>(b.tlo)[e];
+    const float4 pv = reinterpret_cast<const float4*>(b.p)[e];
+    float g[4];
+    sum_ranges(reinterpret_cast<const float4*>(b.Gpart) + e, split4, b.nsplit, g);
     const float th[4] = {h.x + l.x, h.y + l.y, h.z + l.z, h.w + l.w};
-    float g[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int s = 0; s < b.nsplit; ++s) {
-      const float4 v = Gp[s * split4 + e];
-      g[0] += v.x; g[1] += v.y; g[2] += v.z; g[3] += v.w;
-    }
-    const float4 pv = p4[e];
     const float pin[4] = {pv.x, pv.y, pv.z, pv.w};
-    float pout[4], hi[4], lo[4];
+    float pout[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       g[k] -= th[k];
       sq = fmaf(th[k], th[k], sq);
-      if (!b.last) {
-        pout[k] = fmaf(eps, g[k], pin[k]);
-        split_tf32(fmaf(eps, pout[k], th[k]), hi[k], lo[k]);
-      } else {
-        pout[k] = fmaf(0.5f * eps, g[k], pin[k]);
-      }
+      pout[k] = fmaf(0.5f * eps, g[k], pin[k]);
     }
-    p4[e] = make_float4(pout[0], pout[1], pout[2], pout[3]);
-    if (!b.last) {
-      reinterpret_cast<float4*>(b.thi)[e] = make_float4(hi[0], hi[1], hi[2], hi[3]);
-      reinterpret_cast<float4*>(b.tlo)[e] = make_float4(lo[0], lo[1], lo[2], lo[3]);
-    } else {
-      reinterpret_cast<float4*>(b.gL)[e] = make_float4(g[0], g[1], g[2], g[3]);
-    }
+    reinterpret_cast<float4*>(b.p)[e] = make_float4(pout[0], pout[1], pout[2], pout[3]);
+    reinterpret_cast<float4*>(b.gL)[e] = make_float4(g[0], g[1], g[2], g[3]);
   }
-  if (b.last) {
-    sq = warp_sum(sq);
-    if (lane == 0) {
-      float lp = 0.f;
-      for (int s = 0; s < b.nsplit; ++s) lp += b.lp_part[static_cast<int64_t>(s) * a.C + c];
-      b.lpL[c] = lp - 0.5f * sq;
-    }
+  sq = warp_sum(sq);
+  // the ranges' log-likelihoods in order: loaded by the lanes, added by all
+  float lp = 0.f;
+  for (int s0 = 0; s0 < b.nsplit; s0 += 32) {
+    const float v = s0 + lane < b.nsplit ? b.lp_part[static_cast<int64_t>(s0 + lane) * a.C + c] : 0.f;
+    const int n = min(32, b.nsplit - s0);
+    for (int k = 0; k < n; ++k) lp += __shfl_sync(0xffffffffu, v, k);
   }
+  if (lane == 0) b.lpL[c] = lp - 0.5f * sq;
 }
 
-// H_L, Metropolis-Hastings select, traces, dual averaging
+// H_L, Metropolis-Hastings select, traces, dual averaging (warp per chain)
 __global__ void k_lr_accept(LrStepArgs b) {
   const StepArgs& a = b.s;
   const int c = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
@@ -482,6 +508,7 @@ __global__ void k_lr_accept(LrStepArgs b) {
     const int64_t row = static_cast<int64_t>(c) * D, wrow = static_cast<int64_t>(c) * b.ld;
     const uint32_t chain = static_cast<uint32_t>(c) + a.chain_offset;
     float kin = 0.f;
+#pragma unroll 4
     for (int d = lane; d < D; d += 32) kin = fmaf(b.p[wrow + d], b.p[wrow + d], kin);
     kin = 0.5f * warp_sum(kin);
     const float lp1 = b.lpL[c];
@@ -490,13 +517,18 @@ __global__ void k_lr_accept(LrStepArgs b) {
     int acc = 0;
     if (lane == 0) acc = accept_log_uniform(a.seed, chain, a.t) < la;
     acc = __shfl_sync(0xffffffffu, acc, 0);
+#pragma unroll 4
     for (int d = lane; d < D; d += 32) {
       const int64_t e = row + d, w = wrow + d;
+      float x = 0.f;
       if (acc) {
-        a.x[e] = b.thi[w] + b.tlo[w];
+        x = b.thi[w] + b.tlo[w];
+        a.x[e] = x;
         a.g[e] = b.gL[w];
+      } else if (a.sample_out) {
+        x = a.x[e];
       }
-      if (a.sample_out) a.sample_out[e] = a.x[e];
+      if (a.sample_out) a.sample_out[e] = x;
     }
     if (lane == 0) {
       if (acc) a.lp[c] = lp1;
@@ -734,7 +766,9 @@ cudaError_t launch_logreg_tc_transition(const StepArgs& a, LogregTc& tc, int* er
     if (timer) timer->end(s);
     if (e != cudaSuccess) return e;
     b.last = l == a.L;
-    k_lr_update<<<nb, 32 * kWarpsPerBlock, 0, s>>>(b);
+    const int64_t n4 = static_cast<int64_t>(a.C) * (tc.ld / 4);
+    if (b.last) k_lr_update<<<nb, 32 * kWarpsPerBlock, 0, s>>>(b);
+    else k_lr_update_middle<<<static_cast<unsigned>((n4 + 127) / 128), 128, 0, s>>>(b);
     count_launch(2);
   }
   k_lr_accept<<<nb, 32 * kWarpsPerBlock, 0, s>>>(b);
