@@ -176,6 +176,8 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
   else __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  ptx::grid_dependents_launch();
+  ptx::grid_dependency_wait();
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer
@@ -670,6 +672,8 @@ k_lr_z_persist(const __grid_constant__ CUtensorMap mAhi, const __grid_constant__
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  ptx::grid_dependents_launch();
+  ptx::grid_dependency_wait();
 
   // tile t: chains (t % mt) 128, data rows (t / mt) 64
   if (warp == 0 && lane == 0) {
@@ -828,6 +832,7 @@ struct TcBeginAccept {
 
 // p0 ~ N(0, I); H0; half kick with the cached gradient; first drift (warp per chain)
 __global__ void k_gauss_tc_begin(TcBeginAccept b) {
+  ptx::grid_dependents_launch();
   const StepArgs& a = b.s;
   if (b.met && blockIdx.x == 0)
     for (int i = threadIdx.x; i < b.nmet; i += blockDim.x) b.met[i] = 0u;
@@ -954,6 +959,8 @@ struct LrSumArgs {
 constexpr int kMaxSplit = 16;      // the most K-splits of the gradient product G = R X
 
 __global__ void __launch_bounds__(256) k_lr_gemm_update_middle(LrSumArgs b) {
+  ptx::grid_dependents_launch();
+  ptx::grid_dependency_wait();
   const int ld4 = b.ld >> 2;
   const int64_t n4 = static_cast<int64_t>(b.C) * ld4;
   const int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -1359,51 +1366,39 @@ size_t a1k(size_t b) { return (b + 1023) & ~static_cast<size_t>(1023); }
 // (96 KB), so that two CTAs share an SM and one's epilogue (the residual,
 // R to HBM) overlaps the other's products -- 128-row tiles at one CTA per SM
 // measured 5 % slower on a dim-254, 19102-row, 1204-chain gradient; G = R X
-// in one tile over the dims up to 256 wide (each re-reads R, C x Npad, from
-// HBM: four times at 64 columns for a dim of 256)
+// in tiles of 64 to 256 dims (lr_tiles)
 struct LrTiles {
   int bnz, bng, nrt, ndt;
 };
 // R X's tile: split-K products, bn columns (a multiple of 32)
 template <int EPI>
-void launch_tile(int bn, dim3 grid, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc,
-                 const CUtensorMap& md, const TcStepArgs& st, cudaStream_t s) {
-  if (bn == 64)
-    k_gauss_tc_step<EPI, 64><<<grid, kThreads, Tile<64>::kSmem, s>>>(ma, mb, mc, md, st);
-  else if (bn == 96)
-    k_gauss_tc_step<EPI, 96><<<grid, kThreads, Tile<96>::kSmem, s>>>(ma, mb, mc, md, st);
-  else if (bn == 128)
-    k_gauss_tc_step<EPI, 128><<<grid, kThreads, Tile<128>::kSmem, s>>>(ma, mb, mc, md, st);
-  else if (bn == 160)
-    k_gauss_tc_step<EPI, 160><<<grid, kThreads, Tile<160>::kSmem, s>>>(ma, mb, mc, md, st);
-  else if (bn == 192)
-    k_gauss_tc_step<EPI, 192><<<grid, kThreads, Tile<192>::kSmem, s>>>(ma, mb, mc, md, st);
-  else if (bn == 224)
-    k_gauss_tc_step<EPI, 224><<<grid, kThreads, Tile<224>::kSmem, s>>>(ma, mb, mc, md, st);
-  else
-    k_gauss_tc_step<EPI, 256><<<grid, kThreads, Tile<256>::kSmem, s>>>(ma, mb, mc, md, st);
+cudaError_t launch_tile(int bn, dim3 grid, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc,
+                        const CUtensorMap& md, const TcStepArgs& st, cudaStream_t s) {
+  // (NUTS: the active flags decide before the kernel waits for the launch
+  // before it, so there it is an ordinary launch)
+  auto go = [&](StepKernel k, size_t smem) {
+    if (!st.active) return launch_dependent(k, grid, dim3(kThreads), smem, s, ma, mb, mc, md, st);
+    k<<<grid, kThreads, smem, s>>>(ma, mb, mc, md, st);
+    return cudaGetLastError();
+  };
+  switch (bn) {
+    case 64: return go(k_gauss_tc_step<EPI, 64>, Tile<64>::kSmem);
+    case 96: return go(k_gauss_tc_step<EPI, 96>, Tile<96>::kSmem);
+    case 128: return go(k_gauss_tc_step<EPI, 128>, Tile<128>::kSmem);
+    case 160: return go(k_gauss_tc_step<EPI, 160>, Tile<160>::kSmem);
+    case 192: return go(k_gauss_tc_step<EPI, 192>, Tile<192>::kSmem);
+    case 224: return go(k_gauss_tc_step<EPI, 224>, Tile<224>::kSmem);
+    default: return go(k_gauss_tc_step<EPI, 256>, Tile<256>::kSmem);
+  }
 }
 
-LrTiles lr_tiles(int64_t npad, int ld) {
-  LrTiles q{};
-  q.bnz = 64;
-  q.nrt = static_cast<int>((npad + q.bnz - 1) / q.bnz);
-  // the dims in tiles of up to 256, as even as multiples of 32 allow: 301 dims
-  // take two tiles of 160, not 256 + 48 (each tile's width costs its loads of X
-  // and its MMAs; 47.7 us -> 32.5 us at 8000 rows, 700 chains)
-  q.ndt = (ld + 255) / 256;
-  q.bng = std::max(64, ((ld + q.ndt - 1) / q.ndt + 31) / 32 * 32);
-  return q;
-}
-
-// G = R X has K = Npad but only (C / 128) x ndt tiles: split K when the tiles
-// would not fill two waves of the SMs, and sum the splits afterwards
-void lr_splits(const LogregGemm& g, int C, int* S_out, int* kc_out) {
-  const int64_t mt = (C + kBM - 1) / kBM;
-  const int nk_all = g.npad / kBK;
-  const int64_t tiles = mt * g.ndt;
+// K-splits of G = R X, which has K = Npad but few tiles (blocks of 128 chains x
+// 256 dims): enough to fill two waves of the SMs with those, summed afterwards.
+// (The splits fix the order of the sums; the tiles below do not.)
+void lr_splits(int64_t C, int64_t npad, int ld, int* S_out, int* kc_out) {
+  const int64_t tiles = (C + kBM - 1) / kBM * ((ld + 255) / 256), sms = current_sm_count();
+  const int nk_all = static_cast<int>(npad / kBK);
   int S = 1, kc_split = nk_all;
-  const int64_t sms = g.sms;
   if (tiles < 2 * sms && nk_all >= 2) {
     S = static_cast<int>(std::min<int64_t>({kMaxSplit, (2 * sms + tiles - 1) / tiles, nk_all}));
     kc_split = (nk_all + S - 1) / S;
@@ -1412,12 +1407,40 @@ void lr_splits(const LogregGemm& g, int C, int* S_out, int* kc_out) {
   *S_out = S;
   *kc_out = kc_split;
 }
+
+// The dims of G in even tiles, as few as are within an eighth of the least of
+// waves x bytes per K-chunk (a CTA's loads -- 16 KB of R and 128 B per column, for
+// each of head and remainder -- are what a tile takes its time for; more tiles
+// read R more often).  Per gradient: 300 chains x 15000 rows x 200 dims, one tile of
+// 224 on 48 CTAs 73.0 us, three of 96 on 144 58.9; 64 x 20000 x 512 94.5 -> 70.1
+// (eight of 64); 700 x 8000 x 512 118.1 -> 113.1 (three of 192); at 700 x 8000 x 301 two
+// tiles of 160 (78.7) beat three of 128 (79.5) and 256 + 48.
+LrTiles lr_tiles(int64_t npad, int ld, int64_t C) {
+  LrTiles q{};
+  q.bnz = 64;
+  q.nrt = static_cast<int>((npad + q.bnz - 1) / q.bnz);
+  int S = 1, kc = 1;
+  lr_splits(C, npad, ld, &S, &kc);
+  const int64_t mt = (C + kBM - 1) / kBM, sms = current_sm_count();
+  int64_t best = 0;
+  for (int n = (ld + 255) / 256; n <= (ld + 63) / 64; ++n) {
+    const int bn = std::max(64, ((ld + n - 1) / n + 31) / 32 * 32);
+    const int ndt = (ld + bn - 1) / bn;
+    const int64_t cost = (mt * ndt * S + sms - 1) / sms * (128 + bn);
+    if (best == 0 || 100 * cost < 88 * best) {
+      best = cost;
+      q.bng = bn;
+      q.ndt = ndt;
+    }
+  }
+  return q;
+}
 }  // namespace
 
 size_t logreg_gemm_workspace_bytes(const hmc_target& t, int64_t C) {
   const size_t npad = static_cast<size_t>(lr_npad(t.n_data)), D = static_cast<size_t>((t.dim + 3) / 4 * 4);
   const size_t ND = npad * D, CN = static_cast<size_t>(C) * npad, CD = static_cast<size_t>(C) * D;
-  const LrTiles q = lr_tiles(static_cast<int64_t>(npad), static_cast<int>(D));
+  const LrTiles q = lr_tiles(static_cast<int64_t>(npad), static_cast<int>(D), C);
   const size_t ntot = static_cast<size_t>(q.nrt + q.ndt);
   return 4 * a1k(ND * 4) + a1k(npad * 4) + 2 * a1k(CN * 4) + 6 * a1k(CD * 4) +
          a1k(static_cast<size_t>(C) * ntot * 4) + a1k(static_cast<size_t>(C) * 4) + a1k(sizeof(int)) +
@@ -1437,7 +1460,7 @@ cudaError_t logreg_gemm_setup(LogregGemm* g, const hmc_target& t, int64_t C, voi
   cudaError_t qe = cudaGetDevice(&dev);
   if (qe == cudaSuccess) qe = cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, dev);
   if (qe != cudaSuccess) return qe;
-  const LrTiles q = lr_tiles(npad, ld);
+  const LrTiles q = lr_tiles(npad, ld, C);
   g->bnz = q.bnz;
   g->bng = q.bng;
   g->nrt = q.nrt;
@@ -1522,7 +1545,7 @@ cudaError_t launch_logreg_gemm_transition(const StepArgs& a, LogregGemm& g, cuda
   count_launch();
   const unsigned mt = static_cast<unsigned>((a.C + kBM - 1) / kBM);
   int S = 1, kc_split = 1;
-  lr_splits(g, a.C, &S, &kc_split);
+  lr_splits(a.C, g.npad, g.ld, &S, &kc_split);
   for (int l = 1; l <= a.L; ++l) {
     const int in = (l - 1) & 1, out = l & 1;
     const bool last = l == a.L;
@@ -1564,20 +1587,23 @@ cudaError_t launch_logreg_gemm_transition(const StepArgs& a, LogregGemm& g, cuda
     if (timer) timer->begin(s);
     {
       const int zt = static_cast<int>(mt) * g.nrt;      // Z tiles, one persistent CTA per SM
-      k_lr_z_persist<<<static_cast<unsigned>(std::min(zt, g.sms)), kThreads, kZpSmem, s>>>(
-          g.mThi[in], g.mTlo[in], g.mXhi, g.mXlo, z, static_cast<int>(mt), zt);
+      const cudaError_t e =
+          launch_dependent(k_lr_z_persist, dim3(static_cast<unsigned>(std::min(zt, g.sms))), dim3(kThreads), kZpSmem,
+                           s, g.mThi[in], g.mTlo[in], g.mXhi, g.mXlo, z, static_cast<int>(mt), zt);
+      if (e != cudaSuccess) return e;
     }
     {
       // the split products G = R X, then their sum with the prior and the
       // leapfrog update (k_lr_gemm_update)
       st.kc_split = kc_split;
       st.part = g.part;
-      launch_tile<kEpiStore>(g.bng, dim3(mt, g.ndt, S), g.mRhi, g.mRlo, g.mXThi, g.mXTlo, st, s);
+      const cudaError_t e = launch_tile<kEpiStore>(g.bng, dim3(mt, g.ndt, S), g.mRhi, g.mRlo, g.mXThi, g.mXTlo, st, s);
+      if (e != cudaSuccess) return e;
       LrSumArgs u{a.C, a.D, g.ld, S, last ? 1 : 0, g.nrt, g.ntot, g.part, g.xhi[in], g.xlo[in],
                   g.xhi[out], g.xlo[out], g.p, g.gL, g.lp_part, a.da};
       const int64_t n4 = static_cast<int64_t>(a.C) * (g.ld / 4);
       if (last) k_lr_gemm_update<<<nb, 32 * kWarpsPerBlock, 0, s>>>(u);
-      else k_lr_gemm_update_middle<<<static_cast<unsigned>((n4 + 255) / 256), 256, 0, s>>>(u);
+      else launch_dependent(k_lr_gemm_update_middle, dim3(static_cast<unsigned>((n4 + 255) / 256)), dim3(256), 0, s, u);
       count_launch();
     }
     if (timer) timer->end(s);
@@ -1594,7 +1620,7 @@ cudaError_t launch_logreg_gemm_products(LogregGemm& g, int C, int D, const DASta
                                         const uint8_t* active, int* splits, cudaStream_t s) {
   const unsigned mt = static_cast<unsigned>((C + kBM - 1) / kBM);
   int S = 1, kc_split = 1;
-  lr_splits(g, C, &S, &kc_split);
+  lr_splits(C, g.npad, g.ld, &S, &kc_split);
   TcStepArgs z{};
   z.C = C;
   z.D = D;
@@ -1626,10 +1652,10 @@ cudaError_t launch_logreg_gemm_products(LogregGemm& g, int C, int D, const DASta
   st.active = active;
   k_gauss_tc_step<kEpiLrResid, 64, 2><<<dim3(mt, g.nrt), kThreads, Tile<64, 2>::kSmem, s>>>(
       g.mThi[0], g.mTlo[0], g.mXhi, g.mXlo, z);
-  launch_tile<kEpiStore>(g.bng, dim3(mt, g.ndt, S), g.mRhi, g.mRlo, g.mXThi, g.mXTlo, st, s);
+  const cudaError_t e = launch_tile<kEpiStore>(g.bng, dim3(mt, g.ndt, S), g.mRhi, g.mRlo, g.mXThi, g.mXTlo, st, s);
   count_launch(2);
   *splits = S;
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace hmc

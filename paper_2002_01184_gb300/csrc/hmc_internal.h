@@ -63,6 +63,26 @@ cudaError_t launch_vjp(const hmc_target& t, int64_t C, const float* x, const flo
 // dx[c, :] = w[c] g[c, :]
 cudaError_t launch_scale_rows(int64_t C, int D, const float* w, const float* g, float* dx, cudaStream_t s);
 
+// Launch `kernel` so that its prologue may overlap the end of the launch before
+// it on the stream (programmatic dependent launch).  The kernel waits
+// (ptx::grid_dependency_wait) before it touches what earlier launches wrote or
+// still read.
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                    A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Set the error text that hmc_last_error(NULL) returns on this thread.
 void set_global_error(const std::string& msg);
 

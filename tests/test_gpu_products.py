@@ -124,3 +124,29 @@ def test_trajectory_launch_equals_step_launches(D, L):
     for x, s, a in out[1:]:
         C = x.shape[0]
         assert torch.equal(x, out[0][0][:C]) and torch.equal(s, out[0][1][:, :C]) and torch.equal(a, out[0][2][:, :C])
+
+
+# R X in one to eight tiles of the dims, past one launch's widest tile
+@pytest.mark.parametrize("C,N,D", [(40, 5000, 140), (128, 3000, 200), (300, 2500, 301), (90, 2200, 512)])
+def test_logreg_tiles_against_float64(C, N, D):
+    gen = torch.Generator(device="cuda").manual_seed(D)
+    X = torch.randn(N, D, device="cuda", generator=gen)
+    y = (torch.rand(N, device="cuda", generator=gen) < 0.5).float()
+    x0 = torch.randn(C, D, device="cuda", generator=gen) / D ** 0.5
+    cfg = H.make_config(2, 1e-3 / D ** 0.5, seed=3)
+    ctx = H.hmc_create(H.make_target("logreg", D, X=X, y=y), C, cfg)
+    assert H.hmc_uses_tensor_cores(ctx)
+    x = x0.clone()
+    H.hmc_bootstrap(ctx, x)
+    r = H.hmc_step(ctx, x, 0)
+    H.hmc_synchronize(ctx)
+    from paper_2002_01184_gb300.sampler import device_view
+    g = device_view(r.grad, (C, D), "<f4").clone().double()
+    acc = device_view(r.is_accepted, (C,), "|u1").clone().bool()
+    H.hmc_destroy(ctx)
+    assert acc.any()
+    x64 = x.double()
+    ref = (y.double() - torch.sigmoid(x64 @ X.double().T)) @ X.double() - x64
+    # the tensor-core gradient's tolerance: 1e-4 of each chain's largest element
+    err = (g - ref).abs().amax(1) / ref.abs().amax(1)
+    assert (err[acc] < 1e-4).all()
