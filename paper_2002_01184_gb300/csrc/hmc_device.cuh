@@ -200,6 +200,7 @@ __device__ __forceinline__ bool tile_partial_then_da(DAState* s, double* partial
                                                      int num_chains, long long t, int tile,
                                                      int ntiles) {
   __shared__ bool last;
+  __shared__ DACoef coef;
   if (threadIdx.x == 0) {
     partials[tile] = block_sum;
     __threadfence();
@@ -210,15 +211,26 @@ __device__ __forceinline__ bool tile_partial_then_da(DAState* s, double* partial
   const bool mine = last;
   if (!mine) return false;
   __threadfence();
+  // (float64 latency is 64 cycles: another warp forms the update's
+  // coefficients meanwhile, and eight partials are in flight at a time)
   double acc = 0.0;
   if (threadIdx.x < 32) {
-    for (int b = threadIdx.x; b < ntiles; b += 32) acc += static_cast<volatile double*>(partials)[b];
-    acc = warp_sum_d(acc);
-    if (threadIdx.x == 0) {
-      da_update(s, acc / static_cast<double>(num_chains), t);
-      s->arrive = 0u;
-      __threadfence();
+    for (int b = threadIdx.x; b < ntiles; b += 256) {
+      double v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = b + 32 * i < ntiles ? __ldcg(partials + b + 32 * i) : 0.0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc += v[i];
     }
+    acc = warp_sum_d(acc);
+  } else if (threadIdx.x == 32) {
+    coef = da_prepare(s, t);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    da_apply(s, coef, acc / static_cast<double>(num_chains), t);
+    s->arrive = 0u;
+    __threadfence();
   }
   return true;
 }
