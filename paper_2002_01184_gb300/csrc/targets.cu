@@ -80,6 +80,7 @@ struct GemmTile {
   static constexpr int BM = 16 * TM;
   static constexpr int QA = BM * kBK / 4 / kGemmThreads;         // float4 per thread and buffer
   static constexpr int QB = kBN * kBK / 4 / kGemmThreads;
+  static_assert(BM % 32 == 0 && TM % 2 == 0, "whole swizzle groups, pairs of rows");
   float a[2][kBK][BM];
   float b[2][kBK][kBN];
 };
@@ -150,11 +151,17 @@ __device__ __forceinline__ void gemm_tile(const Gemm& g, int m0, int n0, GemmTil
     for (int kk = 0; kk < kBK; ++kk) {
       const int u = kk >> 2;
       unsigned long long av[TM / 2];
+      if (TM % 4 == 0) {
 #pragma unroll
-      for (int i = 0; i < TM; i += 4) {
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&s.a[buf][kk][(ty * TM + i) ^ (4 * u)]);
-        av[i / 2] = v.x;
-        av[i / 2 + 1] = v.y;
+        for (int i = 0; i < TM; i += 4) {
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&s.a[buf][kk][(ty * TM + i) ^ (4 * u)]);
+          av[i / 2] = v.x;
+          av[(i / 2 + 1) % (TM / 2)] = v.y;
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < TM; i += 2)
+          av[i / 2] = *reinterpret_cast<const unsigned long long*>(&s.a[buf][kk][(ty * TM + i) ^ (4 * u)]);
       }
       const float4 bq = *reinterpret_cast<const float4*>(&s.b[buf][kk][(4 * tx) ^ (4 * u)]);
       const float bv[4] = {bq.x, bq.y, bq.z, bq.w};
@@ -393,31 +400,35 @@ __global__ void k_scale_rows(int C, int D, const float* __restrict__ w, const fl
   }
 }
 
-// Rows of the tiles of an M x N product in `splits` parts: 128 or 64.  The
-// larger tile loads less per multiply-add (1.13 - 1.21 times as fast with all SMs
-// busy: 583 against 661 us at 2048 x 20000 x 128, 214 against 260 us at 700 x
-// 8000 x 301), the smaller one divides more evenly over the SMs (56 against 70 us
-// at 64 x 20000 x 128).
-bool tall_tiles(int64_t M, int64_t N, int64_t splits) {
+// Rows of the tiles of an M x N product in `splits` parts, as TM: 8 (128 rows), 6
+// or 4.  The larger tile loads less per multiply-add (128 rows against 64: 583
+// against 661 us at 2048 x 20000 x 128, 214 against 260 us at 700 x 8000 x 301), the
+// smaller one divides more evenly over the SMs (56 against 70 us at 64 x 20000 x
+// 128); 96 rows make the 2048 x 128 x 20000 product in 10 splits 440 tiles, three an
+// SM at most (583 -> 535 us for the whole gradient), and lose to 128 where those fill
+// as many waves (29 against 21 us at 4096 x 256 x 256).
+int tile_rows(int64_t M, int64_t N, int64_t splits) {
   const int64_t sms = current_sm_count();
-  auto cost = [&](int64_t bm, double rate) {
-    const int64_t tiles = ((M + bm - 1) / bm) * ((N + kBN - 1) / kBN) * splits;
+  auto cost = [&](int tm, double rate) {
+    const int64_t bm = 16 * tm, tiles = ((M + bm - 1) / bm) * ((N + kBN - 1) / kBN) * splits;
     return static_cast<double>((tiles + sms - 1) / sms * bm) / rate;
   };
-  return cost(128, 1.16) <= cost(64, 1.0);
+  const double c8 = cost(8, 1.16), c6 = cost(6, 1.08), c4 = cost(4, 1.0);
+  return c8 <= c6 && c8 <= c4 ? 8 : c6 < c4 ? 6 : 4;
 }
 
-dim3 gemm_grid(const Gemm& q, bool tall, int splits = 1) {
-  return dim3((q.N + kBN - 1) / kBN, tall ? (q.M + 127) / 128 : (q.M + 63) / 64, splits);
+dim3 gemm_grid(const Gemm& q, int tm, int splits = 1) {
+  return dim3((q.N + kBN - 1) / kBN, (q.M + 16 * tm - 1) / (16 * tm), splits);
 }
 
 inline bool rows16(const float* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && ld % 4 == 0; }
 
 void corr_gauss_product(int C, int D, const float* x, const float* P, const float* w, float* g, cudaStream_t s) {
   const Gemm q{x, D, P, D, C, D, 0, D, rows16(x, D), rows16(P, D)};
-  const bool tall = tall_tiles(C, D, 1), vec = rows16(g, D);
-  if (tall) k_corr_gauss_grad<8><<<gemm_grid(q, tall), kGemmThreads, 0, s>>>(q, w, g, vec);
-  else k_corr_gauss_grad<4><<<gemm_grid(q, tall), kGemmThreads, 0, s>>>(q, w, g, vec);
+  const int tm = tile_rows(C, D, 1);
+  const bool vec = rows16(g, D);
+  auto k = tm == 8 ? k_corr_gauss_grad<8> : tm == 6 ? k_corr_gauss_grad<6> : k_corr_gauss_grad<4>;
+  k<<<gemm_grid(q, tm), kGemmThreads, 0, s>>>(q, w, g, vec);
 }
 
 template <bool LP>
@@ -425,15 +436,13 @@ void logreg_products(const hmc_target& t, int C, const float* x, const LogregPla
                      cudaStream_t s) {
   const int D = t.dim, N = static_cast<int>(t.n_data);
   const Gemm z{x, D, t.X, D, C, N, 0, D, rows16(x, D), rows16(t.X, D)};
-  if (const bool tall = tall_tiles(C, N, 1))
-    k_logreg_residual<8, LP><<<gemm_grid(z, tall), kGemmThreads, 0, s>>>(z, t.y, R, lpp);
-  else
-    k_logreg_residual<4, LP><<<gemm_grid(z, tall), kGemmThreads, 0, s>>>(z, t.y, R, lpp);
+  const int zm = tile_rows(C, N, 1);
+  auto kz = zm == 8 ? k_logreg_residual<8, LP> : zm == 6 ? k_logreg_residual<6, LP> : k_logreg_residual<4, LP>;
+  kz<<<gemm_grid(z, zm), kGemmThreads, 0, s>>>(z, t.y, R, lpp);
   const Gemm r{R, N, t.X, D, C, D, 0, N, rows16(R, N), rows16(t.X, D)};
-  if (const bool tall = tall_tiles(C, D, p.splits))
-    k_logreg_grad_partial<8><<<gemm_grid(r, tall, p.splits), kGemmThreads, 0, s>>>(r, p.chunk, Gp, D % 4 == 0);
-  else
-    k_logreg_grad_partial<4><<<gemm_grid(r, tall, p.splits), kGemmThreads, 0, s>>>(r, p.chunk, Gp, D % 4 == 0);
+  const int gm = tile_rows(C, D, p.splits);
+  auto kg = gm == 8 ? k_logreg_grad_partial<8> : gm == 6 ? k_logreg_grad_partial<6> : k_logreg_grad_partial<4>;
+  kg<<<gemm_grid(r, gm, p.splits), kGemmThreads, 0, s>>>(r, p.chunk, Gp, D % 4 == 0);
 }
 
 }  // namespace

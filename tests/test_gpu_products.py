@@ -150,3 +150,13 @@ def test_logreg_tiles_against_float64(C, N, D):
     # the tensor-core gradient's tolerance: 1e-4 of each chain's largest element
     err = (g - ref).abs().amax(1) / ref.abs().amax(1)
     assert (err[acc] < 1e-4).all()
+
+
+# sizes at which tiles of 96 rows fill one wave where 128 leave SMs idle and 64
+# need two: the gradient's product, the residuals, the split sum over the rows
+@pytest.mark.parametrize("offset", [0, 1])
+def test_tiles_of_96_rows(offset):
+    for C, D in ((14592, 31), (14591, 68)):
+        test_gaussian_gradient_at_tile_edges(C, D, offset)
+    for C, N, D in ((2000, 400, 37), (767, 9000, 31)):
+        test_logreg_gradient_at_tile_edges(C, N, D, offset)
