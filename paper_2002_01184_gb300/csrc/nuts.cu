@@ -18,6 +18,17 @@
 // ends and the two candidates in a per-chain scratch of kNutsSlots slots of
 // D floats.
 //
+// What bounds it is the time of one leaf of the longest chain, a warp alone on its
+// scheduler for most of a launch: the instructions of a leaf one after another,
+// with every branch that is taken and every shuffle level waited for.  So a
+// leaf's gradient does not wait for its own sum of squares: x of leaf k + 1 needs
+// only leaf k's gradient, and its sum of squares rides in leaf k's butterfly with
+// |p|^2 and the U-turn dot products (the exponential of the funnel's v runs
+// beneath it); the usual leaf has no branch but the loop's; an even leaf is kept
+// once for all the spans it opens.  Measured: a leaf of the 100-dim funnel 646 -> 537
+// ns at 1024 chains (1000 -> 832 us for 20 transitions), 800 -> 731 ns at 4096,
+// 1577 -> 1471 at 16384, of the 10-dim one 617 -> 509; 500 dims, 1000 chains 1050 -> 867.
+//
 // The random streams and the choice rule are those of nuts_common.cuh.
 #include <cmath>
 
@@ -48,10 +59,19 @@ size_t span_smem_bytes(int Dp, int max_depth) {
   return static_cast<size_t>(kWarps) * 2 * (max_depth > 1 ? max_depth - 1 : 0) * Dp * sizeof(float);
 }
 
-// residency: 7 blocks (28 warps, 4256 chains on 152 SMs) per SM at NB = 1, 4
-// at NB = 2, 4 (registers)
-template <int TARGET, int NB, bool SMEM>
-__global__ void __launch_bounds__(32 * kWarps, NB == 1 ? 7 : 4) k_nuts(NutsArgs na) {
+// resident blocks per SM, which set the registers a thread may have: WIDE for
+// calls whose chains all fit so, else as many as a leaf's state allows without
+// spills on its critical path (funnel, 4096 x 100: 1458 us for 20 transitions at 5
+// blocks, 1869 at 7; standard normal, 4096 x 7: 491 at 7, 550 at 5)
+constexpr int nuts_blocks(int target, int nb, bool wide) {
+  return wide ? (nb == 1 ? 4 : 2) : target == HMC_T_FUNNEL ? (nb == 1 ? 5 : nb == 2 ? 4 : 3) : nb == 1 ? 7 : 4;
+}
+
+template <int TARGET, int NB, bool SMEM, bool WIDE>
+__global__ void __launch_bounds__(32 * kWarps, nuts_blocks(TARGET, NB, WIDE)) k_nuts(NutsArgs na) {
+  // the next leaf's position held over this leaf's decisions; the open pair's
+  // first leaf in registers
+  constexpr bool kKeepNext = WIDE || (TARGET == HMC_T_FUNNEL && NB == 1), kKeepFirst = kKeepNext && NB == 1;
   extern __shared__ float4 span_smem[];
   const StepArgs& a = na.s;
   const int warp = threadIdx.x >> 5;
@@ -118,73 +138,11 @@ __global__ void __launch_bounds__(32 * kWarps, NB == 1 ? 7 : 4) k_nuts(NutsArgs 
     };
     const float half_n = 0.5f * static_cast<float>(D - 1);
 
-    // The second half kick at the drifted x and every sum the leaf needs, in
-    // one butterfly: log p (through the sum of squares), |p|^2 and, where
-    // the span of two leaves closes here (close1), its U-turn dot products
-    // dx . pf and dx . p with dx = sv (x - xf) against the span's first leaf
-    // (xf, pf).  Sets g and p; returns log p, H = -log p + |p|^2 / 2 and
-    // whether that span makes a U-turn.
-    auto leaf_sums = [&](float h, float sv, bool close1, const float (&xf)[NB][4],
-                         const float (&pf)[NB][4], float* H, bool* turn) {
-      float q = 0.f, pp = 0.f, d1 = 0.f, d2 = 0.f;
-      if (TARGET == HMC_T_STD_NORMAL) {
-#pragma unroll
-        for (int b = 0; b < NB; ++b)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            g[b][i] = -x[b][i];
-            p[b][i] = fmaf(h, g[b][i], p[b][i]);
-            q = fmaf(x[b][i], x[b][i], q);
-            pp = fmaf(p[b][i], p[b][i], pp);
-            const float dx = sv * (x[b][i] - xf[b][i]);
-            d1 = fmaf(dx, pf[b][i], d1);
-            d2 = fmaf(dx, p[b][i], d2);
-          }
-        warp_sum4(q, pp, d1, d2);
-        const float lp = -0.5f * q;
-        *H = -lp + 0.5f * pp;
-        *turn = close1 && (d1 < 0.f || d2 < 0.f);
-        return lp;
-      } else {
-        // funnel: dim 0 (lane 0, b 0, i 0) is v; its gradient needs the sum
-        // of the others' squares, which the butterfly brings to every lane,
-        // so its terms are added after it from broadcast copies
-        const float v = __shfl_sync(0xffffffffu, x[0][0], 0);
-        const float p0 = __shfl_sync(0xffffffffu, p[0][0], 0);
-        const float xf0 = __shfl_sync(0xffffffffu, xf[0][0], 0);
-        const float pf0 = __shfl_sync(0xffffffffu, pf[0][0], 0);
-        const float ev = expf(-v);
-#pragma unroll
-        for (int b = 0; b < NB; ++b)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const bool is_v = b == 0 && i == 0 && lane == 0;
-            g[b][i] = -ev * x[b][i];
-            if (!is_v) {
-              p[b][i] = fmaf(h, g[b][i], p[b][i]);
-              q = fmaf(x[b][i], x[b][i], q);
-              pp = fmaf(p[b][i], p[b][i], pp);
-              const float dx = sv * (x[b][i] - xf[b][i]);
-              d1 = fmaf(dx, pf[b][i], d1);
-              d2 = fmaf(dx, p[b][i], d2);
-            }
-          }
-        warp_sum4(q, pp, d1, d2);
-        const float g0 = v * (-1.f / 9.f) - half_n + 0.5f * ev * q;
-        const float p0n = fmaf(h, g0, p0);
-        if (lane == 0) {
-          g[0][0] = g0;
-          p[0][0] = p0n;
-        }
-        const float dx0 = sv * (v - xf0);
-        d1 = fmaf(dx0, pf0, d1);
-        d2 = fmaf(dx0, p0n, d2);
-        const float lp = v * v * (-1.f / 18.f) - half_n * v - 0.5f * ev * q;
-        *H = -lp + 0.5f * fmaf(p0n, p0n, pp);
-        *turn = close1 && (d1 < 0.f || d2 < 0.f);
-        return lp;
-      }
-    };
+    // dim 0 of the funnel is v (lane 0, b 0, i 0); every lane keeps copies of
+    // its position, momentum and gradient, and the row sums leave it out: its
+    // terms are added to them afterwards
+    auto is_v = [&](int b, int i) { return TARGET == HMC_T_FUNNEL && b == 0 && i == 0 && lane == 0; };
+    auto lane0 = [&](const float (&u)[NB][4]) { return __shfl_sync(0xffffffffu, u[0][0], 0); };
 
     // the chain's state at the start of the launch
     float lp = a.lp[c];
@@ -214,7 +172,8 @@ __global__ void __launch_bounds__(32 * kWarps, NB == 1 ? 7 : 4) k_nuts(NutsArgs 
       const float logU = accept_log_uniform(a.seed, chain, t);
       store(kSlotLeft, x); store(kSlotLeft + 1, p); store(kSlotLeft + 2, g);
       store(kSlotRight, x); store(kSlotRight + 1, p); store(kSlotRight + 2, g);
-      store(kSlotCand, x); store(kSlotCand + 1, g);
+      int cand = kSlotCand, sub = kSlotSub;     // trade places when the subtree's is taken
+      store(cand, x); store(cand + 1, g);
       float lp_end[2] = {lp, lp};     // [0]: left, [1]: right
       float lpm = lp;
       uint32_t n = 1;
@@ -233,92 +192,163 @@ __global__ void __launch_bounds__(32 * kWarps, NB == 1 ? 7 : 4) k_nuts(NutsArgs 
         bool ok_sub = true;
         float lps = 0.f;
         const int leaves = 1 << jd;
-        uint4 wsub4 = make_uint4(0u, 0u, 0u, 0u);
-        for (int k = 0; k < leaves; ++k) {
-          // the subtree-choice words depend on nothing the leaves compute:
-          // drawn first, four at a time, the generator's arithmetic fills the
-          // butterfly's latency
-          if ((k & 3) == 0)
-            wsub4 = philox(make_uint4(static_cast<uint32_t>(k >> 2), chain, t, kNutsTagSubtree + jd),
-                           static_cast<uint32_t>(a.seed), static_cast<uint32_t>(a.seed >> 32));
-          const int kq = k & 3;
-          const uint32_t wsub = kq == 0 ? wsub4.x : kq == 1 ? wsub4.y : kq == 2 ? wsub4.z : wsub4.w;
-          // spans of 2^i leaves closing at leaf k (2^i | k + 1); the span of
-          // two leaves (i = 1) is tested inside the leaf's butterfly
-          const int close = min(jd, __ffs(k + 1) - 1);
-          float xf[NB][4], pf[NB][4];
+        // the first leaf's position: half a kick, the drift; its sum of squares
+        const float sv = static_cast<float>(v);
+        float v0 = lane0(x), p0 = lane0(p), g0 = lane0(g), q = 0.f;
+        p0 = fmaf(hv, g0, p0);
+        v0 = fmaf(ev, p0, v0);
 #pragma unroll
-          for (int b = 0; b < NB; ++b) {
-            xf[b][0] = xf[b][1] = xf[b][2] = xf[b][3] = 0.f;
-            pf[b][0] = pf[b][1] = pf[b][2] = pf[b][3] = 0.f;
-            if (close >= 1 && in_slot(b)) {
-              get(span4(0, b), xf, b);
-              get(span4(1, b), pf, b);
-            }
+        for (int b = 0; b < NB; ++b)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            p[b][i] = fmaf(hv, g[b][i], p[b][i]);
+            x[b][i] = fmaf(ev, p[b][i], x[b][i]);
+            if (!is_v(b, i)) q = fmaf(x[b][i], x[b][i], q);
           }
-          // one leapfrog step of step v eps
+        float em = expf(-v0);
+        q = warp_sum(q);
+        // first leaf of the span of two leaves in progress
+        float xf[NB][4], pf[NB][4];
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) xf[b][i] = pf[b][i] = 0.f;
+        float xf0 = 0.f, pf0 = 0.f;
+        // the subtree-choice words of 128 leaves at a time, four per lane
+        auto words = [&](int k) {
+          return philox(make_uint4(static_cast<uint32_t>((k >> 2) + lane), chain, t, kNutsTagSubtree + jd),
+                        static_cast<uint32_t>(a.seed), static_cast<uint32_t>(a.seed >> 32));
+        };
+        uint4 wsub4 = words(0);
+        int k = 0;
+        for (;;) {
+          const int kq = k & 3;
+          const uint32_t wsub = __shfl_sync(0xffffffffu, kq == 0 ? wsub4.x : kq == 1 ? wsub4.y : kq == 2 ? wsub4.z : wsub4.w,
+                                            (k >> 2) & 31);
+          // the gradient at the drifted x, whose sum of squares is known, and the
+          // second half kick
+          if (TARGET == HMC_T_FUNNEL) g0 = v0 * (-1.f / 9.f) - half_n + 0.5f * em * q;
+          const float p0n = fmaf(hv, g0, p0);
+          lp = TARGET == HMC_T_FUNNEL ? v0 * v0 * (-1.f / 18.f) - half_n * v0 - 0.5f * em * q : -0.5f * q;
+          if (!kKeepFirst && (k & 1)) {
+            const int o = k == 1 ? jd : __ffs(k - 1) - 1;
+#pragma unroll
+            for (int b = 0; b < NB; ++b)
+              if (in_slot(b)) {
+                get(span4(2 * (o - 1), b), xf, b);
+                get(span4(2 * (o - 1) + 1, b), pf, b);
+              }
+          }
+          // |p|^2, the next leaf's sum of squares and, for the span of two leaves
+          // that closes at an odd one, its U-turn dot products dx . pf and
+          // dx . p, dx = sv (x - xf) against its first leaf (xf, pf)
+          float xn[NB][4], pn[NB][4], pp = 0.f, qn = 0.f, d1 = 0.f, d2 = 0.f;
 #pragma unroll
           for (int b = 0; b < NB; ++b)
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
+              g[b][i] = is_v(b, i) ? g0 : TARGET == HMC_T_FUNNEL ? -em * x[b][i] : -x[b][i];
               p[b][i] = fmaf(hv, g[b][i], p[b][i]);
-              x[b][i] = fmaf(ev, p[b][i], x[b][i]);
+              pn[b][i] = fmaf(hv, g[b][i], p[b][i]);
+              xn[b][i] = fmaf(ev, pn[b][i], x[b][i]);
+              if (!is_v(b, i)) {
+                pp = fmaf(p[b][i], p[b][i], pp);
+                qn = fmaf(xn[b][i], xn[b][i], qn);
+                const float dx = sv * (x[b][i] - xf[b][i]);
+                d1 = fmaf(dx, pf[b][i], d1);
+                d2 = fmaf(dx, p[b][i], d2);
+              }
             }
-          float H;
-          bool turn;
-          lp = leaf_sums(hv, static_cast<float>(v), close >= 1, xf, pf, &H, &turn);
+          const float p0h = fmaf(hv, g0, p0n), v0n = fmaf(ev, p0h, v0);
+          em = expf(-v0n);
+          warp_sum4(qn, pp, d1, d2);
+          if (TARGET == HMC_T_FUNNEL) {
+            const float dx0 = sv * (v0 - xf0);
+            d1 = fmaf(dx0, pf0, d1);
+            d2 = fmaf(dx0, p0n, d2);
+          }
+          const float H = -lp + 0.5f * (TARGET == HMC_T_FUNNEL ? fmaf(p0n, p0n, pp) : pp);
           const bool finite = isfinite(H);
-          if (!finite || H - H0 >= kNutsDeltaMax - logU) ok_sub = false;     // divergence
-          a_sum += finite ? accept_prob(H0 - H) : 0.f;
-          ++n_a;
-          if (finite && logU <= H0 - H) {
-            ++n_sub;
-            if (nuts_take(wsub, 1u, n_sub)) {
-              store(kSlotSub, x);
-              store(kSlotSub + 1, g);
-              lps = lp;
-            }
+          // U-turn, divergence
+          ok_sub = !((k & 1) && (d1 < 0.f || d2 < 0.f)) && finite && !(H - H0 >= kNutsDeltaMax - logU);
+          const float pr = accept_prob(H0 - H);
+          a_sum += finite ? pr : 0.f;
+          const bool valid = finite && logU <= H0 - H;
+          n_sub += valid;
+          if (valid && nuts_take(wsub, 1u, n_sub)) {
+            store(sub, x);
+            store(sub + 1, g);
+            lps = lp;
           }
-          if (turn) ok_sub = false;
-          // spans of 2^i leaves opening at leaf k (2^i | k); no span both
-          // opens and closes at one leaf
-          const int open = k == 0 ? jd : min(jd, __ffs(k) - 1);
-          for (int i = 1; i <= open; ++i) {
+          // an even leaf opens spans of 2^i leaves for every i with 2^i | k: kept
+          // once, in the row of the largest (no other leaf of that row comes
+          // before they close)
+          if (!(k & 1) && jd) {
+            const int o = k ? __ffs(k) - 1 : jd;
 #pragma unroll
             for (int b = 0; b < NB; ++b)
               if (in_slot(b)) {
-                put(span4(2 * (i - 1), b), x, b);
-                put(span4(2 * (i - 1) + 1, b), p, b);
+                put(span4(2 * (o - 1), b), x, b);
+                put(span4(2 * (o - 1) + 1, b), p, b);
               }
           }
-          for (int i = 2; i <= close && ok_sub; ++i) {
-            float dx[NB][4], pg[NB][4];
+          // longer spans that close here (2^i | k + 1)
+          if ((k & 3) == 3) {
+            const int close = __ffs(k + 1) - 1;
+            for (int i = 2; i <= close && ok_sub; ++i) {
+              const int first = k + 1 - (1 << i), o = first ? __ffs(first) - 1 : jd;
+              float dx[NB][4], pg[NB][4];
 #pragma unroll
-            for (int b = 0; b < NB; ++b) {
-              dx[b][0] = dx[b][1] = dx[b][2] = dx[b][3] = 0.f;
-              pg[b][0] = pg[b][1] = pg[b][2] = pg[b][3] = 0.f;
-              if (in_slot(b)) {
-                get(span4(2 * (i - 1), b), dx, b);
-                get(span4(2 * (i - 1) + 1, b), pg, b);
+              for (int b = 0; b < NB; ++b) {
+                dx[b][0] = dx[b][1] = dx[b][2] = dx[b][3] = 0.f;
+                pg[b][0] = pg[b][1] = pg[b][2] = pg[b][3] = 0.f;
+                if (in_slot(b)) {
+                  get(span4(2 * (o - 1), b), dx, b);
+                  get(span4(2 * (o - 1) + 1, b), pg, b);
+                }
+              }
+#pragma unroll
+              for (int b = 0; b < NB; ++b)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) dx[b][e] = sv * (x[b][e] - dx[b][e]);
+              if (u_turn(dx, pg, p)) ok_sub = false;
+            }
+          }
+          if (++k == leaves || !ok_sub) break;
+          // on to the next leaf (k is its number)
+          float hv2 = hv, ev2 = ev;
+          if (!kKeepNext) asm volatile("" : "+f"(hv2), "+f"(ev2));
+#pragma unroll
+          for (int b = 0; b < NB; ++b)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              if (kKeepFirst) {
+                xf[b][i] = k & 1 ? x[b][i] : xf[b][i];
+                pf[b][i] = k & 1 ? p[b][i] : pf[b][i];
+              }
+              if (kKeepNext) {
+                x[b][i] = xn[b][i];
+                p[b][i] = pn[b][i];
+              } else {          // formed again: held over the decisions they cost registers
+                p[b][i] = fmaf(hv2, g[b][i], p[b][i]);
+                x[b][i] = fmaf(ev2, p[b][i], x[b][i]);
               }
             }
-#pragma unroll
-            for (int b = 0; b < NB; ++b)
-#pragma unroll
-              for (int q = 0; q < 4; ++q) dx[b][q] = static_cast<float>(v) * (x[b][q] - dx[b][q]);
-            if (u_turn(dx, pg, p)) ok_sub = false;
-          }
-          if (!ok_sub) break;
+          xf0 = k & 1 ? v0 : xf0;
+          pf0 = k & 1 ? p0n : pf0;
+          v0 = v0n;
+          p0 = p0h;
+          q = qn;
+          if (__builtin_expect((k & 127) == 0, 0)) wsub4 = words(k);
         }
+        n_a += k;
+        if (!ok_sub) break;
         store(side, x); store(side + 1, p); store(side + 2, g);
         lp_end[v > 0 ? 1 : 0] = lp;
-        if (!ok_sub) break;
         if (n_sub > 0 && nuts_take(nuts_word0(a.seed, static_cast<uint32_t>(jd), chain, t, kNutsTagTop), n_sub, n)) {
-          float t1[NB][4], t2[NB][4];
-          load(kSlotSub, t1);
-          load(kSlotSub + 1, t2);
-          store(kSlotCand, t1);
-          store(kSlotCand + 1, t2);
+          const int was = cand;
+          cand = sub;
+          sub = was;
           lpm = lps;
           moved = 1;
         }
@@ -334,8 +364,8 @@ __global__ void __launch_bounds__(32 * kWarps, NB == 1 ? 7 : 4) k_nuts(NutsArgs 
         if (u_turn(xr, pl, pr)) break;
       }
       // the new state
-      load(kSlotCand, x);
-      load(kSlotCand + 1, g);
+      load(cand, x);
+      load(cand + 1, g);
       lp = lpm;
       prob = a_sum / static_cast<float>(n_a);
       leaves_total += n_a;
@@ -386,19 +416,28 @@ __global__ void __launch_bounds__(32 * kWarps, NB == 1 ? 7 : 4) k_nuts(NutsArgs 
   }
 }
 
-template <int TARGET, int NB, bool SMEM>
+template <int TARGET, int NB, bool SMEM, bool WIDE>
 cudaError_t launch_v(const NutsArgs& na, size_t smem, cudaStream_t s) {
   const unsigned grid = nuts_grid(na.s.C);
-  k_nuts<TARGET, NB, SMEM><<<grid, 32 * kWarps, SMEM ? smem : 0, s>>>(na);
+  k_nuts<TARGET, NB, SMEM, WIDE><<<grid, 32 * kWarps, SMEM ? smem : 0, s>>>(na);
   count_launch();
   return cudaGetLastError();
+}
+
+// resident blocks per SM with the span starts in scratch and in shared memory
+// (0: they do not fit)
+template <int TARGET, int NB, bool WIDE>
+cudaError_t residency(size_t smem, int* glob, int* shared) {
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(glob, k_nuts<TARGET, NB, false, WIDE>, 32 * kWarps, 0);
+  *shared = 0;
+  if (e == cudaSuccess && smem > 0 && smem <= kNutsSpanSmemMax)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(shared, k_nuts<TARGET, NB, true, WIDE>, 32 * kWarps, smem);
+  return e;
 }
 
 template <int TARGET, int NB>
 cudaError_t launch_nb(const NutsArgs& na, cudaStream_t s) {
   const size_t smem = span_smem_bytes(na.Dp, na.max_depth);
-  // shared-memory span starts unless they cost resident chains: as many
-  // blocks per SM as the scratch form, or enough for every chain
   static int sms = 0;
   if (!sms) {
     int dev = 0;
@@ -406,17 +445,21 @@ cudaError_t launch_nb(const NutsArgs& na, cudaStream_t s) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       return cudaErrorUnknown;
   }
-  int occ_smem = 0, occ_glob = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &occ_glob, k_nuts<TARGET, NB, false>, 32 * kWarps, 0);
-  if (e == cudaSuccess && smem <= kNutsSpanSmemMax)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_smem, k_nuts<TARGET, NB, true>,
-                                                      32 * kWarps, smem);
+  auto fit = [&](int blocks) { return static_cast<int64_t>(blocks) * kWarps * sms >= na.s.C; };
+  int glob = 0, shared = 0;
+  cudaError_t e = residency<TARGET, NB, true>(smem, &glob, &shared);
   if (e != cudaSuccess) return e;
-  const bool use_smem = smem > 0 && occ_smem > 0 &&
-                        (occ_smem >= occ_glob ||
-                         static_cast<int64_t>(occ_smem) * kWarps * sms >= na.s.C);
-  return use_smem ? launch_v<TARGET, NB, true>(na, smem, s) : launch_v<TARGET, NB, false>(na, 0, s);
+  // the wide form where all its chains are resident at once: 1024 x 100 funnel
+  // 832 us for 20 transitions (837 at 5 blocks), 1000 x 500 1605 against 1813,
+  // but 2000 x 200 standard normal 362 us against 262, in two waves
+  if (fit(shared)) return launch_v<TARGET, NB, true, true>(na, smem, s);
+  const bool wide = fit(glob);
+  e = residency<TARGET, NB, false>(smem, &glob, &shared);
+  if (e != cudaSuccess) return e;
+  // shared-memory span starts unless they cost resident chains: as many
+  // blocks per SM as the scratch form, or enough for every chain
+  if (shared > 0 && (shared >= glob || fit(shared))) return launch_v<TARGET, NB, true, false>(na, smem, s);
+  return wide ? launch_v<TARGET, NB, false, true>(na, 0, s) : launch_v<TARGET, NB, false, false>(na, 0, s);
 }
 
 template <int TARGET>
@@ -429,8 +472,11 @@ cudaError_t launch_t(const NutsArgs& na, cudaStream_t s) {
 
 template <int TARGET, int NB>
 cudaError_t allow_smem() {
-  return cudaFuncSetAttribute(k_nuts<TARGET, NB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(kNutsSpanSmemMax));
+  const cudaError_t e = cudaFuncSetAttribute(k_nuts<TARGET, NB, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             static_cast<int>(kNutsSpanSmemMax));
+  return e != cudaSuccess ? e
+                          : cudaFuncSetAttribute(k_nuts<TARGET, NB, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 static_cast<int>(kNutsSpanSmemMax));
 }
 
 }  // namespace
