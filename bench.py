@@ -677,8 +677,9 @@ def main():
                     "peak_source": f"derived: {SM_COUNT} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x {sm_max:.0f} MHz",
                     **common}
         else:
-            # fused elementwise transition: x and g read and written once per chain row
-            bytes_per_launch = 4.0 * 4 * C * D
+            # elementwise transitions, a range per launch: x and g read and written once,
+            # one kept sample written per transition
+            bytes_per_launch = 4.0 * C * D * (4 + evals_per_launch / (C * p.num_leapfrog))
             achieved = bytes_per_launch / kernel_s / 1e9
             roof = {"bound": "hbm", "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s",
                     "frac": achieved / pk["hbm_gbs"], "traffic": None,

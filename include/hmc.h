@@ -86,8 +86,10 @@ typedef enum {
                                      (whatever its size) */
   HMC_IMPL_FUSED_SIMT = 4         /* as FUSED, but a logistic regression
                                      always takes the shared-memory SIMT
-                                     transition (dim <= 512; 8 chains per
-                                     CTA tile) */
+                                     transition (dim <= 512; the whole chain
+                                     in one or two launches where the data
+                                     fits shared memory, else 8 chains per
+                                     CTA tile, a launch per transition) */
 } hmc_impl;
 
 /* Inner (uncalibrated) kernel of the Metropolis-Hastings composition,
@@ -111,9 +113,10 @@ typedef enum {
                                     tree independent; CORR_GAUSS and LOGREG: the
                                     chains advance in lockstep, one leaf per
                                     iteration (tensor-core gradient products of
-                                    the chains still building, then one leaf
-                                    kernel), the iterations a conditional node
-                                    of a CUDA graph: a call that enqueues
+                                    the chains still building, then their
+                                    leaves), the iterations inside one launch
+                                    (CORR_GAUSS) or a conditional node of a
+                                    CUDA graph (LOGREG): a call that enqueues
                                     transitions on a stream that is not
                                     capturing captures them on the context's
                                     private stream and launches the graph; the
@@ -141,12 +144,15 @@ typedef struct {
                                replays it while its pointer and count
                                arguments stay the same; 0: plain launches */
   int32_t max_transitions_per_launch;
-                            /* dense Gaussian on CTA pairs: hmc_sample_chain
-                               runs at most this many transitions per kernel
-                               launch (>= 0; 0: no limit, the whole chain in
-                               one cooperative launch; 1: one launch per
-                               transition, e.g. for a profiler that cannot
-                               replay cooperative cluster launches) */
+                            /* dense Gaussians of dim <= 256, elementwise
+                               targets and small logistic regressions:
+                               hmc_sample_chain runs at most this many
+                               transitions per kernel launch (>= 0; 0: no
+                               limit, the whole chain in one launch, or in one
+                               while the step size adapts and one after; 1:
+                               one launch per transition, e.g. for a profiler
+                               that cannot replay cooperative cluster
+                               launches).  Results do not depend on it */
   int32_t proposal;         /* hmc_proposal_kind: the inner kernel of the
                                Metropolis-Hastings composition (Section 4.1) */
 } hmc_config;
@@ -528,7 +534,8 @@ hmc_status hmc_target_vjp_workspace_bytes(const hmc_target* target, int64_t num_
  * autograd binding; the paper obtains gradients by automatic differentiation,
  * Section 3 and its footnote on TF autodiff): dx[c, :] = w[c] * grad log p(x_c)
  * for x, dx [chains x dim] and w [chains] (device, caller-owned).  The forward
- * pass is recomputed, nothing from it is stored.  `workspace` (device,
+ * pass is recomputed, nothing from it is stored; a caller that kept its
+ * gradient calls hmc_target_vjp_from_grad instead.  `workspace` (device,
  * 256-byte aligned, >= hmc_target_vjp_workspace_bytes) is caller-owned.
  * HMC_E_INVALID on bad sizes, pointers or workspace. */
 hmc_status hmc_target_vjp(const hmc_target* target, int64_t num_chains, const float* x,

@@ -1336,6 +1336,7 @@ hmc_status hmc_dominant_kernel_info(const hmc_ctx* ctx, char* name, int32_t name
     per = ctx->C * ctx->cfg.num_leapfrog;
   } else if (ctx->use_tc) {
     n = "k_gauss_tc_step";
+    if (ctx->tc.traj) per = ctx->C * ctx->cfg.num_leapfrog;   // all steps in one launch
   } else if (ctx->use_lrtc) {
     n = "k_lr_grad";
   } else if (ctx->use_lrgemm) {

@@ -1,5 +1,5 @@
 // HMC transitions for the dense Gaussian target (dim <= 256) on CTA pairs
-// (tcgen05 cta_group::2).  A pair owns 64 chains; one launch runs T
+// (tcgen05 cta_group::2), and on single CTAs for dim <= 128 (k_gauss_one, below).  A pair owns 64 chains; one launch runs T
 // consecutive transitions of them (Section 2.1's transition, Section 4.2's
 // driver loop), so that P stays resident across transitions and no launch
 // sits between them.  Each leapfrog gradient G^T = P X^T (3xTF32) is one

@@ -1,11 +1,13 @@
-// Dense Gaussian target on the tcgen05 tensor cores: each leapfrog step is
-// one launch that computes a 128-chain x 64-column tile of the gradient
+// Dense Gaussian target on the tcgen05 tensor cores: each leapfrog step
+// computes a 128-chain x 64-column tile of the gradient
 // G = -X P (a C x D x D product, Section 2.1's batched "list of vectors"
 // evaluation) in 3xTF32 -- A_lo B_hi + A_hi B_lo + A_hi B_hi, float32
 // accumulation in tensor memory -- and applies the leapfrog update to the
 // same tile in its epilogue, so the gradient never goes to HBM.
 //
-// A transition (identity mass, step eps, L steps) is L + 2 launches:
+// A transition (identity mass, step eps, L steps) is begin, L steps and accept.
+// The steps are one cooperative launch where all their tiles are resident at
+// once (k_gauss_tc_traj), else one launch each (k_gauss_tc_step):
 //   begin:  p0 ~ N(0, I); H0 = -lp(x0) + |p0|^2/2; p = p0 + eps/2 g(x0);
 //           x1 = x0 + eps p                          (cached g(x0) reused)
 //   step l = 1 .. L-1:  g = -x_l P;  p += eps g;  x_{l+1} = x_l + eps p

@@ -1,5 +1,6 @@
 // One launch per HMC transition for Bayesian logistic regression: the tile
-// function in logreg_tile.cuh, one CTA per tile of chains.
+// function in logreg_tile.cuh, one CTA per tile of chains.  Taken where the data
+// does not fit shared memory beside a chain (logreg_chain.cu).
 #include "logreg_tile.cuh"
 
 namespace hmc {

@@ -1,5 +1,6 @@
-// Fused HMC transition for Bayesian logistic regression as a tile function
-// (Section 2.1's transition with the batched target of a "list of vectors"):
+// Fused HMC transition for Bayesian logistic regression as a tile function, for
+// the batch's grouped launch and for data that does not fit shared memory
+// (logreg_chain.cu has the rest, sum by sum the same) (Section 2.1's transition with the batched target of a "list of vectors"):
 // one CTA owns kLrTC chains for the whole transition -- momentum draw, L
 // leapfrog steps, Metropolis-Hastings select -- with positions, momenta and
 // gradients in shared memory.  Each gradient streams the data X in tiles of
