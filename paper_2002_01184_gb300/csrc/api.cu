@@ -377,12 +377,12 @@ bool uses_logreg_chain(const hmc_ctx* ctx) {
 
 // T transitions in one launch, either kind
 cudaError_t launch_chain(hmc_ctx* ctx, const StepArgs& a, bool adapting, int T, long long keep_from, float* samples,
-                         float* trace_eps, uint8_t* trace_acc) {
+                         float* trace_eps, uint8_t* trace_acc, hmc::KernelTimer* timer) {
   return uses_fused_elementwise(ctx)
              ? hmc::launch_elementwise_chain(ctx->target.id, a, adapting, T, keep_from, samples, trace_eps, trace_acc,
-                                             ctx->chain_sync, ctx->stream, &ctx->timer)
+                                             ctx->chain_sync, ctx->stream, timer)
              : hmc::launch_logreg_chain(ctx->target, a, adapting, T, keep_from, samples, trace_eps, trace_acc,
-                                        ctx->chain_sync, ctx->stream, &ctx->timer);
+                                        ctx->chain_sync, ctx->stream, timer);
 }
 
 StepArgs make_args(hmc_ctx* ctx, float* x, uint64_t t) {
@@ -419,7 +419,7 @@ cudaError_t enqueue_transition(hmc_ctx* ctx, const StepArgs& a) {
     return hmc::launch_logreg_tc_transition(a, ctx->lrtc, ctx->lr_err, ctx->stream, &ctx->timer);
   if (ctx->use_lrgemm) return hmc::launch_logreg_gemm_transition(a, ctx->lrg, ctx->stream, &ctx->timer);
   if (uses_fused_elementwise(ctx) || uses_logreg_chain(ctx))
-    return launch_chain(ctx, a, false, 1, a.t_full, a.sample_out, a.trace_eps, a.trace_acc);
+    return launch_chain(ctx, a, false, 1, a.t_full, a.sample_out, a.trace_eps, a.trace_acc, &ctx->timer);
   if (uses_fused_logreg(ctx))
     return hmc::launch_logreg_fused_transition(ctx->target, a, ctx->stream, &ctx->timer);
   return hmc::launch_plain_transition(ctx->target, a, ctx->plain, ctx->grad_ws, ctx->stream,
@@ -554,7 +554,9 @@ hmc_status enqueue_range(hmc_ctx* ctx, float* x, int64_t B, int64_t t_begin, int
       StepArgs a = make_args(ctx, x, static_cast<uint64_t>(t0));
       if (ctx->s_mean && t0 + n > B)
         a.w = hmc::WelfordOut{ctx->s_mean, ctx->s_m2, ctx->s_bsize, ctx->bm_sum, ctx->bm_mean, ctx->bm_m2};
-      cudaError_t e = launch_chain(ctx, a, t0 < t_fixed, n, B + out0, samples, trace_eps, trace_acc);
+      // (the kernel timer takes the kind of launch that ends the chain)
+      cudaError_t e = launch_chain(ctx, a, t0 < t_fixed, n, B + out0, samples, trace_eps, trace_acc,
+                                   stop == t_end ? &ctx->timer : nullptr);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "chain launch");
       t0 += n;
     }
