@@ -1243,7 +1243,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   __shared__ uint64_t acc_full[1], own_full[1];
   __shared__ uint32_t tmem_slot[4];
-  __shared__ float red[2][4][kHalf], kin_s[2][4][kHalf], lu_s[2][kHalf];
+  // |p0|^2 of transition j at j % 3: with one leapfrog step a warp may write
+  // transition j + 1's while another still decides j - 1 (the accumulator that
+  // every thread's positions of j lead to is the only meeting between them)
+  __shared__ float red[2][4][kHalf], kin_s[3][4][kHalf], lu_s[2][kHalf];
   __shared__ DAState da_s;
   __shared__ DACoef coef_s;
   __shared__ unsigned long long psum_s;
@@ -1338,7 +1341,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
     };
     // |p0|^2 of the warp's 16 chains over its 32 dims, in the pair's order:
     // the butterfly's first step in full, then halving
-    auto kinetic = [&](const float (&z)[16], uint32_t tn) {
+    auto kinetic = [&](const float (&z)[16], int j) {
       float v[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) v[i] = z[i] * z[i];
@@ -1354,7 +1357,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
           v[k] = keep + __shfl_xor_sync(0xffffffffu, send, w);
         }
       }
-      if (lane < 16) kin_s[tn & 1u][quarter][16 * sub + lane] = v[0];
+      if (lane < 16) kin_s[j % 3][quarter][16 * sub + lane] = v[0];
     };
     // momenta of slots 4 g .. 4 g + 3 at transition tn
     auto draw = [&](float (&z)[16], int g0, int g1, uint32_t tn) {
@@ -1404,7 +1407,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
       }
     }
     draw(z, 0, 4, a.t);
-    kinetic(z, a.t);
+    kinetic(z, 0);
     // lane c of every warp decides chain c0 + c (the same inputs, the same answer)
     const int chain = c0 + lane;
     float lpc = chain < C ? a.lp[chain] : 0.f;
@@ -1440,7 +1443,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
       }
       if (more) {
         draw(zn, (L - 1) * per_wait, 4, t + 1);
-        kinetic(zn, t + 1);
+        kinetic(zn, j + 1);
       }
       wait_acc(s0 + L - 1);
       load_acc(acc);
@@ -1469,7 +1472,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
         for (int q = 0; q < 4; ++q) {
           xg += red[0][q][lane];
           pp += red[1][q][lane];
-          k0 += kin_s[t & 1u][q][lane];
+          k0 += kin_s[j % 3][q][lane];
         }
         const float kin0 = 0.5f * k0, lp1 = 0.5f * xg;
         la = (-lpc + kin0) - (-lp1 + 0.5f * pp);
