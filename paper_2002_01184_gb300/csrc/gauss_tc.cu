@@ -112,13 +112,7 @@ struct TcStepArgs {
   const uint8_t* active;    // null, or per-chain flags: a tile with none set is skipped
 };
 
-// Clusters of CM x CN tiles (CM chain blocks, CN column blocks): tiles of one
-// chain block read the same A, tiles of one column block the same B, so each CTA
-// loads its share of the rows of both and multicasts it to the others.  What
-// bounds these products without it is L2: a 128 x 64 tile takes 48 KB per 12
-// MMAs (0.28 us).  A stage is refilled once every CTA that gets this one's rows has
-// consumed it: the MMA issuer's commit arrives at all senders' barriers.
-template <int EPI, int BN = kBN, int ST = Tile<BN>::kStages, int CM = 1, int CN = 1>
+template <int EPI, int BN = kBN, int ST = Tile<BN>::kStages>
 __global__ void __launch_bounds__(kThreads, Tile<BN, ST>::kCtasPerSm)
 k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant__ CUtensorMap mAlo,
                 const __grid_constant__ CUtensorMap mBhi, const __grid_constant__ CUtensorMap mBlo,
@@ -138,15 +132,7 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
-  constexpr bool kCluster = CM * CN > 1;
-  // place in the cluster (grid x: chain blocks, y: column blocks)
-  const int cm = CM > 1 ? static_cast<int>(blockIdx.x) % CM : 0, cn = CN > 1 ? static_cast<int>(blockIdx.y) % CN : 0;
-  uint16_t row_mask = 0, col_mask = 0;      // the tiles that share this one's A, B
-  if (kCluster) {
-    for (int j = 0; j < CN; ++j) row_mask |= static_cast<uint16_t>(1u << (cm + CM * j));
-    for (int i = 0; i < CM; ++i) col_mask |= static_cast<uint16_t>(1u << (i + CM * cn));
-  }
-  if (!kCluster && a.active) {
+  if (a.active) {
     // NUTS: a tile whose chains have all finished their trees has no work
     const int r = threadIdx.x;
     const bool mine = r < kBM && m0 + r < a.C && a.active[m0 + r] != 0;
@@ -159,7 +145,7 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       ptx::mbar_init(&full[s], 1);
-      ptx::mbar_init(&empty[s], CM + CN - 1);
+      ptx::mbar_init(&empty[s], 1);
     }
     ptx::mbar_init(acc_full, 1);
     ptx::fence_mbar_init();
@@ -173,9 +159,7 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
-  __syncwarp();
-  if (kCluster) ptx::cluster_sync();      // the peers' barriers exist before anything is sent
-  else __syncthreads();
+  __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   ptx::grid_dependents_launch();
@@ -185,26 +169,13 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
     // ---- TMA producer
     for (int kc = 0; kc < nk; ++kc) {
       const int s = kc % kStages, round = kc / kStages;
-      if (kc >= kStages &&
-          !(kCluster ? ptx::mbar_wait_cluster(&empty[s], (round - 1) & 1) : ptx::mbar_wait(&empty[s], (round - 1) & 1))) {
+      if (kc >= kStages && !ptx::mbar_wait(&empty[s], (round - 1) & 1)) {
         atomicExch(a.err, 1);
         break;
       }
       uint8_t* st = smem + s * kStageBytes;
       ptx::mbar_arrive_expect_tx(&full[s], kStageBytes);
       const int kx = (kc0 + kc) * kBK;
-      if (kCluster) {
-        // this CTA's share: 128 / CN rows of A, BN / CM rows of B
-        constexpr int kRowsA = kBM / CN, kRowsB = BN / CM;
-        static_assert(kRowsA % 8 == 0 && kRowsB % 8 == 0, "whole swizzle atoms");
-        uint8_t* sa = st + cn * kRowsA * 128;
-        uint8_t* sb = st + 2 * kABytes + cm * kRowsB * 128;
-        ptx::tma_load_2d_multicast(sa, &mAhi, &full[s], kx, m0 + cn * kRowsA, row_mask);
-        ptx::tma_load_2d_multicast(sa + kABytes, &mAlo, &full[s], kx, m0 + cn * kRowsA, row_mask);
-        ptx::tma_load_2d_multicast(sb, &mBhi, &full[s], kx, n0 + cm * kRowsB, col_mask);
-        ptx::tma_load_2d_multicast(sb + kBBytes, &mBlo, &full[s], kx, n0 + cm * kRowsB, col_mask);
-        continue;
-      }
       ptx::tma_load_2d(st, &mAhi, &full[s], kx, m0);
       ptx::tma_load_2d(st + kABytes, &mAlo, &full[s], kx, m0);
       ptx::tma_load_2d(st + 2 * kABytes, &mBhi, &full[s], kx, n0);
@@ -231,10 +202,7 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
         ptx::mma_tf32(tmem, a_hi, b_lo, idesc, 1u);
         ptx::mma_tf32(tmem, a_hi, b_hi, idesc, 1u);
       }
-      // (the last stages are not refilled: no arrival may be on its way to a
-      // peer that has left)
-      if (!kCluster) ptx::mma_commit(&empty[s]);
-      else if (kc + kStages < nk) ptx::mma_commit_multicast(&empty[s], row_mask | col_mask);
+      ptx::mma_commit(&empty[s]);
     }
     ptx::mma_commit(acc_full);
   } else if (warp >= 2) {
@@ -346,15 +314,12 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
         // Gaussian: log p = <x, g> / 2; logistic regression: the rows'
         // log-likelihood terms, or the prior's -|theta|^2 / 2
         const float v = EPI == kEpiLrResid ? part : 0.5f * part;
-        // (a cluster's last column blocks may lie past the columns)
-        if (lane == 0 && n0 < a.ncols) a.lp_part[static_cast<int64_t>(m) * a.ntn + a.lp_col0 + blockIdx.y] = v;
+        if (lane == 0) a.lp_part[static_cast<int64_t>(m) * a.ntn + a.lp_col0 + blockIdx.y] = v;
       }
     }
   }
   ptx::tc_fence_before();
-  __syncwarp();
-  if (kCluster) ptx::cluster_sync();      // no CTA leaves while a peer's loads or arrivals may still reach it
-  else __syncthreads();
+  __syncthreads();
   if (warp == 0) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, kTmemCols);
@@ -371,9 +336,10 @@ k_gauss_tc_step(const __grid_constant__ CUtensorMap mAhi, const __grid_constant_
 // them -- the next stages' rows of P, which never change, are on their way by
 // then.  Arithmetic, and the order of every sum, are k_gauss_tc_step's.
 // Measured, per step of 16 with begin and accept: 2048 chains x 512 dims 17.7 ->
-// 13.7 us, 2048 x 300 16.5 -> 10.6 us, 64 x 512 14.7 -> 13.0 us.  What bounds it
+// 13.4 us, 2048 x 300 16.6 -> 10.3 us, 64 x 512 14.7 -> 12.2 us.  What bounds it
 // now is shared memory: 32 dims of a 128 x 64 tile bring 48 KB and their 12 MMAs
-// read 72 KB, 0.46 us at 128 bytes a cycle, 7.4 us for 512 dims.
+// read 72 KB, 0.46 us at 128 bytes a cycle, 7.4 us for 512 dims.  (Clusters of
+// 2 x 2 tiles that shared their loads by multicast took 13.7 and 10.6 us.)
 struct TcTrajArgs {
   int C, D, L, ntn;
   float* xhi[2];            // x_l at [(l - 1) & 1], row length D
@@ -386,7 +352,6 @@ struct TcTrajArgs {
   int* err;
 };
 
-template <int CM, int CN>
 __global__ void __launch_bounds__(kThreads, 1)
 k_gauss_tc_traj(const __grid_constant__ CUtensorMap mAhi0, const __grid_constant__ CUtensorMap mAlo0,
                 const __grid_constant__ CUtensorMap mAhi1, const __grid_constant__ CUtensorMap mAlo1,
@@ -396,7 +361,6 @@ k_gauss_tc_traj(const __grid_constant__ CUtensorMap mAhi0, const __grid_constant
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   using T = Tile<kTrajBN, kTrajStages>;
   constexpr int BN = kTrajBN, kStages = kTrajStages;
-  constexpr bool kCluster = CM * CN > 1;
   float* stg = reinterpret_cast<float*>(smem + kStages * T::kStageBytes);     // [kBM][BN + 1]
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * T::kStageBytes + kTrajStgBytes);
   uint64_t* empty = full + kStages;
@@ -404,15 +368,11 @@ k_gauss_tc_traj(const __grid_constant__ CUtensorMap mAhi0, const __grid_constant
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
-  const int cm = CM > 1 ? static_cast<int>(blockIdx.x) % CM : 0, cn = CN > 1 ? static_cast<int>(blockIdx.y) % CN : 0;
-  uint16_t row_mask = 0, col_mask = 0;
-  for (int j = 0; j < CN; ++j) row_mask |= static_cast<uint16_t>(1u << (cm + CM * j));
-  for (int i = 0; i < CM; ++i) col_mask |= static_cast<uint16_t>(1u << (i + CM * cn));
   const int nk = (a.D + kBK - 1) / kBK;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       ptx::mbar_init(&full[s], 1);
-      ptx::mbar_init(&empty[s], CM + CN - 1);
+      ptx::mbar_init(&empty[s], 1);
     }
     ptx::mbar_init(acc_full, 1);
     ptx::fence_mbar_init();
@@ -428,41 +388,32 @@ k_gauss_tc_traj(const __grid_constant__ CUtensorMap mAhi0, const __grid_constant
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
-  __syncwarp();
-  if (kCluster) ptx::cluster_sync();
-  else __syncthreads();
+  __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer
-    constexpr int kRowsA = kBM / CN, kRowsB = BN / CM;
-    static_assert(kRowsA % 8 == 0 && kRowsB % 8 == 0, "whole swizzle atoms");
     bool ok = true;
-    auto load = [&](const CUtensorMap* map, uint8_t* dst, int s, int k, int r, uint16_t mask) {
-      if (kCluster) ptx::tma_load_2d_multicast(dst, map, &full[s], k, r, mask);
-      else ptx::tma_load_2d(dst, map, &full[s], k, r);
-    };
     auto arm_and_load_b = [&](int it, int kc) {
       const int s = it % kStages, round = it / kStages;
-      if (it >= kStages && !(kCluster ? ptx::mbar_wait_cluster(&empty[s], (round - 1) & 1)
-                                      : ptx::mbar_wait(&empty[s], (round - 1) & 1))) {
+      if (it >= kStages && !ptx::mbar_wait(&empty[s], (round - 1) & 1)) {
         ok = false;
         return;
       }
-      uint8_t* sb = smem + s * T::kStageBytes + 2 * kABytes + cm * kRowsB * 128;
+      uint8_t* sb = smem + s * T::kStageBytes + 2 * kABytes;
       ptx::mbar_arrive_expect_tx(&full[s], T::kStageBytes);
-      load(&mBhi, sb, s, kc * kBK, n0 + cm * kRowsB, col_mask);
-      load(&mBlo, sb + T::kBBytes, s, kc * kBK, n0 + cm * kRowsB, col_mask);
+      ptx::tma_load_2d(sb, &mBhi, &full[s], kc * kBK, n0);
+      ptx::tma_load_2d(sb + T::kBBytes, &mBlo, &full[s], kc * kBK, n0);
     };
     for (int l = 1; l <= a.L && ok; ++l) {
       const CUtensorMap* hi = l & 1 ? &mAhi0 : &mAhi1;
       const CUtensorMap* lo = l & 1 ? &mAlo0 : &mAlo1;
       auto load_a = [&](int it, int kc) {
         const int s = it % kStages;
-        uint8_t* sa = smem + s * T::kStageBytes + cn * kRowsA * 128;
-        load(hi, sa, s, kc * kBK, m0 + cn * kRowsA, row_mask);
-        load(lo, sa + kABytes, s, kc * kBK, m0 + cn * kRowsA, row_mask);
+        uint8_t* sa = smem + s * T::kStageBytes;
+        ptx::tma_load_2d(sa, hi, &full[s], kc * kBK, m0);
+        ptx::tma_load_2d(sa + kABytes, lo, &full[s], kc * kBK, m0);
       };
       const int it0 = (l - 1) * nk, ahead = min(kStages, nk);
       for (int kc = 0; kc < ahead && ok; ++kc) arm_and_load_b(it0 + kc, kc);
@@ -515,11 +466,7 @@ k_gauss_tc_traj(const __grid_constant__ CUtensorMap mAhi0, const __grid_constant
           ptx::mma_tf32(tmem, a_hi, b_lo, idesc, 1u);
           ptx::mma_tf32(tmem, a_hi, b_hi, idesc, 1u);
         }
-        // (no arrival for a stage that is not refilled: it may find its CTA gone)
-        if (it + kStages < a.L * nk) {
-          if (kCluster) ptx::mma_commit_multicast(&empty[s], row_mask | col_mask);
-          else ptx::mma_commit(&empty[s]);
-        }
+        ptx::mma_commit(&empty[s]);
       }
       if (ok) ptx::mma_commit(acc_full);
     }
@@ -583,7 +530,7 @@ k_gauss_tc_traj(const __grid_constant__ CUtensorMap mAhi0, const __grid_constant
         }
         if (last && ok && m < a.C) {
           part = warp_sum(part);
-          if (lane == 0 && n0 < a.D) a.lp_part[static_cast<int64_t>(m) * a.ntn + blockIdx.y] = 0.5f * part;
+          if (lane == 0) a.lp_part[static_cast<int64_t>(m) * a.ntn + blockIdx.y] = 0.5f * part;
         }
       }
       if (!last) {
@@ -599,9 +546,7 @@ k_gauss_tc_traj(const __grid_constant__ CUtensorMap mAhi0, const __grid_constant
     }
   }
   ptx::tc_fence_before();
-  __syncwarp();
-  if (kCluster) ptx::cluster_sync();
-  else __syncthreads();
+  __syncthreads();
   if (warp == 0) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, T::kTmemCols);
@@ -1118,63 +1063,13 @@ inline unsigned blocks_for(int64_t n) {
 
 namespace {
 using StepKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, TcStepArgs);
-using TrajKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, TcTrajArgs);
-StepKernel gauss_step_kernel(int c) {
-  return c == 1 ? k_gauss_tc_step<kEpiGauss> : k_gauss_tc_step<kEpiGauss, kBN, Tile<kBN>::kStages, 2, 2>;
-}
-TrajKernel gauss_traj_kernel(int c) { return c == 1 ? k_gauss_tc_traj<1, 1> : k_gauss_tc_traj<2, 2>; }
-
-// grid, block and attributes of a trajectory launch
-struct TrajLaunch {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[2];
-  TrajLaunch(const GaussTc& tc, int64_t mt, cudaStream_t s) {
-    const unsigned cm = static_cast<unsigned>(tc.cm), cn = static_cast<unsigned>(tc.cn);
-    cfg.gridDim = dim3((static_cast<unsigned>(mt) + cm - 1) / cm * cm, (tc.ntn + cn - 1) / cn * cn);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kTrajSmem;
-    cfg.stream = s;
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cm;
-    attr[0].val.clusterDim.y = cn;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeCooperative;
-    attr[1].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-  }
-};
 
 // whether all tiles of the trajectory launch are resident at once
-cudaError_t gauss_traj_fits(const GaussTc& tc, int64_t mt, bool* fits) {
-  *fits = false;
-  if (mt * tc.ntn > 4096) return cudaSuccess;
-  TrajLaunch t(tc, mt, nullptr);
-  t.cfg.numAttrs = 1;
-  int clusters = 0;
-  const cudaError_t e = cudaOccupancyMaxActiveClusters(&clusters, gauss_traj_kernel(tc.cm), &t.cfg);
-  if (e != cudaSuccess) return e;
-  *fits = clusters * tc.cm * tc.cn >= static_cast<int>(t.cfg.gridDim.x * t.cfg.gridDim.y);
-  return cudaSuccess;
-}
-
-// one launch of a tile kernel whose clusters are cm x cn tiles
-cudaError_t launch_clusters(StepKernel k, dim3 grid, int cm, int cn, size_t smem, cudaStream_t s,
-                            const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const CUtensorMap& md,
-                            const TcStepArgs& st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((grid.x + cm - 1) / cm * cm, (grid.y + cn - 1) / cn * cn, grid.z);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned>(cm);
-  attr[0].val.clusterDim.y = static_cast<unsigned>(cn);
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = cm * cn > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k, ma, mb, mc, md, st);
+cudaError_t gauss_traj_fits(int64_t mt, int ntn, bool* fits) {
+  int occ = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gauss_tc_traj, kThreads, kTrajSmem);
+  *fits = e == cudaSuccess && mt * ntn <= static_cast<int64_t>(occ) * current_sm_count();
+  return e;
 }
 }  // namespace
 
@@ -1227,25 +1122,13 @@ cudaError_t gauss_tc_setup(GaussTc* tc, const hmc_target& t, int64_t C, void* ws
   for (int i = 0; i < 2 && ok; ++i)
     ok = make_map(&tc->mAhi[i], tc->xhi[i], C, t.dim, kBM) &&
          make_map(&tc->mAlo[i], tc->xlo[i], C, t.dim, kBM);
-  // the per-step kernel's clusters (dim > 256)
-  const int64_t mt = (C + kBM - 1) / kBM;
-  tc->cm = tc->cn = mt > 1 ? 2 : 1;
-  for (int i = 0; i < 2 && ok; ++i)
-    ok = make_map(&tc->mAhi_share[i], tc->xhi[i], C, t.dim, kBM / tc->cn) &&
-         make_map(&tc->mAlo_share[i], tc->xlo[i], C, t.dim, kBM / tc->cn);
-  ok = ok && make_map(&tc->mBhi_share, tc->Phi, t.dim, t.dim, kBN / tc->cm) &&
-       make_map(&tc->mBlo_share, tc->Plo, t.dim, t.dim, kBN / tc->cm);
   if (!ok) return cudaErrorInvalidValue;
-  cudaError_t e = cudaSuccess;
-  for (int c : {1, 2}) {
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(gauss_step_kernel(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(kSmemBytes));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(gauss_traj_kernel(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(kTrajSmem));
-  }
-  if (e == cudaSuccess && t.dim > 256) e = gauss_traj_fits(*tc, mt, &tc->traj);
+  cudaError_t e = cudaFuncSetAttribute(k_gauss_tc_step<kEpiGauss>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(kSmemBytes));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_gauss_tc_traj, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kTrajSmem));
+  if (e == cudaSuccess && t.dim > 256) e = gauss_traj_fits((C + kBM - 1) / kBM, tc->ntn, &tc->traj);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_gauss_tc_step<kEpiStore>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kSmemBytes));
@@ -1283,22 +1166,30 @@ cudaError_t launch_gauss_tc_transition(const StepArgs& a, GaussTc& tc, cudaStrea
   const unsigned nb = static_cast<unsigned>((a.C + kWarpsPerBlock - 1) / kWarpsPerBlock);
   const int mt = (a.C + kBM - 1) / kBM;
   b.met = tc.traj ? tc.met : nullptr;
-  b.nmet = (mt + tc.cm - 1) / tc.cm * tc.cm;
+  b.nmet = mt;
   k_gauss_tc_begin<<<nb, 32 * kWarpsPerBlock, 0, s>>>(b);
   count_launch();
+  const dim3 grid(mt, tc.ntn);
   if (tc.traj) {
     TcTrajArgs st{a.C, a.D, a.L, tc.ntn, {tc.xhi[0], tc.xhi[1]}, {tc.xlo[0], tc.xlo[1]}, tc.p, tc.gL, tc.lp_part,
                   tc.met, a.da, tc.err};
-    TrajLaunch t(tc, mt, s);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kTrajSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     if (timer) timer->begin(s);
-    const cudaError_t e =
-        cudaLaunchKernelEx(&t.cfg, gauss_traj_kernel(tc.cm), tc.mAhi_share[0], tc.mAlo_share[0], tc.mAhi_share[1],
-                           tc.mAlo_share[1], tc.mBhi_share, tc.mBlo_share, st);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_gauss_tc_traj, tc.mAhi[0], tc.mAlo[0], tc.mAhi[1], tc.mAlo[1],
+                                             tc.mBhi, tc.mBlo, st);
     if (e != cudaSuccess) return e;
     if (timer) timer->end(s);
     count_launch();
   }
-  const dim3 grid(mt, tc.ntn);
   for (int l = 1; l <= a.L && !tc.traj; ++l) {
     TcStepArgs st{};
     st.C = a.C;
@@ -1320,9 +1211,7 @@ cudaError_t launch_gauss_tc_transition(const StepArgs& a, GaussTc& tc, cudaStrea
     st.da = a.da;
     st.err = tc.err;
     if (timer) timer->begin(s);
-    const cudaError_t e = launch_clusters(gauss_step_kernel(tc.cm), grid, tc.cm, tc.cn, kSmemBytes, s,
-                                          tc.mAhi_share[in], tc.mAlo_share[in], tc.mBhi_share, tc.mBlo_share, st);
-    if (e != cudaSuccess) return e;
+    k_gauss_tc_step<kEpiGauss><<<grid, kThreads, kSmemBytes, s>>>(tc.mAhi[in], tc.mAlo[in], tc.mBhi, tc.mBlo, st);
     if (timer) timer->end(s);
     count_launch();
   }

@@ -244,9 +244,6 @@ namespace hmc {
 // Device buffers and TMA descriptors of the tensor-core Gaussian path.
 struct GaussTc {
   CUtensorMap mAhi[2], mAlo[2], mBhi, mBlo;
-  // the per-step kernel's clusters of cm x cn tiles: a CTA's share of the rows
-  CUtensorMap mAhi_share[2], mAlo_share[2], mBhi_share, mBlo_share;
-  int cm = 1, cn = 1;
   bool traj = false;         // all steps of a trajectory in one launch (every tile resident)
   unsigned* met = nullptr;   // ... and its counters, one per 128 chains
   CUtensorMap mAhi_blk, mAlo_blk;   // positions xhi[0], xlo[0] in boxes of a NUTS cluster's chains
