@@ -298,12 +298,13 @@ hmc_status hmc_state_bytes(const hmc_ctx* ctx, uint64_t* bytes);
 hmc_status hmc_save_state(hmc_ctx* ctx, void* out, uint64_t bytes);
 hmc_status hmc_restore_state(hmc_ctx* ctx, const void* in, uint64_t bytes);
 
-/* Test support (no counterpart in the paper): for every later launch of the
- * dense-Gaussian CTA-pair kernel, the time after which its grid barrier (the
- * dual-averaging meeting point of a multi-transition launch) gives up, in
- * nanoseconds (default 500000000), and a barrier generation (1, 2, ...; 0:
+/* Test support (no counterpart in the paper): for every later launch whose CTAs
+ * meet on the way -- the dual-averaging meeting point of the dense Gaussian's
+ * multi-transition launches (dim <= 256), the meeting after a leapfrog step of its
+ * trajectory launches (dim > 256) -- the time after which a meeting gives up, in
+ * nanoseconds (default 500000000), and a meeting of the launch (1, 2, ...; 0:
  * none) that can never complete, so that a test can make the bounded wait
- * run out: the kernel then skips its remaining transitions and returns, and
+ * run out: the kernel then skips what remains and returns, and
  * hmc_synchronize reports HMC_E_TIMEOUT.  Process-wide. */
 void hmc_debug_set_grid_barrier(uint64_t wait_limit_ns, int32_t unreachable_generation);
 

@@ -1611,7 +1611,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
 
 }  // namespace
 
-// Test support: the grid barrier's wait limit and an unreachable generation
+// Test support: the meetings' wait limit and an unreachable generation
 // (set by hmc_debug_set_grid_barrier; read at every launch).
 std::atomic<unsigned long long> g_grid_wait_ns{ptx::kWaitLimitNs};
 std::atomic<int> g_unreachable_gen{0};
@@ -1620,6 +1620,8 @@ void set_grid_barrier_debug(unsigned long long wait_ns, int unreachable_gen) {
   g_grid_wait_ns.store(wait_ns);
   g_unreachable_gen.store(unreachable_gen);
 }
+
+MeetingLimits meeting_limits() { return {g_grid_wait_ns.load(), g_unreachable_gen.load()}; }
 
 unsigned gauss_pair_grid(int64_t C) {
   return static_cast<unsigned>(2 * ((C + kPairChains - 1) / kPairChains));

@@ -350,7 +350,23 @@ struct TcTrajArgs {
   unsigned* met;            // [chain blocks] column blocks that have written their positions (zeroed before)
   const DAState* da;
   int* err;
+  MeetingLimits lim;        // the meeting after step g is the g-th
 };
+
+// Whether all epilogue threads say so (a barrier of theirs): one of them that gave
+// up a wait must not leave the others at the next barrier.
+__device__ __forceinline__ bool epilogue_all(bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.and.pred q, 1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(ok ? 1u : 0u), "n"(32 * kEpiWarps)
+      : "memory");
+  return r != 0;
+}
 
 __global__ void __launch_bounds__(kThreads, 1)
 k_gauss_tc_traj(const __grid_constant__ CUtensorMap mAhi0, const __grid_constant__ CUtensorMap mAlo0,
@@ -419,13 +435,14 @@ k_gauss_tc_traj(const __grid_constant__ CUtensorMap mAhi0, const __grid_constant
       for (int kc = 0; kc < ahead && ok; ++kc) arm_and_load_b(it0 + kc, kc);
       if (l > 1 && ok) {
         // every column block of these chains has written x_l
+        const bool never = l - 1 == a.lim.unreachable_gen;      // (tests)
         const unsigned target = static_cast<unsigned>(l - 1) * gridDim.y;
         const unsigned long long t0 = ptx::global_timer_ns();
         unsigned seen = 0;
         while (true) {
           asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.met + blockIdx.x) : "memory");
-          if (seen >= target) break;
-          if (ptx::global_timer_ns() - t0 > ptx::kWaitLimitNs) {
+          if (seen >= target && !never) break;
+          if (ptx::global_timer_ns() - t0 > a.lim.wait_ns) {
             ok = false;
             break;
           }
@@ -499,7 +516,8 @@ k_gauss_tc_traj(const __grid_constant__ CUtensorMap mAhi0, const __grid_constant
         for (int j = 0; j < 16; ++j) stg[(quarter * 32 + lane) * kLd + c0 + j] = acc[j];
       }
       ptx::tc_fence_before();
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+      __syncwarp();
+      ok = epilogue_all(ok);
       const bool last = l == a.L;
       float* xhi = l & 1 ? a.xhi[1] : a.xhi[0];
       float* xlo = l & 1 ? a.xlo[1] : a.xlo[0];
@@ -1172,7 +1190,7 @@ cudaError_t launch_gauss_tc_transition(const StepArgs& a, GaussTc& tc, cudaStrea
   const dim3 grid(mt, tc.ntn);
   if (tc.traj) {
     TcTrajArgs st{a.C, a.D, a.L, tc.ntn, {tc.xhi[0], tc.xhi[1]}, {tc.xlo[0], tc.xlo[1]}, tc.p, tc.gL, tc.lp_part,
-                  tc.met, a.da, tc.err};
+                  tc.met, a.da, tc.err, meeting_limits()};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kThreads);

@@ -1,0 +1,53 @@
+"""Launches whose CTAs meet on the way: a meeting that cannot complete runs into
+its time limit, the launch returns, the call reports it, and the next context
+works.  The limit is a host-side setting; nothing faults or hangs."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+from paper_2002_01184_gb300 import hmc as H  # noqa: E402
+
+
+def gaussian(D):
+    gen = torch.Generator(device="cuda").manual_seed(D)
+    A = torch.randn(D, D, device="cuda", generator=gen, dtype=torch.float64)
+    return (A @ A.T / D + 0.1 * torch.eye(D, device="cuda", dtype=torch.float64)).float().contiguous()
+
+
+def run(target, cfg, x0, B, K):
+    C, D = x0.shape
+    ctx = H.hmc_create(target, C, cfg)
+    x, s = x0.clone(), torch.empty(K, C, D, device="cuda")
+    try:
+        H.hmc_sample_chain(ctx, x, B, K, s)
+        H.hmc_synchronize(ctx)
+    finally:
+        H.hmc_destroy(ctx)
+    return x, s
+
+
+def check_meeting_runs_out(target, cfg, x0, B, K, meeting, message):
+    before = run(target, cfg, x0, B, K)
+    try:
+        H.hmc_debug_set_grid_barrier(20_000_000, meeting)
+        with pytest.raises(H.HMCError) as err:
+            run(target, cfg, x0, B, K)
+        assert err.value.status == H.HMC_E_TIMEOUT and message in str(err.value)
+    finally:
+        H.hmc_debug_set_grid_barrier()
+    after = run(target, cfg, x0, B, K)
+    assert torch.equal(before[0], after[0]) and torch.equal(before[1], after[1])
+    assert torch.isfinite(after[1]).all()
+
+
+# one chain block and several; the meeting after the first step and the last one
+@pytest.mark.parametrize("C,D,meeting", [(64, 260, 1), (300, 320, 3)])
+def test_trajectory_launch(C, D, meeting):
+    P = gaussian(D)
+    x0 = torch.randn(C, D, device="cuda", generator=torch.Generator(device="cuda").manual_seed(C))
+    cfg = H.make_config(4, 0.05, seed=5, use_graph=False)
+    check_meeting_runs_out(H.make_target("corr_gauss", D, P=P), cfg, x0, 0, 1, meeting, "site 1")
