@@ -299,8 +299,9 @@ hmc_status hmc_save_state(hmc_ctx* ctx, void* out, uint64_t bytes);
 hmc_status hmc_restore_state(hmc_ctx* ctx, const void* in, uint64_t bytes);
 
 /* Test support (no counterpart in the paper): for every later launch whose CTAs
- * meet on the way -- the dual-averaging meeting point of the dense Gaussian's
- * multi-transition launches (dim <= 256), the meeting after a leapfrog step of its
+ * meet on the way -- the dual-averaging meeting point of a multi-transition launch
+ * (dense Gaussians of dim <= 256, elementwise targets and small logistic
+ * regressions while they adapt), the meeting after a leapfrog step of its
  * trajectory launches (dim > 256) -- the time after which a meeting gives up, in
  * nanoseconds (default 500000000), and a meeting of the launch (1, 2, ...; 0:
  * none) that can never complete, so that a test can make the bounded wait

@@ -54,6 +54,7 @@ struct EwArgs {
   unsigned* ctr;         // adapting launches: CTAs that left (0 between launches)
   int* err;
   unsigned long long* slots;   // adapting launches: [2][tiles] statistics (chain_sync.cuh)
+  MeetingLimits lim;     // adapting launches: the meeting after transition i is meeting i + 1
 };
 
 template <int G>
@@ -64,8 +65,9 @@ __device__ __forceinline__ float group_sum(float v) {
 }
 
 // Sum of all tiles' slots once written, in the order of tile_partial_then_da
-// (a whole warp); false after the time limit.
-__device__ __forceinline__ bool slots_sum(const unsigned long long* slots, int ntiles, bool negative, double* sum) {
+// (a whole warp); false after the time limit (never: nothing counts as written).
+__device__ __forceinline__ bool slots_sum(const unsigned long long* slots, int ntiles, bool negative,
+                                          unsigned long long wait_ns, bool never, double* sum) {
   const unsigned long long want = negative ? kSlotSign : 0ull;
   const int lane = threadIdx.x & 31;
   unsigned long long t0 = 0;
@@ -80,13 +82,13 @@ __device__ __forceinline__ bool slots_sum(const unsigned long long* slots, int n
 #pragma unroll
       for (int i = 0; i < 8; ++i)
         if ((w[i] & kSlotSign) != want) w[i] = read_slot(slots + b0 + lane + 32 * i);
-      bool ready = true;
+      bool ready = !never;
 #pragma unroll
       for (int i = 0; i < 8; ++i) ready = ready && (w[i] & kSlotSign) == want;
       if (__all_sync(0xffffffffu, ready)) break;
       const unsigned long long now = ptx::global_timer_ns();
       if (!t0) t0 = now;
-      if (__any_sync(0xffffffffu, now - t0 > ptx::kWaitLimitNs)) {
+      if (__any_sync(0xffffffffu, now - t0 > wait_ns)) {
         ok = false;
         break;
       }
@@ -422,7 +424,8 @@ __global__ void __launch_bounds__(32 * W, W == 32 ? 1 : W == 16 ? 2 : NB == 1 ? 
       // every tile's statistic, then the same update in every CTA
       if (warp == 0) {
         double sum;
-        const bool ok = slots_sum(e.slots + (i & 1 ? ntiles : 0), ntiles, (i & 2) != 0, &sum);
+        const bool ok = slots_sum(e.slots + (i & 1 ? ntiles : 0), ntiles, (i & 2) != 0, e.lim.wait_ns,
+                                 i + 1 == e.lim.unreachable_gen, &sum);
         if (lane == 0) {
           if (ok) {
             da_apply_sum(&da_s, coef_s[i & 31], sum, n_c, inv_c, a.t_full + i);
@@ -544,6 +547,7 @@ cudaError_t launch_elementwise_chain(int target_id, const StepArgs& a, bool adap
   e.ctr = sync.left;
   e.err = sync.err;
   e.slots = sync.slots;
+  e.lim = meeting_limits();
   e.vec = a.D % 4 == 0 && aligned16(a.x) && aligned16(a.g) && aligned16(samples);
   int G = a.K > 1 ? 32 : 1;
   while (G < 32 && 4 * G < a.D) G *= 2;

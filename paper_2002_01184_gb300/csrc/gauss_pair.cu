@@ -1621,7 +1621,7 @@ void set_grid_barrier_debug(unsigned long long wait_ns, int unreachable_gen) {
   g_unreachable_gen.store(unreachable_gen);
 }
 
-MeetingLimits meeting_limits() { return {g_grid_wait_ns.load(), g_unreachable_gen.load()}; }
+MeetingLimits meeting_limits() { return {std::max(1ull, g_grid_wait_ns.load()), g_unreachable_gen.load()}; }
 
 unsigned gauss_pair_grid(int64_t C) {
   return static_cast<unsigned>(2 * ((C + kPairChains - 1) / kPairChains));

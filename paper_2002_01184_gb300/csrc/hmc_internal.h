@@ -187,6 +187,10 @@ struct ChainSync {
   int* err = nullptr;
   unsigned long long* slots = nullptr;
 };
+struct MeetingLimits {           // (hmc_debug_set_grid_barrier)
+  unsigned long long wait_ns;
+  int unreachable_gen;           // 0: none
+};
 inline size_t chain_sync_bytes(int64_t C) { return 16 + 16 * static_cast<size_t>((C + 7) / 8); }
 
 // Transitions a.t_full .. a.t_full + T - 1 of the standard normal or the
@@ -352,10 +356,6 @@ cudaError_t launch_gauss_pair_transitions(const StepArgs& a, GaussTc& tc, int T,
 // Test support: wait limit of the meetings inside a launch and a generation that
 // can never complete (0: none), for every later launch.
 void set_grid_barrier_debug(unsigned long long wait_ns, int unreachable_gen);
-struct MeetingLimits {
-  unsigned long long wait_ns;
-  int unreachable_gen;
-};
 MeetingLimits meeting_limits();
 unsigned gauss_fused_grid(int64_t C);
 cudaError_t gauss_fused_setup();

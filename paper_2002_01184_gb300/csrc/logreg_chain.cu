@@ -82,6 +82,7 @@ struct LrChainArgs {
   float* trace_eps;
   uint8_t* trace_acc;
   ChainSync sync;            // one slot per chain
+  MeetingLimits lim;         // adapting launches: the meeting after transition i is meeting i + 1
 };
 
 template <int GT>
@@ -132,9 +133,10 @@ __device__ __forceinline__ void rows_pass(const LrLayout& l, const float* Xs, co
 
 // The sum over C chains of the written slots, tile by tile (eight in chain
 // order), the tiles as tile_partial_then_da adds them; all threads, the value
-// in warp 0.  wait: poll until written; false after the time limit.
-__device__ __forceinline__ bool tile_slots_sum(const unsigned long long* slots, int C, bool negative, bool wait,
-                                               double* sum) {
+// in warp 0.  wait_ns > 0: poll until written; false after that time (never:
+// nothing counts as written).
+__device__ __forceinline__ bool tile_slots_sum(const unsigned long long* slots, int C, bool negative,
+                                               unsigned long long wait_ns, bool never, double* sum) {
   __shared__ double tile_s[kLrGroup * kLrMaxGroups];
   __shared__ int gave_up;
   const int ntiles = (C + 7) / 8;
@@ -151,17 +153,17 @@ __device__ __forceinline__ bool tile_slots_sum(const unsigned long long* slots, 
       for (int i = 0; i < 8; ++i) w[i] = 8 * tile + i < C ? want ^ kSlotSign : want;
       bool ready = false;
       while (!ready) {
-        ready = true;
+        ready = !never;
 #pragma unroll
         for (int i = 0; i < 8; ++i)
           if ((w[i] & kSlotSign) != want) w[i] = read_slot(slots + 8 * tile + i);
 #pragma unroll
         for (int i = 0; i < 8; ++i) ready = ready && (w[i] & kSlotSign) == want;
-        if (!wait) break;
+        if (wait_ns == 0) break;
         if (!ready) {
           const unsigned long long now = ptx::global_timer_ns();
           if (!t0) t0 = now;
-          if (now - t0 > ptx::kWaitLimitNs) {
+          if (now - t0 > wait_ns) {
             gave_up = 1;
             break;
           }
@@ -394,7 +396,7 @@ __global__ void __launch_bounds__(kLrGroup * kLrMaxGroups, 1) k_logreg_chain(LrC
     }
     if (COOP) {
       double sum = 0.0;
-      const bool ok = tile_slots_sum(slots, C, (i & 2) != 0, true, &sum);
+      const bool ok = tile_slots_sum(slots, C, (i & 2) != 0, e.lim.wait_ns, i + 1 == e.lim.unreachable_gen, &sum);
       if (threadIdx.x == 0) {
         if (ok) {
           da_apply_sum(&da_s, coef_s[i & 31], sum, n_c, inv_c, a.t_full + i);
@@ -421,7 +423,7 @@ __global__ void __launch_bounds__(kLrGroup * kLrMaxGroups, 1) k_logreg_chain(LrC
     __syncthreads();
     if (flag_s) {
       double sum = 0.0;
-      tile_slots_sum(e.sync.slots, C, false, false, &sum);
+      tile_slots_sum(e.sync.slots, C, false, 0, false, &sum);
       __syncthreads();
       if (threadIdx.x == 0) {
         da_update(a.da, sum / static_cast<double>(C), a.t_full + e.T - 1);
@@ -481,6 +483,7 @@ cudaError_t launch_logreg_chain(const hmc_target& t, const StepArgs& a, bool ada
   e.trace_eps = trace_eps;
   e.trace_acc = trace_acc;
   e.sync = sync;
+  e.lim = meeting_limits();
   const LrLayout l = lr_layout(e.N, t.dim);
   // a chain per CTA while every chain gets an SM of its own, then two and four
   // groups per CTA (as far as their areas fit) and more chains per group

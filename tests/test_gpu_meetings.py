@@ -51,3 +51,37 @@ def test_trajectory_launch(C, D, meeting):
     x0 = torch.randn(C, D, device="cuda", generator=torch.Generator(device="cuda").manual_seed(C))
     cfg = H.make_config(4, 0.05, seed=5, use_graph=False)
     check_meeting_runs_out(H.make_target("corr_gauss", D, P=P), cfg, x0, 0, 1, meeting, "site 1")
+
+
+# the dual-averaging meetings: CTA pairs, single CTAs
+@pytest.mark.parametrize("C,D", [(128, 132), (4096, 256), (256, 128)])
+@pytest.mark.parametrize("meeting", [1, 4])
+def test_adapting_gaussian_chain(C, D, meeting):
+    P = gaussian(D)
+    x0 = torch.randn(C, D, device="cuda", generator=torch.Generator(device="cuda").manual_seed(C))
+    cfg = H.make_config(3, 0.5 / D ** 0.5, seed=5, adapt=True, num_adapt_steps=4, use_graph=False)
+    check_meeting_runs_out(H.make_target("corr_gauss", D, P=P), cfg, x0, 4, 2, meeting, "site 7")
+
+
+# one CTA; CTAs of 8, 16 and 32 warps; chains that go through memory
+@pytest.mark.parametrize("kind,C,D", [("std_normal", 5, 1), ("funnel", 300, 100), ("funnel", 1300, 100),
+                                      ("funnel", 4096, 100), ("funnel", 9000, 100), ("funnel", 700, 1000)])
+@pytest.mark.parametrize("meeting", [1, 4])
+def test_adapting_elementwise_chain(kind, C, D, meeting):
+    x0 = torch.randn(C, D, device="cuda", generator=torch.Generator(device="cuda").manual_seed(C))
+    cfg = H.make_config(3, 0.1 / D ** 0.25, seed=5, adapt=True, num_adapt_steps=4, use_graph=False)
+    check_meeting_runs_out(H.make_target(kind, D), cfg, x0, 4, 2, meeting, "grid barrier of a multi-transition launch")
+
+
+# one chain; a group per CTA, four groups, several chains per group
+@pytest.mark.parametrize("N,D,C", [(17, 3, 1), (800, 11, 64), (300, 8, 600), (100, 5, 2000)])
+@pytest.mark.parametrize("meeting", [1, 4])
+def test_adapting_logreg_chain(N, D, C, meeting):
+    gen = torch.Generator(device="cuda").manual_seed(N)
+    X = torch.randn(N, D, device="cuda", generator=gen)
+    y = (torch.rand(N, device="cuda", generator=gen) < 0.5).float()
+    x0 = torch.randn(C, D, device="cuda", generator=gen) / D ** 0.5
+    cfg = H.make_config(3, 0.3 / (N * D) ** 0.5, seed=5, adapt=True, num_adapt_steps=4, use_graph=False,
+                        impl=H.HMC_IMPL_FUSED_SIMT)
+    check_meeting_runs_out(H.make_target("logreg", D, X=X, y=y), cfg, x0, 4, 2, meeting,
+                           "grid barrier of a multi-transition launch")
