@@ -548,20 +548,25 @@ hmc_status enqueue_range(hmc_ctx* ctx, float* x, int64_t B, int64_t t_begin, int
   const int64_t t_fixed = ctx->cfg.adapt ? std::min(t_end, std::max(t_begin, ctx->cfg.num_adapt_steps)) : t_begin;
   if (ctx->K == 1 && T > 0 &&
       (uses_logreg_chain(ctx) || (uses_fused_elementwise(ctx) && !(ctx->s_mean && t_fixed > B)))) {
+    // CTAs that meet may have a share of the chains more or less, so a meeting
+    // waits for up to a transition's time, and no wait may take kWaitLimitNs.  A
+    // step takes up to 10 us: past this many a transition is a launch, which is
+    // nothing beside the 5 ms and more that it takes.
+    constexpr int kMeetingMaxLeapfrog = 16384;
+    const int64_t t_meet = ctx->cfg.num_leapfrog <= kMeetingMaxLeapfrog ? t_fixed : t_begin;
     for (int64_t t0 = t_begin; t0 < t_end;) {
       const int64_t stop = t0 < t_fixed ? t_fixed : t_end;
-      const int n = static_cast<int>(std::min(chunk, stop - t0));
+      const int n = static_cast<int>(t_meet <= t0 && t0 < t_fixed ? 1 : std::min(chunk, stop - t0));
       StepArgs a = make_args(ctx, x, static_cast<uint64_t>(t0));
       if (ctx->s_mean && t0 + n > B)
         a.w = hmc::WelfordOut{ctx->s_mean, ctx->s_m2, ctx->s_bsize, ctx->bm_sum, ctx->bm_mean, ctx->bm_m2};
       // (the kernel timer takes the kind of launch that ends the chain)
-      cudaError_t e = launch_chain(ctx, a, t0 < t_fixed, n, B + out0, samples, trace_eps, trace_acc,
+      if (stop == t_end) ctx->dom_transitions = std::max<int64_t>(ctx->dom_transitions, n);
+      cudaError_t e = launch_chain(ctx, a, t0 < t_meet, n, B + out0, samples, trace_eps, trace_acc,
                                    stop == t_end ? &ctx->timer : nullptr);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "chain launch");
       t0 += n;
     }
-    // (the last launch's)
-    ctx->dom_transitions = std::min(chunk, t_end - (t_fixed < t_end ? t_fixed : t_begin));
     return HMC_OK;
   }
   // NUTS: the transitions that do not adapt the step size run in as few

@@ -85,3 +85,32 @@ def test_adapting_logreg_chain(N, D, C, meeting):
                         impl=H.HMC_IMPL_FUSED_SIMT)
     check_meeting_runs_out(H.make_target("logreg", D, X=X, y=y), cfg, x0, 4, 2, meeting,
                            "grid barrier of a multi-transition launch")
+
+
+# 609 chains are 153 groups of four on 152 SMs, 9000 more elementwise chains than are
+# resident: some CTAs have twice the work of others in every transition, which
+# takes far longer here than a meeting may wait
+@pytest.mark.parametrize("kind,N,D,C", [("logreg", 17, 2, 609), ("funnel", 0, 100, 9000)])
+def test_long_transitions_do_not_run_into_the_limit(kind, N, D, C):
+    gen = torch.Generator(device="cuda").manual_seed(C)
+    data = {}
+    if kind == "logreg":
+        data = {"X": torch.randn(N, D, device="cuda", generator=gen),
+                "y": (torch.rand(N, device="cuda", generator=gen) < 0.5).float()}
+    target = H.make_target(kind, D, **data)
+    x0 = torch.randn(C, D, device="cuda", generator=gen)
+    B, K = 2, 1
+    cfg = H.make_config(20000, 1e-4, seed=5, adapt=True, num_adapt_steps=B, use_graph=False)
+    try:
+        H.hmc_debug_set_grid_barrier(1_000_000)
+        x, s = run(target, cfg, x0, B, K)
+    finally:
+        H.hmc_debug_set_grid_barrier()
+    ctx = H.hmc_create(target, C, cfg)
+    y = x0.clone()
+    H.hmc_bootstrap(ctx, y)
+    for t in range(B + K):
+        H.hmc_step(ctx, y, t)
+    H.hmc_synchronize(ctx)
+    H.hmc_destroy(ctx)
+    assert torch.equal(x, y) and torch.equal(s[0], y)
