@@ -234,7 +234,9 @@ std::map<std::tuple<int, int64_t, int64_t, int>, TuneResult> g_tune_cache;
 
 // Milliseconds per transition of `target` with C chains under `impl`, from
 // a zero state with the configuration's step size held fixed; +inf if the
-// context cannot be made.
+// context cannot be made.  With HMC_IMPL_FUSED_SIMT a logistic regression's
+// tiles are launched as the grouped launch runs them (a context of its own
+// may run a small one as whole chains, many times faster).
 double time_transition(const hmc_target& t, int64_t C, const hmc_config& base, int impl, cudaStream_t s) {
   hmc_config c = base;
   c.impl = impl;
@@ -252,9 +254,14 @@ double time_transition(const hmc_target& t, int64_t C, const hmc_config& base, i
   if (e == cudaSuccess) e = cudaMemsetAsync(x, 0, sizeof(float) * C * t.dim, s);
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
-  if (e == cudaSuccess && hmc_bootstrap(ctx, x) == HMC_OK && hmc_step(ctx, x, 0, nullptr) == HMC_OK) {
+  auto step = [&](uint64_t k) {
+    if (impl == HMC_IMPL_FUSED_SIMT)
+      return hmc::launch_logreg_fused_transition(t, hmc::ctx_step_args(ctx, x, k), s, nullptr) == cudaSuccess;
+    return hmc_step(ctx, x, k, nullptr) == HMC_OK;
+  };
+  if (e == cudaSuccess && hmc_bootstrap(ctx, x) == HMC_OK && step(0)) {
     e = cudaEventRecord(e0, s);
-    const bool ok = e == cudaSuccess && hmc_step(ctx, x, 1, nullptr) == HMC_OK;
+    const bool ok = e == cudaSuccess && step(1);
     if (ok && cudaEventRecord(e1, s) == cudaSuccess && cudaEventSynchronize(e1) == cudaSuccess) {
       float f = 0.f;
       if (cudaEventElapsedTime(&f, e0, e1) == cudaSuccess) ms = f;
