@@ -485,6 +485,23 @@ def run_serve(args):
     print(json.dumps(line), flush=True)
 
 
+def elementwise_launch_bytes(kernel, C, D, transitions, burnin, kept, adapt, streaming, replicas):
+    """Bytes that one launch of the elementwise targets' timed kernel cannot do
+    without.  The chain launch reads and writes x and g once, and writes the
+    kept samples of its transitions (the timed launches run burn-in too where
+    nothing adapts; a replica set's samples are copied by another kernel) or,
+    streaming, reads and writes the five moment buffers once.  The plain
+    path's gradient reads x and writes g."""
+    if kernel != "k_elementwise_chain":
+        return 4.0 * C * D * 2
+    rows = 4.0
+    if streaming:
+        rows += 10.0
+    elif replicas == 1 and kept:
+        rows += transitions * kept / (kept if adapt else burnin + kept)
+    return 4.0 * C * D * rows
+
+
 def main():
     args = parse()
     if args.impl == "reference":
@@ -677,9 +694,8 @@ def main():
                     "peak_source": f"derived: {SM_COUNT} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x {sm_max:.0f} MHz",
                     **common}
         else:
-            # elementwise transitions, a range per launch: x and g read and written once,
-            # one kept sample written per transition
-            bytes_per_launch = 4.0 * C * D * (4 + evals_per_launch / (C * p.num_leapfrog))
+            bytes_per_launch = elementwise_launch_bytes(kname, C, D, evals_per_launch / (C * p.num_leapfrog), B, K,
+                                                        p.adapt, streaming, args.replicas)
             achieved = bytes_per_launch / kernel_s / 1e9
             roof = {"bound": "hbm", "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s",
                     "frac": achieved / pk["hbm_gbs"], "traffic": None,
