@@ -33,6 +33,7 @@ struct hmc_ctx {
   void* grad_ws = nullptr;
   size_t grad_ws_bytes = 0;
   bool bootstrapped = false;
+  int64_t adapt_until = 0;         // transitions below it adapt (as the device's adaptation state says)
   // device staging for hmc_sample_chain_host, grown on demand
   void* stage = nullptr;
   size_t stage_bytes = 0;
@@ -429,7 +430,7 @@ cudaError_t enqueue_transition(hmc_ctx* ctx, const StepArgs& a) {
 // After a stream synchronisation: report a bounded device wait that gave up.
 hmc_status check_device_flag(hmc_ctx* ctx) {
   // (of the chain launches only the adapting ones wait)
-  const bool chain_waits = ctx->chain_sync.err && ctx->cfg.adapt;
+  const bool chain_waits = ctx->chain_sync.err && ctx->adapt_until > 0;
   if (!ctx->use_tc && !ctx->use_lrtc && !ctx->use_lrgemm && !chain_waits) return HMC_OK;
   int flag = 0;
   cudaError_t e = cudaMemcpyAsync(&flag,
@@ -449,6 +450,9 @@ hmc_status check_device_flag(hmc_ctx* ctx) {
   return HMC_OK;
 }
 
+// the state that launch_da_init leaves
+void note_fresh_adaptation(hmc_ctx* ctx) { ctx->adapt_until = ctx->cfg.adapt ? ctx->cfg.num_adapt_steps : 0; }
+
 hmc_status bootstrap(hmc_ctx* ctx, const float* x0) {
   cudaError_t e = hmc::launch_grad(ctx->target, ctx->C, x0, ctx->lp, ctx->g, ctx->grad_ws, ctx->stream);
   if (e == cudaSuccess && ctx->K > 1)
@@ -457,6 +461,7 @@ hmc_status bootstrap(hmc_ctx* ctx, const float* x0) {
   e = hmc::launch_da_init(ctx->da, ctx->cfg.step_size, ctx->cfg.adapt, ctx->cfg.target_accept,
                           ctx->cfg.adapt ? ctx->cfg.num_adapt_steps : 0, ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "dual-averaging init");
+  note_fresh_adaptation(ctx);
   ctx->bootstrapped = true;
   return HMC_OK;
 }
@@ -545,7 +550,7 @@ hmc_status enqueue_range(hmc_ctx* ctx, float* x, int64_t B, int64_t t_begin, int
   // adapt the step size in one cooperative launch, the others in one ordinary
   // launch (elementwise moments of transitions that still adapt: one launch
   // per transition, below)
-  const int64_t t_fixed = ctx->cfg.adapt ? std::min(t_end, std::max(t_begin, ctx->cfg.num_adapt_steps)) : t_begin;
+  const int64_t t_fixed = std::min(t_end, std::max(t_begin, ctx->adapt_until));
   if (ctx->K == 1 && T > 0 &&
       (uses_logreg_chain(ctx) || (uses_fused_elementwise(ctx) && !(ctx->s_mean && t_fixed > B)))) {
     // CTAs that meet may have a share of the chains more or less, so a meeting
@@ -574,8 +579,7 @@ hmc_status enqueue_range(hmc_ctx* ctx, float* x, int64_t B, int64_t t_begin, int
   // the run (those that adapt need every chain's statistic in between)
   int64_t t_multi = t_end;
   if (ctx->cfg.proposal == HMC_PROPOSAL_NUTS && !ctx->nuts_dense && ctx->K == 1 && !ctx->s_mean)
-    t_multi = std::min<int64_t>(
-        t_end, std::max<int64_t>(t_begin, ctx->cfg.adapt ? ctx->cfg.num_adapt_steps : 0));
+    t_multi = t_fixed;
   for (int64_t t = t_begin; t < t_multi; ++t) {
     StepArgs a = make_args(ctx, x, static_cast<uint64_t>(t));
     const int64_t k = t - B - out0;
@@ -678,6 +682,7 @@ hmc_status run_chain(hmc_ctx* ctx, float* x, int64_t B, int64_t K, float* sample
   ctx->timer.seen += ctx->g_dominant;
   // every replay re-records the event pairs captured in the graph
   ctx->timer.recorded = std::max(ctx->timer.recorded, ctx->g_recorded);
+  note_fresh_adaptation(ctx);
   ctx->bootstrapped = true;
   return HMC_OK;
 }
@@ -1191,6 +1196,9 @@ hmc_status hmc_restore_state(hmc_ctx* ctx, const void* in, uint64_t bytes) {
   p += sizeof(float) * ctx->C;
   if (e == cudaSuccess) e = cudaMemcpy(ctx->g, p, sizeof(float) * ctx->C * ctx->target.dim, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "restore state");
+  DAState da;
+  std::memcpy(&da, base + sizeof(h), sizeof(da));
+  ctx->adapt_until = da.adapt ? da.num_adapt : 0;
   ctx->bootstrapped = true;
   return HMC_OK;
 }
