@@ -906,7 +906,7 @@ __global__ void k_gauss_tc_accept(TcBeginAccept b) {
 // split order, minus theta (the prior), and the leapfrog update.  Warp per
 // chain, four dims per lane (ld % 4 == 0; the library's own buffers).
 struct LrSumArgs {
-  int C, D, ld, S, last, nrt, ntot;
+  int C, D, ld, S, nrt, ntot;
   const float* part;        // [S x C x ld]
   const float* xhi_in;
   const float* xlo_in;
@@ -984,33 +984,21 @@ __global__ void k_lr_gemm_update(LrSumArgs b) {
     }
     const float4 pv = reinterpret_cast<float4*>(b.p)[e];
     const float pin[4] = {pv.x, pv.y, pv.z, pv.w};
-    float pout[4], hi[4], lo[4];
+    float pout[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       // padding dims (>= D) hold zeros everywhere and stay zero
       g[k] = 4 * j + k < b.D ? g[k] - th[k] : 0.f;
-      if (!b.last) {
-        pout[k] = fmaf(eps, g[k], pin[k]);
-        split_tf32(fmaf(eps, pout[k], th[k]), hi[k], lo[k]);
-      } else {
-        pout[k] = fmaf(0.5f * eps, g[k], pin[k]);
-        sq = fmaf(th[k], th[k], sq);
-      }
+      pout[k] = fmaf(0.5f * eps, g[k], pin[k]);
+      sq = fmaf(th[k], th[k], sq);
     }
     reinterpret_cast<float4*>(b.p)[e] = make_float4(pout[0], pout[1], pout[2], pout[3]);
-    if (!b.last) {
-      reinterpret_cast<float4*>(b.xhi_out)[e] = make_float4(hi[0], hi[1], hi[2], hi[3]);
-      reinterpret_cast<float4*>(b.xlo_out)[e] = make_float4(lo[0], lo[1], lo[2], lo[3]);
-    } else {
-      reinterpret_cast<float4*>(b.g_out)[e] = make_float4(g[0], g[1], g[2], g[3]);
-    }
+    reinterpret_cast<float4*>(b.g_out)[e] = make_float4(g[0], g[1], g[2], g[3]);
   }
-  if (b.last) {
-    sq = warp_sum(sq);
-    // the prior's -|theta|^2 / 2 in the first prior column, the others zero
-    for (int k = lane; k < b.ntot - b.nrt; k += 32)
-      b.lp_part[static_cast<int64_t>(c) * b.ntot + b.nrt + k] = k == 0 ? -0.5f * sq : 0.f;
-  }
+  sq = warp_sum(sq);
+  // the prior's -|theta|^2 / 2 in the first prior column, the others zero
+  for (int k = lane; k < b.ntot - b.nrt; k += 32)
+    b.lp_part[static_cast<int64_t>(c) * b.ntot + b.nrt + k] = k == 0 ? -0.5f * sq : 0.f;
 }
 
 // P -> (tf32 head, float32 remainder)
@@ -1506,13 +1494,17 @@ cudaError_t launch_logreg_gemm_transition(const StepArgs& a, LogregGemm& g, cuda
       // leapfrog update (k_lr_gemm_update)
       st.kc_split = kc_split;
       st.part = g.part;
-      const cudaError_t e = launch_tile<kEpiStore>(g.bng, dim3(mt, g.ndt, S), g.mRhi, g.mRlo, g.mXThi, g.mXTlo, st, s);
+      cudaError_t e = launch_tile<kEpiStore>(g.bng, dim3(mt, g.ndt, S), g.mRhi, g.mRlo, g.mXThi, g.mXTlo, st, s);
       if (e != cudaSuccess) return e;
-      LrSumArgs u{a.C, a.D, g.ld, S, last ? 1 : 0, g.nrt, g.ntot, g.part, g.xhi[in], g.xlo[in],
+      LrSumArgs u{a.C, a.D, g.ld, S, g.nrt, g.ntot, g.part, g.xhi[in], g.xlo[in],
                   g.xhi[out], g.xlo[out], g.p, g.gL, g.lp_part, a.da};
       const int64_t n4 = static_cast<int64_t>(a.C) * (g.ld / 4);
-      if (last) k_lr_gemm_update<<<nb, 32 * kWarpsPerBlock, 0, s>>>(u);
-      else launch_dependent(k_lr_gemm_update_middle, dim3(static_cast<unsigned>((n4 + 255) / 256)), dim3(256), 0, s, u);
+      if (last) {
+        k_lr_gemm_update<<<nb, 32 * kWarpsPerBlock, 0, s>>>(u);
+      } else {
+        e = launch_dependent(k_lr_gemm_update_middle, dim3(static_cast<unsigned>((n4 + 255) / 256)), dim3(256), 0, s, u);
+        if (e != cudaSuccess) return e;
+      }
       count_launch();
     }
     if (timer) timer->end(s);

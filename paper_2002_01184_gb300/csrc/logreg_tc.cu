@@ -384,7 +384,6 @@ struct LrStepArgs {
   const float* Gpart;
   const float* lp_part;
   int nsplit;
-  int last;         // final leapfrog step
 };
 
 // p0 ~ N(0, I); H0; half kick with the cached gradient; first drift
@@ -784,8 +783,7 @@ cudaError_t launch_logreg_tc_transition(const StepArgs& a, LogregTc& tc, int* er
                                        tc.mXTlo, g);
     if (timer) timer->end(s);
     if (e != cudaSuccess) return e;
-    b.last = l == a.L;
-    if (b.last) {
+    if (l == a.L) {
       k_lr_update<<<nb, 32 * kWarpsPerBlock, 0, s>>>(b);
     } else {
       e = cudaLaunchKernelEx(&ucfg, k_lr_update_middle, b);
