@@ -376,6 +376,11 @@ bool uses_logreg_chain(const hmc_ctx* ctx) {
   return uses_fused_logreg(ctx) && hmc::logreg_chain_supported(ctx->target);
 }
 
+// whether a range of its transitions is a launch (else a launch each)
+bool chain_pays(const hmc_ctx* ctx, hmc::ChainKind kind) {
+  return !uses_logreg_chain(ctx) || hmc::logreg_chain_pays(ctx->target, ctx->C, ctx->cfg.num_leapfrog, kind);
+}
+
 // T transitions in one launch, either kind
 cudaError_t launch_chain(hmc_ctx* ctx, const StepArgs& a, bool adapting, int T, long long keep_from, float* samples,
                          float* trace_eps, uint8_t* trace_acc, hmc::KernelTimer* timer) {
@@ -558,10 +563,13 @@ hmc_status enqueue_range(hmc_ctx* ctx, float* x, int64_t B, int64_t t_begin, int
     // step takes up to 10 us: past this many a transition is a launch, which is
     // nothing beside the 5 ms and more that it takes.
     constexpr int kMeetingMaxLeapfrog = 16384;
-    const int64_t t_meet = ctx->cfg.num_leapfrog <= kMeetingMaxLeapfrog ? t_fixed : t_begin;
+    const bool fixed_pays = chain_pays(ctx, hmc::ChainKind::kFixed);
+    const int64_t t_meet = ctx->cfg.num_leapfrog <= kMeetingMaxLeapfrog && chain_pays(ctx, hmc::ChainKind::kAdapting)
+                               ? t_fixed : t_begin;
     for (int64_t t0 = t_begin; t0 < t_end;) {
       const int64_t stop = t0 < t_fixed ? t_fixed : t_end;
-      const int n = static_cast<int>(t_meet <= t0 && t0 < t_fixed ? 1 : std::min(chunk, stop - t0));
+      const bool whole = t0 < t_fixed ? t0 < t_meet : fixed_pays;
+      const int n = static_cast<int>(whole ? std::min(chunk, stop - t0) : 1);
       StepArgs a = make_args(ctx, x, static_cast<uint64_t>(t0));
       if (ctx->s_mean && t0 + n > B)
         a.w = hmc::WelfordOut{ctx->s_mean, ctx->s_m2, ctx->s_bsize, ctx->bm_sum, ctx->bm_mean, ctx->bm_m2};
@@ -1356,7 +1364,7 @@ hmc_status hmc_dominant_kernel_info(const hmc_ctx* ctx, char* name, int32_t name
     n = "k_lr_grad";
   } else if (ctx->use_lrgemm) {
     n = "k_gauss_tc_step<logreg>";   // both products of one gradient
-  } else if (uses_logreg_chain(ctx)) {
+  } else if (uses_logreg_chain(ctx) && chain_pays(ctx, hmc::ChainKind::kFixed)) {
     n = "k_logreg_chain";
     per = ctx->C * ctx->cfg.num_leapfrog * ctx->dom_transitions;
   } else if (uses_fused_logreg(ctx)) {

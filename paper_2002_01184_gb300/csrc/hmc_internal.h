@@ -220,6 +220,10 @@ cudaError_t launch_logreg_fused_transition(const hmc_target& t, const StepArgs& 
 // The same for a small logistic regression whose data fits an SM's shared
 // memory (one slot per chain; moments of adapting transitions too).
 bool logreg_chain_supported(const hmc_target& t);
+// whether a launch of this kind is faster than a launch of tiles per transition
+// (a launch of one transition takes the tiles by itself where they are)
+enum class ChainKind { kFixed, kAdapting, kOne };
+bool logreg_chain_pays(const hmc_target& t, int64_t C, int L, ChainKind kind);
 cudaError_t logreg_chain_setup();
 size_t logreg_chain_sync_bytes(int64_t C);
 cudaError_t launch_logreg_chain(const hmc_target& t, const StepArgs& a, bool adapting, int T, long long keep_from,

@@ -456,6 +456,40 @@ bool logreg_chain_supported(const hmc_target& t) {
          lr_layout(static_cast<int>(t.n_data), t.dim).bytes(1) <= kLrChainSmemMax;
 }
 
+// a chain per CTA while every chain gets an SM of its own, then two and four
+// groups per CTA, as far as their areas fit
+static int chain_groups(const LrLayout& l, int64_t C, int sms) {
+  int g = 1;
+  while (g < kLrMaxGroups && C > sms * g && l.bytes(2 * g) <= kLrChainSmemMax) g *= 2;
+  return g;
+}
+
+// Whether a launch of this kind takes the chain kernel, or the 8-chain tiles
+// (logreg_tile.cuh), a launch per transition: the shorter one by these estimates of a
+// transition in us.  The tiles work through their 16-row blocks one after another but
+// keep up to 64 chains on an SM; the chain kernel has all blocks in flight and `g`
+// chains on an SM, so C chains take `rounds` rounds, each with what a transition costs
+// beside its gradients (in a launch of one transition also the data's way into shared
+// memory).  Fitted to both kernels' times at 4400 points, 17-1500 rows, 4-512 dims,
+// 64-30000 chains, 1-20 steps, all three kinds (median error 7 and 5 %); the choice is off by
+// more than 10 % at 1 % of them.  Tile time / chain time measured: 17 x 4 and 2400
+// chains 0.85 in a fixed range of 10 steps, 0.42 one transition of one step; 64 x 4 and
+// 5000 chains 1.22 and 0.35; 200 x 4 and 5000 chains 2.83 and 0.66; 800 x 11 and 64
+// chains 26 and 15.
+bool logreg_chain_pays(const hmc_target& t, int64_t C, int L, ChainKind kind) {
+  const int N = static_cast<int>(t.n_data), D = t.dim, sms = current_sm_count();
+  const LrLayout l = lr_layout(N, D);
+  const int g = chain_groups(l, C, sms);
+  const double nd = static_cast<double>(N) * D, m = static_cast<double>(C) / (8.0 * sms);
+  const double tiles =
+      9.9 + 1.6 * m + (static_cast<double>(L) * l.nblk + 1.0) * std::max(0.88 + 0.022 * D, m * (0.38 + 0.015 * D));
+  const double rounds = std::ceil(std::ceil(static_cast<double>(C) / g) / sms);
+  const double gradient = 0.50 + 0.012 * l.nblk + 0.36e-4 * g * nd + 0.0064 * D;
+  const double once = kind == ChainKind::kFixed ? 1.6 : kind == ChainKind::kAdapting ? 3.8 : 4.2;
+  const double round = kind == ChainKind::kFixed ? 3.8 : kind == ChainKind::kAdapting ? 4.5 : 7.5 + 3.2e-4 * nd;
+  return once + rounds * (round + L * gradient) <= tiles;
+}
+
 cudaError_t logreg_chain_setup() {
   // the attribute belongs to the kernels, shared by every context: the maximum
   cudaError_t e = cudaSuccess;
@@ -472,6 +506,20 @@ cudaError_t launch_logreg_chain(const hmc_target& t, const StepArgs& a, bool ada
                                 float* samples, float* trace_eps, uint8_t* trace_acc, const ChainSync& sync,
                                 cudaStream_t s, KernelTimer* timer) {
   if (!logreg_chain_supported(t) || T < 1 || a.K > 1) return cudaErrorInvalidValue;
+  if (T == 1 && !adapting && !logreg_chain_pays(t, a.C, a.L, ChainKind::kOne)) {
+    StepArgs one = a;
+    const long long k = a.t_full - keep_from;
+    if (k >= 0) {
+      one.sample_out = samples ? samples + k * a.C * static_cast<int64_t>(a.D) : nullptr;
+      one.trace_eps = trace_eps ? trace_eps + k : nullptr;
+      one.trace_acc = trace_acc ? trace_acc + k * a.C : nullptr;
+    }
+    cudaError_t r = launch_logreg_fused_transition(t, one, s, timer);
+    if (r == cudaSuccess && k >= 0 && a.w.mean)
+      r = launch_welford(static_cast<int64_t>(a.C) * a.D, a.x, k, a.w.mean, a.w.m2, a.w.bsize, a.w.bsum, a.w.bmean,
+                         a.w.bm2, s);
+    return r;
+  }
   LrChainArgs e{};
   e.s = a;
   e.X = t.X;
@@ -485,11 +533,9 @@ cudaError_t launch_logreg_chain(const hmc_target& t, const StepArgs& a, bool ada
   e.sync = sync;
   e.lim = meeting_limits();
   const LrLayout l = lr_layout(e.N, t.dim);
-  // a chain per CTA while every chain gets an SM of its own, then two and four
-  // groups per CTA (as far as their areas fit) and more chains per group
+  // (past four groups a CTA, more chains per group)
   const int sms = current_sm_count();
-  e.groups = 1;
-  while (e.groups < kLrMaxGroups && a.C > sms * e.groups && l.bytes(2 * e.groups) <= kLrChainSmemMax) e.groups *= 2;
+  e.groups = chain_groups(l, a.C, sms);
   const int need = (a.C + e.groups - 1) / e.groups;
   // an adapting range's CTAs must all be resident (one per SM is always)
   const int grid = adapting ? std::min(need, sms) : need;

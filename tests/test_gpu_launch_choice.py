@@ -1,0 +1,74 @@
+"""Calls that take one of two launch forms by their size: the results do not
+depend on it.  Sizes on both sides of the lines."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+import numpy as np  # noqa: E402
+
+from paper_2002_01184_gb300 import hmc as H  # noqa: E402
+from tests.test_gpu_chain_launch import chain, check_equal  # noqa: E402
+
+
+def logreg(N, D, C):
+    gen = torch.Generator(device="cuda").manual_seed(N * 10007 + C)
+    X = torch.randn(N, D, device="cuda", generator=gen)
+    y = (torch.rand(N, device="cuda", generator=gen) < 0.5).float()
+    return X, y, torch.randn(C, D, device="cuda", generator=gen) / D ** 0.5
+
+
+# few rows and many chains: tiles, a launch per transition; some of these sizes take
+# them for single transitions only, or while the step size adapts
+LOGREG = [(17, 4, 2400, 1), (17, 4, 2400, 10), (17, 4, 9000, 3), (100, 4, 5000, 1), (64, 20, 3000, 2), (30, 60, 5000, 2),
+          (200, 4, 2400, 1)]
+
+
+@pytest.mark.parametrize("N,D,C,L", LOGREG)
+@pytest.mark.parametrize("adapt,B,K", [(False, 2, 5), (True, 5, 3)])
+def test_small_logreg_with_many_chains(N, D, C, L, adapt, B, K):
+    X, y, x0 = logreg(N, D, C)
+    cfg = H.make_config(L, 0.5 / (N * D) ** 0.5, seed=11, adapt=adapt, target_accept=0.8, num_adapt_steps=B,
+                        impl=H.HMC_IMPL_FUSED_SIMT)
+    target = H.make_target("logreg", D, X=X, y=y)
+    if N * D * C <= 1 << 22:          # what a batch groups
+        check_equal(target, cfg, x0, B, K)
+    x, s, e, a, da = chain(target, cfg, x0, B, K, False)
+    ctx = H.hmc_create(target, C, cfg)
+    y1 = x0.clone()
+    H.hmc_bootstrap(ctx, y1)
+    for t in range(B + K):
+        H.hmc_step(ctx, y1, t)
+        assert t < B or torch.equal(y1, s[t - B])
+    H.hmc_synchronize(ctx)
+    assert H.hmc_read_adaptation(ctx) == da
+    H.hmc_destroy(ctx)
+
+
+@pytest.mark.parametrize("N,D,C,L", LOGREG[:4])
+@pytest.mark.parametrize("adapt_steps", [0, 4, 12])
+def test_small_logreg_with_many_chains_streams_its_moments(N, D, C, L, adapt_steps):
+    X, y, x0 = logreg(N, D, C)
+    B, K = 4, 8                     # (12 adapting transitions: some kept ones adapt)
+    cfg = H.make_config(L, 0.5 / (N * D) ** 0.5, seed=11, adapt=adapt_steps > 0, target_accept=0.8,
+                        num_adapt_steps=adapt_steps, impl=H.HMC_IMPL_FUSED_SIMT)
+    target = H.make_target("logreg", D, X=X, y=y)
+    x, s, _, _, da = chain(target, cfg, x0, B, K, False)
+    ctx = H.hmc_create(target, C, cfg)
+    x2 = x0.clone()
+    mean, m2, ess = torch.empty_like(x2), torch.empty_like(x2), torch.empty(D, device="cuda")
+    H.hmc_sample_chain_streaming_ess(ctx, x2, B, K, 2, mean, m2, ess)
+    H.hmc_synchronize(ctx)
+    assert H.hmc_read_adaptation(ctx) == da
+    H.hmc_destroy(ctx)
+    assert torch.equal(x2, x)
+    smp = s.double().cpu().numpy()
+    scale = np.abs(smp).max(axis=0) + 1e-6
+    # the tolerances of the streaming tests
+    assert np.max(np.abs(mean.double().cpu().numpy() - smp.mean(axis=0)) / scale) < 1e-5
+    ref_m2 = ((smp - smp.mean(axis=0)) ** 2).sum(axis=0)
+    assert np.max(np.abs(m2.double().cpu().numpy() - ref_m2) / (scale ** 2 * K)) < 1e-5
+    assert torch.isfinite(ess).all()
