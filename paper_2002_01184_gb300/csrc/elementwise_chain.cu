@@ -34,6 +34,7 @@
 #include <cmath>
 
 #include "chain_sync.cuh"
+#include "elementwise_tile.cuh"
 
 namespace hmc {
 
@@ -527,6 +528,34 @@ cudaError_t launch_target(EwArgs& e, int G, bool adapting, int sms, cudaStream_t
   }
 }
 
+// One transition, a warp per chain (elementwise_tile.cuh), without what the chain
+// launch carries from one transition to the next.
+template <int TARGET, int NB>
+__global__ void __launch_bounds__(256) k_fused_elementwise(StepArgs a) {
+  elementwise_tile<TARGET, NB>(a, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x));
+}
+
+template <int TARGET>
+void launch_tiles(const StepArgs& a, cudaStream_t s) {
+  const int nblk = (a.D + 3) / 4;
+  const unsigned grid = accept_blocks(a.C);
+  if (nblk <= 32) k_fused_elementwise<TARGET, 1><<<grid, 256, 0, s>>>(a);
+  else if (nblk <= 64) k_fused_elementwise<TARGET, 2><<<grid, 256, 0, s>>>(a);
+  else if (nblk <= 128) k_fused_elementwise<TARGET, 4><<<grid, 256, 0, s>>>(a);
+  else k_fused_elementwise<TARGET, 8><<<grid, 256, 0, s>>>(a);
+}
+
+// Whether a launch of one transition takes them: for chains of a whole warp where
+// they come in more than one round, so that registers per thread (48 of the tile, 64
+// to 128 of the chain launch) set how many loads are in flight.  Measured, chain
+// launch / tiles: 2000 x 300 1.35, 20000 x 200 1.5, 20000 x 128 1.3 with one leapfrog
+// step; 2000 x 200 and 1000 x 500 1.0; below 65 dims 0.9 to 0.2 (chains share a warp there).
+// With many steps the funnel's chain launch is the shorter one up to 128 dims (0.95).
+bool tiles_pay(int target_id, const StepArgs& a, int sms) {
+  if (a.D > 128) return a.C > 8 * sms;
+  return a.D > 64 && a.C > 16 * sms && (target_id == HMC_T_STD_NORMAL || a.L < 8);
+}
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace
@@ -537,6 +566,20 @@ cudaError_t launch_elementwise_chain(int target_id, const StepArgs& a, bool adap
   if (a.D > kFusedElementwiseMaxDim || T < 1) return cudaErrorInvalidValue;
   if (target_id != HMC_T_STD_NORMAL && target_id != HMC_T_FUNNEL) return cudaErrorInvalidValue;
   if (adapting && (a.K > 1 || a.w.mean)) return cudaErrorInvalidValue;
+  const int sms = current_sm_count();
+  if (T == 1 && !adapting && !a.w.mean && tiles_pay(target_id, a, sms)) {
+    StepArgs t = a;
+    const long long k = a.t_full - keep_from;
+    t.sample_out = k >= 0 && samples ? samples + k * a.C * static_cast<int64_t>(a.D) : nullptr;
+    t.trace_eps = k >= 0 && trace_eps ? trace_eps + k : nullptr;
+    t.trace_acc = k >= 0 && trace_acc ? trace_acc + k * a.C : nullptr;
+    if (timer) timer->begin(s);
+    if (target_id == HMC_T_STD_NORMAL) launch_tiles<HMC_T_STD_NORMAL>(t, s);
+    else launch_tiles<HMC_T_FUNNEL>(t, s);
+    if (timer) timer->end(s);
+    count_launch();
+    return cudaGetLastError();
+  }
   EwArgs e{};
   e.s = a;
   e.T = T;
@@ -553,7 +596,6 @@ cudaError_t launch_elementwise_chain(int target_id, const StepArgs& a, bool adap
   while (G < 32 && 4 * G < a.D) G *= 2;
   // one chain per warp while that is at most two warps per scheduler (its
   // spare lanes then draw ahead); more chains pack into a warp
-  const int sms = current_sm_count();
   while ((a.C >> e.lq) > 8 * sms && (G << e.lq) < 32) ++e.lq;
   const int per_set = kEwWarps << e.lq;
   e.nsets = (a.C + per_set - 1) / per_set;

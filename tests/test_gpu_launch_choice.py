@@ -14,6 +14,30 @@ from paper_2002_01184_gb300 import hmc as H  # noqa: E402
 from tests.test_gpu_chain_launch import chain, check_equal  # noqa: E402
 
 
+# one transition per call (tiles for many chains of more than 64 dims) against
+# the whole chain in one launch
+@pytest.mark.parametrize("kind,C,D,L", [("std_normal", 3000, 100, 1), ("std_normal", 2400, 100, 9), ("funnel", 2600, 65, 7),
+                                        ("funnel", 2600, 65, 8), ("std_normal", 1217, 129, 3), ("funnel", 1216, 300, 2),
+                                        ("funnel", 1300, 260, 2), ("std_normal", 1500, 513, 2), ("funnel", 1250, 1023, 1)])
+@pytest.mark.parametrize("adapt", [False, True])
+def test_single_transitions_equal_the_chain(kind, C, D, L, adapt):
+    gen = torch.Generator(device="cuda").manual_seed(C + D)
+    x0 = torch.randn(C, D, device="cuda", generator=gen)
+    B, K = 3, 3
+    cfg = H.make_config(L, 0.4 / D ** 0.25, seed=7, adapt=adapt, target_accept=0.8, num_adapt_steps=B, chain_offset=5)
+    x, s, e, a, da = chain(H.make_target(kind, D), cfg, x0, B, K, False)
+    ctx = H.hmc_create(H.make_target(kind, D), C, cfg)
+    y = x0.clone()
+    H.hmc_bootstrap(ctx, y)
+    for t in range(B + K):
+        H.hmc_step(ctx, y, t)
+        if t >= B:
+            assert torch.equal(y, s[t - B])
+    H.hmc_synchronize(ctx)
+    assert H.hmc_read_adaptation(ctx) == da
+    H.hmc_destroy(ctx)
+
+
 def logreg(N, D, C):
     gen = torch.Generator(device="cuda").manual_seed(N * 10007 + C)
     X = torch.randn(N, D, device="cuda", generator=gen)
@@ -72,3 +96,19 @@ def test_small_logreg_with_many_chains_streams_its_moments(N, D, C, L, adapt_ste
     ref_m2 = ((smp - smp.mean(axis=0)) ** 2).sum(axis=0)
     assert np.max(np.abs(m2.double().cpu().numpy() - ref_m2) / (scale ** 2 * K)) < 1e-5
     assert torch.isfinite(ess).all()
+
+
+# replica sets: tempered tiles against the chain launch's tempered form
+@pytest.mark.parametrize("kind,D", [("std_normal", 100), ("funnel", 200)])
+def test_replica_sets_do_not_depend_on_their_number(kind, D):
+    betas = [1.0, 0.6, 0.3, 0.1]
+    x0 = torch.randn(700 * 4, D, device="cuda", generator=torch.Generator(device="cuda").manual_seed(D))
+    out = []
+    for sets in (700, 20):
+        ctx = H.hmc_remc_create(H.make_target(kind, D), sets, betas, H.make_config(3, 0.1, seed=13))
+        x, s = x0[:4 * sets].clone(), torch.empty(4, 4 * sets, D, device="cuda")
+        H.hmc_sample_chain(ctx, x, 2, 4, s)
+        H.hmc_synchronize(ctx)
+        H.hmc_destroy(ctx)
+        out.append((x, s))
+    assert torch.equal(out[0][0][:80], out[1][0]) and torch.equal(out[0][1][:, :80], out[1][1])
