@@ -505,6 +505,7 @@ __device__ __forceinline__ bool pl_grid_barrier(unsigned* counter, unsigned gen)
   return true;
 }
 
+template <int NB>
 __global__ void __launch_bounds__(kPlThreads, 1)
 k_nuts_gauss_loop(const __grid_constant__ CUtensorMap mAhi, const __grid_constant__ CUtensorMap mAlo,
                   const __grid_constant__ CUtensorMap mBhi, const __grid_constant__ CUtensorMap mBlo,
@@ -662,7 +663,7 @@ k_nuts_gauss_loop(const __grid_constant__ CUtensorMap mAhi, const __grid_constan
     // ---- one leaf of every active chain
     int mine = 0;
     for (int c = gw; c < C; c += gwarps)
-      if (na.st[c].active && nuts_leaf<kModeGauss, 4>(na, c, lane)) ++mine;
+      if (na.st[c].active && nuts_leaf<kModeGauss, NB>(na, c, lane)) ++mine;
     // positions written for the next products' TMA loads (another proxy)
     asm volatile("fence.proxy.async.global;" ::: "memory");
     if (lane == 0 && mine) atomicAdd(&left[it & 1], static_cast<unsigned>(mine));
@@ -888,7 +889,8 @@ cudaError_t set_leaf_attrs() {
 
 // CTAs of the Gaussian's persistent leaf loop for C chains, 0 if it does not
 // apply (every CTA's tiles must fit its list, all CTAs resident at once)
-int gauss_loop_grid(int C, int D, int* sms_out = nullptr) {
+template <int NB>
+int gauss_loop_grid(int C, int D) {
   static int sms = 0, occ = -1;
   if (!sms) {
     int dev = 0;
@@ -900,7 +902,7 @@ int gauss_loop_grid(int C, int D, int* sms_out = nullptr) {
   }
   if (occ < 0) {
     int o = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_nuts_gauss_loop, kPlThreads, kPlSmem);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_nuts_gauss_loop<NB>, kPlThreads, kPlSmem);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return 0;
@@ -908,12 +910,33 @@ int gauss_loop_grid(int C, int D, int* sms_out = nullptr) {
     occ = o;
   }
   if (occ < 1) return 0;
-  if (sms_out) *sms_out = sms;
   const int ntiles = ((C + kPlBM - 1) / kPlBM) * ((D + kPlBN - 1) / kPlBN);
   const int want = std::max(ntiles, (C + kPlWarps - 1) / kPlWarps);
   const int grid = std::min(sms * occ, want);
   if (static_cast<int64_t>(grid) * kPlMaxTiles < ntiles) return 0;
   return grid;
+}
+
+// Whether a cluster per chain block is the shorter form (dim <= 256).  It is while
+// all clusters run at once (1.15-1.8 times the grid-wide loop at 4096 chains).  A
+// second round of them is nearly as long as the first, however few they are:
+// past that the grid-wide loop gains where a leaf's products are most of it (10000
+// chains x 160-256 dims 1.0-1.24, 5000 x 160 1.29) or where the trees end together
+// because the depth allowed is small (10000 chains x 64-128 dims, depth 4: 1.1-1.2);
+// deep trees of few dims end far apart, and a cluster stops with its own chains
+// (5000 x 128 0.98, 6000 x 64 0.67, 10000 x 100 0.86).
+// The loop also gains with few chains of many dims, whose leaves it spreads over all
+// SMs where a cluster has up to 32 on each of its own (200 x 256 0.90, 500 x 256
+// 0.94, 1000 x 256 0.96, 400 x 224 0.96; 64 x 256, 16 on an SM, 1.07).
+template <typename K>
+cudaError_t cluster_pays(K kernel, const cudaLaunchConfig_t& cfg, int ctas, int C, int D, int max_depth, bool* pays) {
+  *pays = false;
+  if (D > 192 && C > 16 * ctas && C <= (D > 224 ? 8 : 4) * current_sm_count()) return cudaSuccess;
+  int resident = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&resident, kernel, &cfg);
+  const int clusters = static_cast<int>(cfg.gridDim.x) / ctas;
+  *pays = clusters <= resident || (D <= 64 && clusters <= 2 * resident) || (D <= 128 && max_depth > 5);
+  return e;
 }
 
 template <int NB>
@@ -941,17 +964,21 @@ cudaError_t enqueue_nb(const hmc_target& t, const NdArgs& base_args, NutsDense& 
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    // (dim <= 256: at most two blocks of 128 dims per lane)
-    e = cudaLaunchKernelEx(&cfg, k_nuts_gauss_cluster<(NB < 4 ? NB : 2)>, tc.mAhi_blk, tc.mAlo_blk, tc.mBhi, tc.mBlo, na,
-                           ctas);
-    count_launch();
+    constexpr int kNb = NB < 4 ? NB : 2;      // (dim <= 256: at most two blocks of 128 dims per lane)
+    bool cluster = false;
+    e = cluster_pays(k_nuts_gauss_cluster<kNb>, cfg, ctas, a.C, a.D, nd.max_depth, &cluster);
     if (e != cudaSuccess) return e;
-    k_nuts_dense_finish<<<nb, 32 * kNdWarps, 0, s>>>(na);
-    count_launch();
-    if (timer) timer->end(s);
-    return cudaGetLastError();
+    if (cluster) {
+      e = cudaLaunchKernelEx(&cfg, k_nuts_gauss_cluster<kNb>, tc.mAhi_blk, tc.mAlo_blk, tc.mBhi, tc.mBlo, na, ctas);
+      count_launch();
+      if (e != cudaSuccess) return e;
+      k_nuts_dense_finish<<<nb, 32 * kNdWarps, 0, s>>>(na);
+      count_launch();
+      if (timer) timer->end(s);
+      return cudaGetLastError();
+    }
   }
-  const int pgrid = nd.mode == kModeGauss ? gauss_loop_grid(a.C, a.D) : 0;
+  const int pgrid = nd.mode == kModeGauss ? gauss_loop_grid<NB>(a.C, a.D) : 0;
   if (pgrid > 0) {
     // the whole leaf loop in one cooperative launch (grid barrier and the
     // two chains-left counters zeroed first)
@@ -968,7 +995,7 @@ cudaError_t enqueue_nb(const hmc_target& t, const NdArgs& base_args, NutsDense& 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     GaussTc& tc = *nd.tc;
-    e = cudaLaunchKernelEx(&cfg, k_nuts_gauss_loop, tc.mAhi[0], tc.mAlo[0], tc.mBhi, tc.mBlo, na);
+    e = cudaLaunchKernelEx(&cfg, k_nuts_gauss_loop<NB>, tc.mAhi[0], tc.mAlo[0], tc.mBhi, tc.mBlo, na);
     count_launch();
     if (e != cudaSuccess) return e;
     k_nuts_dense_finish<<<nb, 32 * kNdWarps, 0, s>>>(na);
@@ -1050,9 +1077,9 @@ cudaError_t nuts_dense_prepare() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_nuts_gauss_cluster<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kClSmem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_nuts_gauss_loop, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kPlSmem));
+  for (auto k : {k_nuts_gauss_loop<1>, k_nuts_gauss_loop<2>, k_nuts_gauss_loop<4>})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kPlSmem));
   return e;
 }
 

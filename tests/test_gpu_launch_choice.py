@@ -98,6 +98,28 @@ def test_small_logreg_with_many_chains_streams_its_moments(N, D, C, L, adapt_ste
     assert torch.isfinite(ess).all()
 
 
+# NUTS on the Gaussian: a cluster per chain block or the grid-wide loop
+@pytest.mark.parametrize("D,depth,sizes", [(64, 4, (10000, 4900, 40)), (128, 4, (5000, 90)), (128, 7, (5000, 90)),
+                                           (160, 5, (5000, 200, 30)), (256, 6, (5000, 600, 300, 50))])
+def test_nuts_chains_do_not_depend_on_the_loops_form(D, depth, sizes):
+    gen = torch.Generator(device="cuda").manual_seed(D)
+    A = torch.randn(D, D, device="cuda", generator=gen, dtype=torch.float64)
+    P = (A @ A.T / D + 0.1 * torch.eye(D, device="cuda", dtype=torch.float64)).float().contiguous()
+    x0 = torch.randn(max(sizes), D, device="cuda", generator=gen)
+    target, first = H.make_target("corr_gauss", D, P=P), None
+    for C in sizes:
+        ctx = H.hmc_create(target, C, H.make_config(depth, 0.3, seed=9, proposal=H.HMC_PROPOSAL_NUTS))
+        x, s = x0[:C].clone(), torch.empty(3, C, D, device="cuda")
+        a = torch.empty(3, C, dtype=torch.uint8, device="cuda")
+        H.hmc_sample_chain(ctx, x, 1, 3, s, None, a)
+        H.hmc_synchronize(ctx)
+        H.hmc_destroy(ctx)
+        if first is None:
+            first = s, a
+        assert torch.equal(s, first[0][:, :C]) and torch.equal(a, first[1][:, :C])
+    assert first[1].any()
+
+
 # replica sets: tempered tiles against the chain launch's tempered form
 @pytest.mark.parametrize("kind,D", [("std_normal", 100), ("funnel", 200)])
 def test_replica_sets_do_not_depend_on_their_number(kind, D):
