@@ -59,19 +59,28 @@ size_t span_smem_bytes(int Dp, int max_depth) {
   return static_cast<size_t>(kWarps) * 2 * (max_depth > 1 ? max_depth - 1 : 0) * Dp * sizeof(float);
 }
 
-// resident blocks per SM, which set the registers a thread may have: WIDE for
-// calls whose chains all fit so, else as many as a leaf's state allows without
-// spills on its critical path (funnel, 4096 x 100: 1458 us for 20 transitions at 5
-// blocks, 1869 at 7; standard normal, 4096 x 7: 491 at 7, 550 at 5)
-constexpr int nuts_blocks(int target, int nb, bool wide) {
-  return wide ? (nb == 1 ? 4 : 2) : target == HMC_T_FUNNEL ? (nb == 1 ? 5 : nb == 2 ? 4 : 3) : nb == 1 ? 7 : 4;
+// Forms of the kernel.  Resident blocks per SM set the registers a thread may have.
+// kWide: for calls whose chains all fit so.  kPlain: as many blocks as a leaf's state
+// allows without spills on its critical path (funnel, 4096 x 100: 1458 us for 20
+// transitions at 5 blocks, 1869 at 7; standard normal, 4096 x 7: 491 at 7, 550 at 5).
+// kLean (past 256 dims): four blocks, for which a leaf forms its own sum of squares
+// first and nothing of the next leaf: with every scheduler's slots full the
+// instructions count and not a leaf's latency.  20 transitions of the funnel in one
+// launch, kPlain / kLean: 2000 x 400 1.31, 4096 x 300 1.19, 3000 x 400 0.98; of the standard
+// normal, 4096 x 260 1.11.  A launch of one transition, which ends with its deepest
+// trees, is the shorter in kPlain for the funnel (1300 x 300 0.90).
+constexpr int kPlain = 0, kWide = 1, kLean = 2;
+constexpr int nuts_blocks(int target, int nb, int form) {
+  return form == kWide ? (nb == 1 ? 4 : 2)
+         : form == kLean ? 4
+         : target == HMC_T_FUNNEL ? (nb == 1 ? 5 : nb == 2 ? 4 : 3) : nb == 1 ? 7 : 4;
 }
 
-template <int TARGET, int NB, bool SMEM, bool WIDE>
-__global__ void __launch_bounds__(32 * kWarps, nuts_blocks(TARGET, NB, WIDE)) k_nuts(NutsArgs na) {
+template <int TARGET, int NB, bool SMEM, int FORM>
+__global__ void __launch_bounds__(32 * kWarps, nuts_blocks(TARGET, NB, FORM)) k_nuts(NutsArgs na) {
   // the next leaf's position held over this leaf's decisions; the open pair's
   // first leaf in registers
-  constexpr bool kKeepNext = WIDE || (TARGET == HMC_T_FUNNEL && NB == 1), kKeepFirst = kKeepNext && NB == 1;
+  constexpr bool kKeepNext = FORM == kWide || (TARGET == HMC_T_FUNNEL && NB == 1), kKeepFirst = kKeepNext && NB == 1;
   extern __shared__ float4 span_smem[];
   const StepArgs& a = na.s;
   const int warp = threadIdx.x >> 5;
@@ -205,8 +214,11 @@ __global__ void __launch_bounds__(32 * kWarps, nuts_blocks(TARGET, NB, WIDE)) k_
             x[b][i] = fmaf(ev, p[b][i], x[b][i]);
             if (!is_v(b, i)) q = fmaf(x[b][i], x[b][i], q);
           }
-        float em = expf(-v0);
-        q = warp_sum(q);
+        float em = 0.f;
+        if (FORM != kLean) {
+          em = expf(-v0);
+          q = warp_sum(q);
+        }
         // first leaf of the span of two leaves in progress
         float xf[NB][4], pf[NB][4];
 #pragma unroll
@@ -225,6 +237,18 @@ __global__ void __launch_bounds__(32 * kWarps, nuts_blocks(TARGET, NB, WIDE)) k_
           const int kq = k & 3;
           const uint32_t wsub = __shfl_sync(0xffffffffu, kq == 0 ? wsub4.x : kq == 1 ? wsub4.y : kq == 2 ? wsub4.z : wsub4.w,
                                             (k >> 2) & 31);
+          if (FORM == kLean) {
+            em = expf(-v0);
+            q = 0.f;
+#pragma unroll
+            for (int b = 0; b < NB; ++b)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                if (!is_v(b, i)) q = fmaf(x[b][i], x[b][i], q);
+                xf[b][i] = pf[b][i] = 0.f;      // (not carried from leaf to leaf)
+              }
+            q = warp_sum(q);
+          }
           // the gradient at the drifted x, whose sum of squares is known, and the
           // second half kick
           if (TARGET == HMC_T_FUNNEL) g0 = v0 * (-1.f / 9.f) - half_n + 0.5f * em * q;
@@ -249,19 +273,26 @@ __global__ void __launch_bounds__(32 * kWarps, nuts_blocks(TARGET, NB, WIDE)) k_
             for (int i = 0; i < 4; ++i) {
               g[b][i] = is_v(b, i) ? g0 : TARGET == HMC_T_FUNNEL ? -em * x[b][i] : -x[b][i];
               p[b][i] = fmaf(hv, g[b][i], p[b][i]);
-              pn[b][i] = fmaf(hv, g[b][i], p[b][i]);
-              xn[b][i] = fmaf(ev, pn[b][i], x[b][i]);
+              if (FORM != kLean) {
+                pn[b][i] = fmaf(hv, g[b][i], p[b][i]);
+                xn[b][i] = fmaf(ev, pn[b][i], x[b][i]);
+              }
               if (!is_v(b, i)) {
                 pp = fmaf(p[b][i], p[b][i], pp);
-                qn = fmaf(xn[b][i], xn[b][i], qn);
+                if (FORM != kLean) qn = fmaf(xn[b][i], xn[b][i], qn);
                 const float dx = sv * (x[b][i] - xf[b][i]);
                 d1 = fmaf(dx, pf[b][i], d1);
                 d2 = fmaf(dx, p[b][i], d2);
               }
             }
           const float p0h = fmaf(hv, g0, p0n), v0n = fmaf(ev, p0h, v0);
-          em = expf(-v0n);
-          warp_sum4(qn, pp, d1, d2);
+          if (FORM == kLean) {
+            pp = warp_sum(pp);
+            if (k & 1) warp_sum2(d1, d2);
+          } else {
+            em = expf(-v0n);
+            warp_sum4(qn, pp, d1, d2);
+          }
           if (TARGET == HMC_T_FUNNEL) {
             const float dx0 = sv * (v0 - xf0);
             d1 = fmaf(dx0, pf0, d1);
@@ -416,50 +447,58 @@ __global__ void __launch_bounds__(32 * kWarps, nuts_blocks(TARGET, NB, WIDE)) k_
   }
 }
 
-template <int TARGET, int NB, bool SMEM, bool WIDE>
+template <int TARGET, int NB, bool SMEM, int FORM>
 cudaError_t launch_v(const NutsArgs& na, size_t smem, cudaStream_t s) {
   const unsigned grid = nuts_grid(na.s.C);
-  k_nuts<TARGET, NB, SMEM, WIDE><<<grid, 32 * kWarps, SMEM ? smem : 0, s>>>(na);
+  k_nuts<TARGET, NB, SMEM, FORM><<<grid, 32 * kWarps, SMEM ? smem : 0, s>>>(na);
   count_launch();
   return cudaGetLastError();
 }
 
 // resident blocks per SM with the span starts in scratch and in shared memory
 // (0: they do not fit)
-template <int TARGET, int NB, bool WIDE>
+template <int TARGET, int NB, int FORM>
 cudaError_t residency(size_t smem, int* glob, int* shared) {
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(glob, k_nuts<TARGET, NB, false, WIDE>, 32 * kWarps, 0);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(glob, k_nuts<TARGET, NB, false, FORM>, 32 * kWarps, 0);
   *shared = 0;
   if (e == cudaSuccess && smem > 0 && smem <= kNutsSpanSmemMax)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(shared, k_nuts<TARGET, NB, true, WIDE>, 32 * kWarps, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(shared, k_nuts<TARGET, NB, true, FORM>, 32 * kWarps, smem);
   return e;
+}
+
+inline bool all_resident(const NutsArgs& na, int blocks, int sms) {
+  return static_cast<int64_t>(blocks) * kWarps * sms >= na.s.C;
+}
+
+// More chains than the wide form holds.  Span starts in shared memory unless
+// they cost resident chains: as many blocks per SM as the scratch form, or
+// enough for every chain.
+template <int TARGET, int NB, int FORM>
+cudaError_t launch_many(const NutsArgs& na, size_t smem, bool wide, int sms, cudaStream_t s) {
+  int glob = 0, shared = 0;
+  const cudaError_t e = residency<TARGET, NB, FORM>(smem, &glob, &shared);
+  if (e != cudaSuccess) return e;
+  if (shared > 0 && (shared >= glob || all_resident(na, shared, sms))) return launch_v<TARGET, NB, true, FORM>(na, smem, s);
+  return wide ? launch_v<TARGET, NB, false, kWide>(na, 0, s) : launch_v<TARGET, NB, false, FORM>(na, 0, s);
 }
 
 template <int TARGET, int NB>
 cudaError_t launch_nb(const NutsArgs& na, cudaStream_t s) {
   const size_t smem = span_smem_bytes(na.Dp, na.max_depth);
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return cudaErrorUnknown;
-  }
-  auto fit = [&](int blocks) { return static_cast<int64_t>(blocks) * kWarps * sms >= na.s.C; };
+  const int sms = current_sm_count();
   int glob = 0, shared = 0;
-  cudaError_t e = residency<TARGET, NB, true>(smem, &glob, &shared);
+  const cudaError_t e = residency<TARGET, NB, kWide>(smem, &glob, &shared);
   if (e != cudaSuccess) return e;
   // the wide form where all its chains are resident at once: 1024 x 100 funnel
   // 832 us for 20 transitions (837 at 5 blocks), 1000 x 500 1605 against 1813,
   // but 2000 x 200 standard normal 362 us against 262, in two waves
-  if (fit(shared)) return launch_v<TARGET, NB, true, true>(na, smem, s);
-  const bool wide = fit(glob);
-  e = residency<TARGET, NB, false>(smem, &glob, &shared);
-  if (e != cudaSuccess) return e;
-  // shared-memory span starts unless they cost resident chains: as many
-  // blocks per SM as the scratch form, or enough for every chain
-  if (shared > 0 && (shared >= glob || fit(shared))) return launch_v<TARGET, NB, true, false>(na, smem, s);
-  return wide ? launch_v<TARGET, NB, false, true>(na, 0, s) : launch_v<TARGET, NB, false, false>(na, 0, s);
+  if (all_resident(na, shared, sms)) return launch_v<TARGET, NB, true, kWide>(na, smem, s);
+  const bool wide = all_resident(na, glob, sms);
+  if constexpr (NB == 4) {
+    if (TARGET == HMC_T_STD_NORMAL || na.T > 1) return launch_many<TARGET, NB, kLean>(na, smem, wide, sms, s);
+  }
+  if constexpr (NB < 4 || TARGET == HMC_T_FUNNEL) return launch_many<TARGET, NB, kPlain>(na, smem, wide, sms, s);
+  return cudaErrorInvalidValue;      // (not reached)
 }
 
 template <int TARGET>
@@ -470,13 +509,24 @@ cudaError_t launch_t(const NutsArgs& na, cudaStream_t s) {
   return launch_nb<TARGET, 4>(na, s);
 }
 
-template <int TARGET, int NB>
+template <int TARGET, int NB, int FORM>
 cudaError_t allow_smem() {
-  const cudaError_t e = cudaFuncSetAttribute(k_nuts<TARGET, NB, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(kNutsSpanSmemMax));
-  return e != cudaSuccess ? e
-                          : cudaFuncSetAttribute(k_nuts<TARGET, NB, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 static_cast<int>(kNutsSpanSmemMax));
+  return cudaFuncSetAttribute(k_nuts<TARGET, NB, true, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(kNutsSpanSmemMax));
+}
+
+template <int TARGET>
+cudaError_t allow_smem_target() {
+  cudaError_t e = allow_smem<TARGET, 1, kWide>();
+  if (e == cudaSuccess) e = allow_smem<TARGET, 2, kWide>();
+  if (e == cudaSuccess) e = allow_smem<TARGET, 4, kWide>();
+  if (e == cudaSuccess) e = allow_smem<TARGET, 1, kPlain>();
+  if (e == cudaSuccess) e = allow_smem<TARGET, 2, kPlain>();
+  if (e == cudaSuccess) e = allow_smem<TARGET, 4, kLean>();
+  if constexpr (TARGET == HMC_T_FUNNEL) {
+    if (e == cudaSuccess) e = allow_smem<TARGET, 4, kPlain>();
+  }
+  return e;
 }
 
 }  // namespace
@@ -492,13 +542,8 @@ size_t nuts_scratch_floats(const hmc_target& t, int64_t C) {
 unsigned nuts_grid(int64_t C) { return static_cast<unsigned>((C + kWarps - 1) / kWarps); }
 
 cudaError_t nuts_prepare() {
-  cudaError_t e = allow_smem<HMC_T_STD_NORMAL, 1>();
-  if (e == cudaSuccess) e = allow_smem<HMC_T_STD_NORMAL, 2>();
-  if (e == cudaSuccess) e = allow_smem<HMC_T_STD_NORMAL, 4>();
-  if (e == cudaSuccess) e = allow_smem<HMC_T_FUNNEL, 1>();
-  if (e == cudaSuccess) e = allow_smem<HMC_T_FUNNEL, 2>();
-  if (e == cudaSuccess) e = allow_smem<HMC_T_FUNNEL, 4>();
-  return e;
+  const cudaError_t e = allow_smem_target<HMC_T_STD_NORMAL>();
+  return e != cudaSuccess ? e : allow_smem_target<HMC_T_FUNNEL>();
 }
 
 cudaError_t launch_nuts_transitions(const hmc_target& t, const StepArgs& a, float* scratch,
