@@ -332,8 +332,12 @@ int32_t hmc_uses_tensor_cores(const hmc_ctx* ctx);
  * hmc_profile_dominant_kernel times for this context and how many chain
  * gradient evaluations one launch of it performs (chains x leapfrog steps for
  * the one-launch-per-transition kernels, times the transitions of the last
- * hmc_sample_chain where one launch ran all of them -- the dense Gaussian on
- * CTA pairs -- and chains for one gradient product). */
+ * hmc_sample_chain's launch where one launch runs many, and chains for one
+ * gradient product).  The name is that of the path: "k_gauss_pair" stands for
+ * its form on single CTAs too (k_gauss_one, dim <= 128 without replicas),
+ * "k_gauss_tc_step" for its form that runs a whole trajectory per launch
+ * (k_gauss_tc_traj), "k_elementwise_chain" for the tiles that single transitions of
+ * many wide chains take (k_fused_elementwise). */
 hmc_status hmc_dominant_kernel_info(const hmc_ctx* ctx, char* name, int32_t name_len,
                                     int64_t* grad_evals_per_launch);
 

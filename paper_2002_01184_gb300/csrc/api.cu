@@ -290,11 +290,15 @@ CreatePlan plan_create(const hmc_target& t, int64_t num_chains, const hmc_config
   // logistic regressions with long data passes or much work per gradient
   // (chains x rows x dim above 2^22): tensor-core products; small ones: the
   // shared-memory SIMT transition
-  // A context whose shared-memory grid (one CTA per 8 chains) covers under
-  // half of the SMs streams each gradient's data pass through few SMs, at
+  // A context whose shared-memory grid (one CTA of tiles per 8 chains) covers
+  // under half of the SMs streams each gradient's data pass through few SMs, at
   // about 9e9 multiply-adds/s per CTA (8 chains x 2000 rows x 128 dims:
   // 0.46 ms per leapfrog step): from 10^4 data entries on, the tensor-core
-  // products' fixed ~15 us per gradient costs less.
+  // products' fixed ~10 us per gradient costs less.  Both lines are the tiles'.
+  // Data that fits an SM beside a chain is a launch of whole chains on the SIMT
+  // path (logreg_chain.cu), which would be the sooner one past these lines too
+  // (HMC_IMPL_FUSED_SIMT against _TENSOR, 10 steps: 900 x 12 and 64 chains 20 against 105
+  // us a transition, 2000 x 16 and 64 38 against 110, 1000 x 20 and 1000 92 against 117).
   const bool lr_narrow = t.id == HMC_T_LOGREG && (num_chains + 7) / 8 < hmc::current_sm_count() / 2 &&
                          t.n_data * t.dim > 10000;
   const bool lr_big = t.id == HMC_T_LOGREG &&
