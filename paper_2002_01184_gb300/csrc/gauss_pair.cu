@@ -1235,7 +1235,10 @@ constexpr size_t kOneSmem = 120 * 1024;            // one CTA per SM: it allocat
 static_assert(kOneSmemUsed <= kOneSmem, "shared memory");
 static_assert(kOneColP + 2 * 128 <= static_cast<int>(kTmemCols), "tensor-memory columns");
 
-template <bool MOMENTS>
+// ONE_STEP: trajectories of one leapfrog step, which need a barrier more (in a kernel
+// of its own: the test of L alone cost the longer trajectories 0.3 %, a third slot
+// instead of the barrier 0.5 to 3 %).
+template <bool MOMENTS, bool ONE_STEP>
 __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
   const StepArgs& a = fa.s;
   extern __shared__ uint8_t smem_raw[];
@@ -1243,10 +1246,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   __shared__ uint64_t acc_full[1], own_full[1];
   __shared__ uint32_t tmem_slot[4];
-  // |p0|^2 of transition j at j % 3: with one leapfrog step a warp may write
-  // transition j + 1's while another still decides j - 1 (the accumulator that
-  // every thread's positions of j lead to is the only meeting between them)
-  __shared__ float red[2][4][kHalf], kin_s[3][4][kHalf], lu_s[2][kHalf];
+  __shared__ float red[2][4][kHalf], kin_s[2][4][kHalf], lu_s[2][kHalf];
   __shared__ DAState da_s;
   __shared__ DACoef coef_s;
   __shared__ unsigned long long psum_s;
@@ -1341,7 +1341,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
     };
     // |p0|^2 of the warp's 16 chains over its 32 dims, in the pair's order:
     // the butterfly's first step in full, then halving
-    auto kinetic = [&](const float (&z)[16], int j) {
+    auto kinetic = [&](const float (&z)[16], uint32_t tn) {
       float v[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) v[i] = z[i] * z[i];
@@ -1357,7 +1357,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
           v[k] = keep + __shfl_xor_sync(0xffffffffu, send, w);
         }
       }
-      if (lane < 16) kin_s[j % 3][quarter][16 * sub + lane] = v[0];
+      if (lane < 16) kin_s[tn & 1u][quarter][16 * sub + lane] = v[0];
     };
     // momenta of slots 4 g .. 4 g + 3 at transition tn
     auto draw = [&](float (&z)[16], int g0, int g1, uint32_t tn) {
@@ -1407,7 +1407,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
       }
     }
     draw(z, 0, 4, a.t);
-    kinetic(z, 0);
+    kinetic(z, a.t);
     // lane c of every warp decides chain c0 + c (the same inputs, the same answer)
     const int chain = c0 + lane;
     float lpc = chain < C ? a.lp[chain] : 0.f;
@@ -1443,7 +1443,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
       }
       if (more) {
         draw(zn, (L - 1) * per_wait, 4, t + 1);
-        kinetic(zn, j + 1);
+        // another warp may still read this slot for its decision of transition
+        // j - 1: every step's accumulator wait proves it past that, but with one
+        // step there has been none yet
+        if (ONE_STEP) epi_barrier();
+        kinetic(zn, t + 1);
       }
       wait_acc(s0 + L - 1);
       load_acc(acc);
@@ -1472,7 +1476,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gauss_one(PairArgs fa) {
         for (int q = 0; q < 4; ++q) {
           xg += red[0][q][lane];
           pp += red[1][q][lane];
-          k0 += kin_s[j % 3][q][lane];
+          k0 += kin_s[t & 1u][q][lane];
         }
         const float kin0 = 0.5f * k0, lp1 = 0.5f * xg;
         la = (-lpc + kin0) - (-lp1 + 0.5f * pp);
@@ -1638,12 +1642,9 @@ cudaError_t launch_gauss_pair_image(const float* Phi, const float* Plo, int D, f
 cudaError_t gauss_pair_setup() {
   cudaError_t e = cudaFuncSetAttribute(k_gauss_pair<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(kSmem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gauss_one<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kOneSmem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gauss_one<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kOneSmem));
+  for (auto k : {k_gauss_one<false, false>, k_gauss_one<true, false>, k_gauss_one<false, true>, k_gauss_one<true, true>})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kOneSmem));
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_gauss_pair<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(kSmem));
@@ -1710,8 +1711,10 @@ cudaError_t launch_gauss_pair_transitions(const StepArgs& a, GaussTc& tc, int T,
     cfg.attrs = coop;
     cfg.numAttrs = T > 1 ? 1 : 0;
     if (timer) timer->begin(s);
-    const cudaError_t e = a.w.mean && nkeep > 0 ? cudaLaunchKernelEx(&cfg, k_gauss_one<true>, fa)
-                                                : cudaLaunchKernelEx(&cfg, k_gauss_one<false>, fa);
+    const bool moments = a.w.mean && nkeep > 0;
+    auto kernel = a.L == 1 ? moments ? k_gauss_one<true, true> : k_gauss_one<false, true>
+                           : moments ? k_gauss_one<true, false> : k_gauss_one<false, false>;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, fa);
     if (timer) timer->end(s);
     count_launch();
     return e;
