@@ -39,3 +39,26 @@ def test_single_step_chain_equals_single_transitions(C, D):
     for u in out[1:]:
         for v, w in zip(u, out[0]):
             assert torch.equal(v, w)
+
+
+# ... and with running moments instead of a trace
+@pytest.mark.parametrize("C,D", [(1500, 128), (70, 40)])
+def test_single_step_streaming_equals_stored_trace(C, D):
+    gen = torch.Generator(device="cuda").manual_seed(C + D)
+    A = torch.randn(D, D, device="cuda", generator=gen, dtype=torch.float64)
+    P = (A @ A.T / D + 0.1 * torch.eye(D, device="cuda", dtype=torch.float64)).float().contiguous()
+    x0 = torch.randn(C, D, device="cuda", generator=gen)
+    B, K = 5, 30
+    ctx = H.hmc_create(H.make_target("corr_gauss", D, P=P), C, H.make_config(1, 0.9 / D ** 0.25, seed=23))
+    x, s = x0.clone(), torch.empty(K, C, D, device="cuda")
+    H.hmc_sample_chain(ctx, x, B, K, s)
+    y, mean, m2 = x0.clone(), torch.empty_like(x0), torch.empty_like(x0)
+    H.hmc_sample_chain_streaming(ctx, y, B, K, mean, m2)
+    H.hmc_synchronize(ctx)
+    H.hmc_destroy(ctx)
+    assert torch.equal(x, y)
+    smp = s.double()
+    scale = smp.abs().amax(0) + 1e-6
+    # the tolerances of the streaming tests
+    assert ((mean.double() - smp.mean(0)).abs() / scale).max() < 1e-5
+    assert ((m2.double() - (smp - smp.mean(0)).square().sum(0)).abs() / (scale ** 2 * K)).max() < 1e-5
