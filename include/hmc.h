@@ -309,6 +309,16 @@ hmc_status hmc_restore_state(hmc_ctx* ctx, const void* in, uint64_t bytes);
  * hmc_synchronize reports HMC_E_TIMEOUT.  Process-wide. */
 void hmc_debug_set_grid_barrier(uint64_t wait_limit_ns, int32_t unreachable_generation);
 
+/* Say that each CUDA graph of the context will be launched once (once = 1; 0, the
+ * default: replayed), as for a served request (no counterpart in the paper).  The
+ * large logistic regressions' chains of short launches overlap each launch's start
+ * with the end of the one before (programmatic dependent launches), which takes 1 to
+ * 12 % off a replay but costs the host about 2 us a launch when the graph is
+ * instantiated and destroyed; with once = 1 their launches are ordinary ones.  Drops
+ * a captured graph where the setting changes.  Results do not depend on it.
+ * HMC_E_INVALID if once is neither 0 nor 1. */
+hmc_status hmc_graphs_run_once(hmc_ctx* ctx, int32_t once);
+
 /* Copy the current dual-averaging state to host memory and synchronise:
  * out[0] = step size of the next transition, out[1] = log eps_bar,
  * out[2] = h_bar, out[3] = adaptation steps taken, out[4] = last transition's

@@ -33,6 +33,7 @@ struct hmc_ctx {
   void* grad_ws = nullptr;
   size_t grad_ws_bytes = 0;
   bool bootstrapped = false;
+  bool graphs_once = false;        // hmc_graphs_run_once
   int64_t adapt_until = 0;         // transitions below it adapt (as the device's adaptation state says)
   // device staging for hmc_sample_chain_host, grown on demand
   void* stage = nullptr;
@@ -415,6 +416,7 @@ StepArgs make_args(hmc_ctx* ctx, float* x, uint64_t t) {
   a.K = ctx->K;
   a.proposal = ctx->cfg.proposal;
   a.merged = ctx->cfg.impl != HMC_IMPL_PLAIN;
+  a.overlap = !ctx->graphs_once;
   return a;
 }
 
@@ -1217,6 +1219,14 @@ hmc_status hmc_restore_state(hmc_ctx* ctx, const void* in, uint64_t bytes) {
 
 void hmc_debug_set_grid_barrier(uint64_t wait_limit_ns, int32_t unreachable_generation) {
   hmc::set_grid_barrier_debug(static_cast<unsigned long long>(wait_limit_ns), unreachable_generation);
+}
+
+hmc_status hmc_graphs_run_once(hmc_ctx* ctx, int32_t once) {
+  if (!ctx) return fail(nullptr, HMC_E_INVALID, "ctx is NULL");
+  if (once != 0 && once != 1) return fail(ctx, HMC_E_INVALID, "once must be 0 or 1");
+  if (ctx->graphs_once != (once != 0)) drop_graph(ctx);
+  ctx->graphs_once = once != 0;
+  return HMC_OK;
 }
 
 hmc_status hmc_read_adaptation(hmc_ctx* ctx, double out[5]) {

@@ -1269,12 +1269,12 @@ struct LrTiles {
 };
 // R X's tile: split-K products, bn columns (a multiple of 32)
 template <int EPI>
-cudaError_t launch_tile(int bn, dim3 grid, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc,
-                        const CUtensorMap& md, const TcStepArgs& st, cudaStream_t s) {
+cudaError_t launch_tile(bool overlap, int bn, dim3 grid, const CUtensorMap& ma, const CUtensorMap& mb,
+                        const CUtensorMap& mc, const CUtensorMap& md, const TcStepArgs& st, cudaStream_t s) {
   // (NUTS: the active flags decide before the kernel waits for the launch
   // before it, so there it is an ordinary launch)
   auto go = [&](StepKernel k, size_t smem) {
-    if (!st.active) return launch_dependent(k, grid, dim3(kThreads), smem, s, ma, mb, mc, md, st);
+    if (!st.active) return launch_dependent(overlap, k, grid, dim3(kThreads), smem, s, ma, mb, mc, md, st);
     k<<<grid, kThreads, smem, s>>>(ma, mb, mc, md, st);
     return cudaGetLastError();
   };
@@ -1485,8 +1485,8 @@ cudaError_t launch_logreg_gemm_transition(const StepArgs& a, LogregGemm& g, cuda
     {
       const int zt = static_cast<int>(mt) * g.nrt;      // Z tiles, one persistent CTA per SM
       const cudaError_t e =
-          launch_dependent(k_lr_z_persist, dim3(static_cast<unsigned>(std::min(zt, g.sms))), dim3(kThreads), kZpSmem,
-                           s, g.mThi[in], g.mTlo[in], g.mXhi, g.mXlo, z, static_cast<int>(mt), zt);
+          launch_dependent(a.overlap != 0, k_lr_z_persist, dim3(static_cast<unsigned>(std::min(zt, g.sms))),
+                           dim3(kThreads), kZpSmem, s, g.mThi[in], g.mTlo[in], g.mXhi, g.mXlo, z, static_cast<int>(mt), zt);
       if (e != cudaSuccess) return e;
     }
     {
@@ -1494,7 +1494,8 @@ cudaError_t launch_logreg_gemm_transition(const StepArgs& a, LogregGemm& g, cuda
       // leapfrog update (k_lr_gemm_update)
       st.kc_split = kc_split;
       st.part = g.part;
-      cudaError_t e = launch_tile<kEpiStore>(g.bng, dim3(mt, g.ndt, S), g.mRhi, g.mRlo, g.mXThi, g.mXTlo, st, s);
+      cudaError_t e = launch_tile<kEpiStore>(a.overlap != 0, g.bng, dim3(mt, g.ndt, S), g.mRhi, g.mRlo, g.mXThi,
+                                             g.mXTlo, st, s);
       if (e != cudaSuccess) return e;
       LrSumArgs u{a.C, a.D, g.ld, S, g.nrt, g.ntot, g.part, g.xhi[in], g.xlo[in],
                   g.xhi[out], g.xlo[out], g.p, g.gL, g.lp_part, a.da};
@@ -1502,7 +1503,8 @@ cudaError_t launch_logreg_gemm_transition(const StepArgs& a, LogregGemm& g, cuda
       if (last) {
         k_lr_gemm_update<<<nb, 32 * kWarpsPerBlock, 0, s>>>(u);
       } else {
-        e = launch_dependent(k_lr_gemm_update_middle, dim3(static_cast<unsigned>((n4 + 255) / 256)), dim3(256), 0, s, u);
+        e = launch_dependent(a.overlap != 0, k_lr_gemm_update_middle, dim3(static_cast<unsigned>((n4 + 255) / 256)),
+                             dim3(256), 0, s, u);
         if (e != cudaSuccess) return e;
       }
       count_launch();
@@ -1553,7 +1555,8 @@ cudaError_t launch_logreg_gemm_products(LogregGemm& g, int C, int D, const DASta
   st.active = active;
   k_gauss_tc_step<kEpiLrResid, 64, 2><<<dim3(mt, g.nrt), kThreads, Tile<64, 2>::kSmem, s>>>(
       g.mThi[0], g.mTlo[0], g.mXhi, g.mXlo, z);
-  const cudaError_t e = launch_tile<kEpiStore>(g.bng, dim3(mt, g.ndt, S), g.mRhi, g.mRlo, g.mXThi, g.mXTlo, st, s);
+  const cudaError_t e =
+      launch_tile<kEpiStore>(false, g.bng, dim3(mt, g.ndt, S), g.mRhi, g.mRlo, g.mXThi, g.mXTlo, st, s);
   count_launch(2);
   *splits = S;
   return e != cudaSuccess ? e : cudaGetLastError();

@@ -64,12 +64,12 @@ cudaError_t launch_vjp(const hmc_target& t, int64_t C, const float* x, const flo
 cudaError_t launch_scale_rows(int64_t C, int D, const float* w, const float* g, float* dx, cudaStream_t s);
 
 // Launch `kernel` so that its prologue may overlap the end of the launch before
-// it on the stream (programmatic dependent launch).  The kernel waits
-// (ptx::grid_dependency_wait) before it touches what earlier launches wrote or
-// still read.
+// it on the stream (programmatic dependent launch; overlap: whether it may).  The
+// kernel waits (ptx::grid_dependency_wait) before it touches what earlier launches
+// wrote or still read.
 template <typename... P, typename... A>
-inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                    A&&... args) {
+inline cudaError_t launch_dependent(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                    cudaStream_t s, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -79,7 +79,7 @@ inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block,
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = overlap ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
@@ -136,6 +136,7 @@ struct StepArgs {
   const float* betas;     // replica exchange: row r targets p^betas[r % K]; null = 1
   int K;                  // replicas per chain (1: no tempering)
   int proposal;           // hmc_proposal_kind
+  int overlap;            // logistic regression's products: programmatic dependent launches
   int merged;             // general path: the elementwise steps between two gradients in one launch
   WelfordOut w;           // the pair kernel updates these at kept transitions (streaming)
 };

@@ -759,7 +759,9 @@ cudaError_t launch_logreg_tc_transition(const StepArgs& a, LogregTc& tc, int* er
   // Programmatic dependent launches: a gradient's prologue (barriers, tensor
   // memory, the first data tiles) runs during the update before it, the
   // update's launch during the gradient's end (per gradient, 152 chains x 2719 rows x
-  // 115: 21.1 -> 19.5 us; 2048 x 20000 x 128: 128.1 -> 127.2 us)
+  // 115: 21.1 -> 19.5 us; 2048 x 20000 x 128: 128.1 -> 127.2 us).  Not in graphs that are
+  // launched once: their edges cost the host 2 us a launch (a server at 400 requests/s,
+  // bound by its admission threads: 26.8 -> 22.0 million gradients/s)
   cudaLaunchAttribute attr[2], uattr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
@@ -768,14 +770,14 @@ cudaError_t launch_logreg_tc_transition(const StepArgs& a, LogregTc& tc, int* er
   attr[1].id = uattr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = uattr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = a.overlap ? 2 : 1;
   const int64_t n4 = static_cast<int64_t>(a.C) * (tc.ld / 4);
   cudaLaunchConfig_t ucfg = {};
   ucfg.gridDim = dim3(static_cast<unsigned>((n4 + 127) / 128));
   ucfg.blockDim = dim3(128);
   ucfg.stream = s;
   ucfg.attrs = uattr;
-  ucfg.numAttrs = 1;
+  ucfg.numAttrs = a.overlap ? 1 : 0;
   for (int l = 1; l <= a.L; ++l) {
     g.need_lp = l == a.L;
     if (timer) timer->begin(s);

@@ -108,6 +108,7 @@ def _load():
                                            ctypes.POINTER(ctypes.c_uint64)],
         "hmc_target_vjp": [ctypes.POINTER(hmc_target), ctypes.c_int64, P, P, P, P, ctypes.c_uint64,
                            P],
+        "hmc_graphs_run_once": [P, ctypes.c_int32],
         "hmc_target_vjp_from_grad": [ctypes.c_int64, ctypes.c_int32, P, P, P, P],
         "hmc_target_log_prob_and_grad_noalloc": [ctypes.POINTER(hmc_target), ctypes.c_int64, P, P,
                                                  P, P],
@@ -282,6 +283,10 @@ def hmc_sample_chain_host(ctx, x_inout, num_burnin, num_results, samples_out=Non
     _check(lib.hmc_sample_chain_host(ctx, _ptr(x_inout), int(num_burnin), int(num_results),
                                      _ptr(samples_out), _ptr(trace_step_size),
                                      _ptr(trace_accept)), ctx)
+
+
+def hmc_graphs_run_once(ctx, once=True):
+    _check(lib.hmc_graphs_run_once(ctx, int(once)), ctx)
 
 
 def hmc_read_adaptation(ctx):

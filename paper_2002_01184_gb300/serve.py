@@ -120,6 +120,7 @@ class Server:
         stream = self.streams[job._slot]
         with torch.cuda.device(self.device), torch.cuda.stream(stream):
             job._sampler = Sampler(p, stream=stream, use_graph=True)
+            hmc.hmc_graphs_run_once(job._sampler.ctx)
             x = torch.empty((p.num_chains, p.dim), dtype=torch.float32, device="cuda")
             x.copy_(torch.from_numpy(p.x0).pin_memory(), non_blocking=True)
             job._x = x
