@@ -412,16 +412,20 @@ __global__ void k_lr_begin(LrStepArgs b) {
   if (lane == 0) b.h0[c] = -a.lp[c] + 0.5f * kin;
 }
 
-// v = sum over s < n of src[s * stride], in order, 16 loads in flight
+// v = sum over s < n of src[s * stride], in order, FLY loads in flight.  FLY = 16, but 4
+// where there are no more ranges: the registers of 16 leave fewer warps on an SM,
+// which many chains of a short data pass wait for (40000 chains, 100 rows x 8, a
+// trajectory of one step: 100 us a transition with 4, 139 with 16).
+template <int FLY>
 __device__ __forceinline__ void sum_ranges(const float4* src, int64_t stride, int n, float (&g)[4]) {
   g[0] = g[1] = g[2] = g[3] = 0.f;
-  for (int s0 = 0; s0 < n; s0 += 16) {
-    float4 v[16];
+  for (int s0 = 0; s0 < n; s0 += FLY) {
+    float4 v[FLY];
 #pragma unroll
-    for (int k = 0; k < 16; ++k)
+    for (int k = 0; k < FLY; ++k)
       if (s0 + k < n) v[k] = src[(s0 + k) * stride];
 #pragma unroll
-    for (int k = 0; k < 16; ++k)
+    for (int k = 0; k < FLY; ++k)
       if (s0 + k < n) {
         g[0] += v[k].x; g[1] += v[k].y; g[2] += v[k].z; g[3] += v[k].w;
       }
@@ -434,6 +438,7 @@ __device__ __forceinline__ void sum_ranges(const float4* src, int64_t stride, in
 // of ld = D rounded up to 4), in small blocks over all SMs.  (A warp per chain
 // with four loads in flight took 8.6 us of a gradient's 126 at 2048 chains, half
 // of the 28 at 152.)
+template <int FLY>
 __global__ void __launch_bounds__(128) k_lr_update_middle(LrStepArgs b) {
   ptx::grid_dependency_wait();
   ptx::grid_dependents_launch();
@@ -445,7 +450,7 @@ __global__ void __launch_bounds__(128) k_lr_update_middle(LrStepArgs b) {
   const float4 h = reinterpret_cast<const float4*>(b.thi)[e], l = reinterpret_cast<const float4*>(b.tlo)[e];
   const float4 pv = reinterpret_cast<const float4*>(b.p)[e];
   float g[4];
-  sum_ranges(reinterpret_cast<const float4*>(b.Gpart) + e, n4, b.nsplit, g);
+  sum_ranges<FLY>(reinterpret_cast<const float4*>(b.Gpart) + e, n4, b.nsplit, g);
   const float th[4] = {h.x + l.x, h.y + l.y, h.z + l.z, h.w + l.w};
   const float pin[4] = {pv.x, pv.y, pv.z, pv.w};
   float pout[4], hi[4], lo[4];
@@ -462,6 +467,7 @@ __global__ void __launch_bounds__(128) k_lr_update_middle(LrStepArgs b) {
 
 // The last step: gradient, log p and the final half kick.  One warp per
 // chain, four dims per lane.
+template <int FLY>
 __global__ void k_lr_update(LrStepArgs b) {
   const StepArgs& a = b.s;
   const int c = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
@@ -477,7 +483,7 @@ __global__ void k_lr_update(LrStepArgs b) {
     const float4 h = reinterpret_cast<const float4*>(b.thi)[e], l = reinterpret_cast<const float4*>(b.tlo)[e];
     const float4 pv = reinterpret_cast<const float4*>(b.p)[e];
     float g[4];
-    sum_ranges(reinterpret_cast<const float4*>(b.Gpart) + e, split4, b.nsplit, g);
+    sum_ranges<FLY>(reinterpret_cast<const float4*>(b.Gpart) + e, split4, b.nsplit, g);
     const float th[4] = {h.x + l.x, h.y + l.y, h.z + l.z, h.w + l.w};
     const float pin[4] = {pv.x, pv.y, pv.z, pv.w};
     float pout[4];
@@ -778,6 +784,7 @@ cudaError_t launch_logreg_tc_transition(const StepArgs& a, LogregTc& tc, int* er
   ucfg.stream = s;
   ucfg.attrs = uattr;
   ucfg.numAttrs = a.overlap ? 1 : 0;
+  const bool few = b.nsplit <= 4;
   for (int l = 1; l <= a.L; ++l) {
     g.need_lp = l == a.L;
     if (timer) timer->begin(s);
@@ -786,9 +793,9 @@ cudaError_t launch_logreg_tc_transition(const StepArgs& a, LogregTc& tc, int* er
     if (timer) timer->end(s);
     if (e != cudaSuccess) return e;
     if (l == a.L) {
-      k_lr_update<<<nb, 32 * kWarpsPerBlock, 0, s>>>(b);
+      (few ? k_lr_update<4> : k_lr_update<16>)<<<nb, 32 * kWarpsPerBlock, 0, s>>>(b);
     } else {
-      e = cudaLaunchKernelEx(&ucfg, k_lr_update_middle, b);
+      e = cudaLaunchKernelEx(&ucfg, few ? k_lr_update_middle<4> : k_lr_update_middle<16>, b);
       if (e != cudaSuccess) return e;
     }
     count_launch(2);
