@@ -68,7 +68,9 @@ size_t span_smem_bytes(int Dp, int max_depth) {
 // instructions count and not a leaf's latency.  20 transitions of the funnel in one
 // launch, kPlain / kLean: 2000 x 400 1.31, 4096 x 300 1.19, 3000 x 400 0.98; of the standard
 // normal, 4096 x 260 1.11.  A launch of one transition, which ends with its deepest
-// trees, is the shorter in kPlain for the funnel (1300 x 300 0.90).
+// trees, is the shorter in kPlain for the funnel (1300 x 300 0.90), unless these are
+// shallow and its three blocks do not hold all chains (2000 x 300, depth 3: 1.4; 4096 x
+// 400, depth 3: 1.2; 2400 x 400 as depth 5 1.4, 10 1.0).
 constexpr int kPlain = 0, kWide = 1, kLean = 2;
 constexpr int nuts_blocks(int target, int nb, int form) {
   return form == kWide ? (nb == 1 ? 4 : 2)
@@ -495,7 +497,10 @@ cudaError_t launch_nb(const NutsArgs& na, cudaStream_t s) {
   if (all_resident(na, shared, sms)) return launch_v<TARGET, NB, true, kWide>(na, smem, s);
   const bool wide = all_resident(na, glob, sms);
   if constexpr (NB == 4) {
-    if (TARGET == HMC_T_STD_NORMAL || na.T > 1) return launch_many<TARGET, NB, kLean>(na, smem, wide, sms, s);
+    // (shallow trees end together: a second round of blocks is what counts there)
+    const bool shallow = na.max_depth <= (all_resident(na, nuts_blocks(TARGET, NB, kLean), sms) ? 7 : 6) &&
+                         !all_resident(na, nuts_blocks(TARGET, NB, kPlain), sms);
+    if (TARGET == HMC_T_STD_NORMAL || na.T > 1 || shallow) return launch_many<TARGET, NB, kLean>(na, smem, wide, sms, s);
   }
   if constexpr (NB < 4 || TARGET == HMC_T_FUNNEL) return launch_many<TARGET, NB, kPlain>(na, smem, wide, sms, s);
   return cudaErrorInvalidValue;      // (not reached)
