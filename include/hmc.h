@@ -88,8 +88,9 @@ typedef enum {
                                      always takes the shared-memory SIMT
                                      transition (dim <= 512; the whole chain
                                      in one or two launches where the data
-                                     fits shared memory, else 8 chains per
-                                     CTA tile, a launch per transition) */
+                                     fits shared memory and that is the
+                                     shorter form, else 8 chains per CTA
+                                     tile, a launch per transition) */
 } hmc_impl;
 
 /* Inner (uncalibrated) kernel of the Metropolis-Hastings composition,

@@ -21,7 +21,9 @@
 // launch, the state's round trip and a last block that finished the step-size
 // update alone.  Measured, per transition: funnel, 100 dims, 10 steps, 4096
 // chains 14.0 us -> 5.1 us (7.5 us while adapting), 100 chains 2.4 us (4.8);
-// the 100 x 1 standard normal of 3 steps 6.0 us -> 0.33 us.
+// the 100 x 1 standard normal of 3 steps 6.0 us -> 0.33 us.  A launch of a single
+// transition has nothing to carry: many chains of a whole warp take the tile
+// kernel then (tiles_pay).
 //
 // Lanes: a chain takes G = 1..32 lanes (four dims each, NB blocks of 128 dims
 // above 128); the butterfly over G lanes is the 32-lane one without its steps

@@ -1,6 +1,7 @@
 // One launch per HMC transition for Bayesian logistic regression: the tile
 // function in logreg_tile.cuh, one CTA per tile of chains.  Taken where the data
-// does not fit shared memory beside a chain (logreg_chain.cu).
+// does not fit shared memory beside a chain, and for many chains of few rows
+// (logreg_chain.cu).
 #include "logreg_tile.cuh"
 
 namespace hmc {

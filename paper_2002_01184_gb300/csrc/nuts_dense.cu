@@ -21,12 +21,14 @@
 // For the logistic regression the iterations are the body of a CUDA-graph
 // conditional WHILE node: the leaf kernel's last block clears the condition
 // when no chain is left.  For the Gaussian the whole loop is one launch: up to
-// 256 dims a cluster of CTAs per chain block, which stops when its own chains
-// are done (k_nuts_gauss_cluster, below), beyond that a persistent cooperative
-// launch of all SMs, products and leaves separated by bounded grid barriers
+// 256 dims, where it is the shorter form (cluster_pays), a cluster of CTAs per
+// chain block, which stops when its own chains are done
+// (k_nuts_gauss_cluster, below), else a persistent cooperative launch of all
+// SMs, products and leaves separated by bounded grid barriers
 // (k_nuts_gauss_loop).  Either way a transition costs as many iterations as
-// its deepest tree and the host never waits on the device in between.  A chain's result depends only on its own row of every product,
-// so it is the same in any batch.
+// its deepest tree and the host never waits on the device in between.  A
+// chain's result depends only on its own row of every product, so it is the
+// same in any batch.
 //
 // Per chain, the tree's scalars (NdChain) and a scratch of kNutsSlots rows of
 // the padded row length (the two trajectory ends, the candidates, the span
@@ -472,8 +474,8 @@ __global__ void __launch_bounds__(32 * kNdWarps) k_nuts_dense_finish(NdArgs na) 
 //
 // The graph loop above pays two kernel launches, the products' set-up
 // (barriers, tensor memory) and the WHILE node's relaunch every leaf: about
-// 15 us whatever the size.  For a Gaussian of more than 256 dims (below that the
-// loop per chain block, further down) the whole loop runs instead in one
+// 15 us whatever the size.  For the Gaussian (where the loop per chain block,
+// further down, does not take its place) the whole loop runs instead in one
 // cooperative launch of one CTA per SM: each iteration is the tile
 // products X P of the 128-chain tiles still building (3xTF32 tcgen05, 64
 // output dims per tile, tiles dealt round-robin to the CTAs; the pipeline's

@@ -21,8 +21,8 @@ namespace hmc {
 std::atomic<uint64_t> g_launches{0};
 
 // SM count of the current device (the logistic regression's split-K and
-// path decisions), asked of the driver once per device; 152, a GB300's count,
-// when no device can be queried.
+// path decisions), queried once per device; 152, a GB300's count, when no
+// device can be queried.
 int current_sm_count() {
   static std::atomic<int> known[64];
   int dev = 0, sms = 0;
